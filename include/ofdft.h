@@ -156,7 +156,9 @@ void ofdft_default_params(ofdft_params* p);
  * cooperative launch per eight iterations where the grid's blocks fit on the
  * device at once), OFDFT_CG_FOLD_BYTES (bytes of the five CG vectors above which
  * a CG folds its iterate update into the next stencil pass; default 96 MiB),
- * multigrid variants (each gives the same preconditioner up to rounding):
+ * OFDFT_FD=0 (multigrid V-cycles where the preconditioner would be the fast
+ * diagonalisation; any OFDFT_MG_* variable below asks for them too, unless
+ * OFDFT_FD=1), multigrid variants (each gives the same preconditioner up to rounding):
  * OFDFT_MG_ZSTREAM=1 (level smoothing passes as radius-1 z-streaming stencils
  * instead of row-per-warp kernels), OFDFT_MG_FUSE_NODES / OFDFT_MG_FUSE_BELOW
  * (levels of at least / coarser levels of at most this many nodes run smoothing,
@@ -185,8 +187,11 @@ int ofdft_destroy(ofdft_ctx* ctx);
  * same relative residual).
  *   OFDFT_PRECOND_NONE: plain CG (the oracle's iteration, iteration for
  *     iteration up to rounding).
- *   OFDFT_PRECOND_MG (default): z = M r with M one symmetric V(1,1)-cycle of the
- *     second-order 7-point Laplacian (damped Jacobi, full weighting, trilinear
+ *   OFDFT_PRECOND_MG (default): z = M r.  On grids whose axes all have 32 to 512
+ *     nodes M inverts -L_h itself, up to rounding, by diagonalising the three
+ *     axes' matrices (one CG step in FP64, one per residual correction in MIXED);
+ *     on the others M is one symmetric V(1,1)-cycle of the second-order 7-point
+ *     Laplacian (damped Jacobi, full weighting, trilinear
  *     prolongation, coarse node I on fine node 2I+1, zero Dirichlet values);
  *     grids whose coarsest level would keep more than 4096 nodes (an extent
  *     below 4 with the others large) fall back to plain CG.

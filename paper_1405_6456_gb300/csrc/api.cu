@@ -90,12 +90,19 @@ int cg_flush(ofdft_ctx* c, const GridDev& g, T* x, const T* pv, CgScalars* sc) {
 
 // Whether the CG on this grid runs preconditioned; allocates what the cycle needs.
 template <typename T>
-int mg_prepare(ofdft_ctx* c, const GridDev& g, double h, MgPlan* P) {
+int mg_prepare(ofdft_ctx* c, const GridDev& g, int R, double h, MgPlan* P) {
   *P = MgPlan{};
   if (c->precond != OFDFT_PRECOND_MG) return OFDFT_OK;
   *P = mg_plan(g, h, sizeof(T), c->mg_omega);
   if (!P->ok) return OFDFT_OK;
   TRY(ensure(c, c->v[V_Z], g.G * sizeof(T)));
+  if (fd_usable(c, g)) {
+    TRY(fd_plan(c, g, R, h, &P->fd));
+    if (P->fd.on) {
+      TRY(ensure(c, c->v[V_T], fd_scratch(g) * sizeof(T)));
+      return ensure_partials(c, (long long)P->fd.pitch * g.n2 / 32 + 1, 1);
+    }
+  }
   TRY(ensure(c, c->v[V_T], g.G * sizeof(T)));
   TRY(ensure(c, c->mgbuf, std::max<long long>(P->elems, 1) * sizeof(T)));
   TRY(ensure_partials(c, pointwise_blocks(c, g.G), 1));
@@ -151,6 +158,7 @@ inline bool mg_level_fused(const ofdft_ctx* c, const MgPlan& P, int l) {
 // PCG scalars (beta, rz).  Every kernel returns at once when the solve is done.
 template <typename T>
 int mg_vcycle(ofdft_ctx* c, const MgPlan& P, const T* r, T* z, CgScalars* sc) {
+  if (P.fd.on) return fd_apply<T>(c, mg_gdev(P.d[0]), P.fd, r, z, c->v[V_T].p, sc);
   T* cb = static_cast<T*>(c->mgbuf.p);
   T* t0 = vec<T>(c, V_T);
   auto rl = [&](int l) -> T* { return l == 0 ? const_cast<T*>(r) : cb + P.off[l]; };
@@ -290,6 +298,7 @@ int mg_vcycle(ofdft_ctx* c, const MgPlan& P, const T* r, T* z, CgScalars* sc) {
 // V-cycle launches per CG iteration.
 inline int mg_launches(const ofdft_ctx* c, const MgPlan& P) {
   if (!P.ok) return 0;
+  if (P.fd.on) return 5;
   int n = 1;
   const int ltop = (c->mg_cluster && P.lq > 0) ? P.lq : P.lc;
   for (int l = 0; l < ltop; ++l) n += (l == 0 && !c->mg_finest_smooth) ? 2 : mg_level_fused(c, P, l) ? 2 : 4;
@@ -404,7 +413,7 @@ int cg_graph(ofdft_ctx* c, int R, const GridDev& g, double h, const Weights<doub
   const std::vector<long long> key = {(long long)sizeof(T), (long long)sizeof(X), R, g.n1, g.n2, g.n3, (long long)x,
                                       (long long)r,
                                       (long long)pv, (long long)qv, (long long)sc, pb,
-                                      (long long)c->partials.p, (long long)(h * 1e12), sample_set, pcg ? 1 : 0,
+                                      (long long)c->partials.p, (long long)(h * 1e12), sample_set, pcg ? (mg->fd.on ? 2 : 1) : 0,
                                       pcg ? (long long)c->mgbuf.p : 0, pcg ? (long long)c->v[V_Z].p : 0,
                                       pcg ? (long long)c->v[V_T].p : 0};
   if (sample_set >= 0 && !c->gev[sample_set][0]) {
@@ -475,7 +484,7 @@ int cg_while_graph(ofdft_ctx* c, int R, const GridDev& g, double h, const Weight
   const bool pcg = mg && mg->ok;
   const std::vector<long long> key = {-1, (long long)sizeof(T), (long long)sizeof(X), R, g.n1, g.n2, g.n3,
                                       (long long)x, (long long)r, (long long)pv, (long long)qv, (long long)sc, pb,
-                                      (long long)c->partials.p, (long long)(h * 1e12), pcg ? 1 : 0,
+                                      (long long)c->partials.p, (long long)(h * 1e12), pcg ? (mg->fd.on ? 2 : 1) : 0,
                                       pcg ? (long long)c->mgbuf.p : 0, pcg ? (long long)c->v[V_Z].p : 0,
                                       pcg ? (long long)c->v[V_T].p : 0};
   for (auto& e : c->graphs)
@@ -652,7 +661,7 @@ int cg_iterate(ofdft_ctx* c, int R, const GridDev& g, double h, const Weights<do
   T* qv = vec<T>(c, V_AP);
   const bool per_launch = (c->prof & (1 << OFDFT_K_CG_UPDATE)) != 0;  // per-kernel timing asked for
   MgPlan mg;
-  TRY(mg_prepare<T>(c, g, h, &mg));
+  TRY(mg_prepare<T>(c, g, R, h, &mg));
   if (c->coop && !per_launch && !mg.ok) {
     bool used = false;
     TRY(cg_coop<T>(c, R, g, Wneg, reinterpret_cast<T*>(x), r, pv, qv, sc, max_it, host_sc, &used));
@@ -670,6 +679,17 @@ int cg_iterate(ofdft_ctx* c, int R, const GridDev& g, double h, const Weights<do
     // attribute outside the capture), then the WHILE graph for the rest
     const int it0 = host_sc->iters;
     TRY((cg_step<T, X>(c, R, g, Wneg, x, r, pv, qv, sc, pb, &mg)));
+    if (mg.fd.on) {
+      // one step of the directly inverted operator mostly ends the solve
+      CgScalars first;
+      TRY(sync_scalars(c, sc, sizeof(CgScalars), &first));
+      if (first.done) {
+        if (first.xdefer) TRY(cg_flush<T>(c, g, reinterpret_cast<T*>(x), pv, sc));
+        *host_sc = first;
+        host_sc->xdefer = 0;
+        return OFDFT_OK;
+      }
+    }
     cudaGraphExec_t wexec = nullptr;
     TRY((cg_while_graph<T, X>(c, R, g, h, Wneg, x, r, pv, qv, sc, pb, &wexec, &mg)));
     CU(cudaGraphLaunch(wexec, c->stream));
@@ -750,7 +770,7 @@ int poisson_fp64(ofdft_ctx* c, int R, const GridDev& g, double h, const double* 
   const Weights<double> W = lap_weights(R, h, 1.0), Wneg = lap_weights(R, h, -1.0);
   double* r = vec<double>(c, V_R);
   MgPlan mg;
-  TRY(mg_prepare<double>(c, g, h, &mg));
+  TRY(mg_prepare<double>(c, g, R, h, &mg));
   TRY(launch_z_r<double>(c, R, g, W, LoadPlain<double>{phi},
                          EpiResidual<double>{rho, u, b, r, c->sc, tol, max_it, 1, mg.ok ? 1 : 0}, OFDFT_K_RESIDUAL));
   CgScalars hs;
@@ -789,7 +809,7 @@ int poisson_mixed(ofdft_ctx* c, int R, const GridDev& g, double h, const float* 
   float* e32 = vec<float>(c, V_E32);
   const int pb = pointwise_blocks(c, g.G);
   MgPlan mg;
-  TRY(mg_prepare<float>(c, g, h, &mg));
+  TRY(mg_prepare<float>(c, g, R, h, &mg));
   int total = 0, rc = OFDFT_OK;
   CgScalars hs, hs32;
   const int max_rounds = 60;
@@ -1958,6 +1978,12 @@ int ofdft_create(ofdft_ctx** out, int device, void* stream) {
   c->cond_graphs = !(cgr && cgr[0] == '0');
   const char* ffr = getenv("OFDFT_FF_RESIDUAL");  // 0: FP64 stencil in the mixed residual pass
   c->ff_residual = !(ffr && ffr[0] == '0');
+  // any multigrid variant asked for by name runs the V-cycle
+  for (const char* v : {"OFDFT_MG_OMEGA", "OFDFT_MG_SWEEPS", "OFDFT_MG_ZSTREAM", "OFDFT_MG_ZSTREAM_NODES",
+                        "OFDFT_MG_CLUSTER", "OFDFT_MG_FUSE_BELOW", "OFDFT_MG_FUSE_NODES", "OFDFT_MG_FINEST_SMOOTH"})
+    if (getenv(v)) c->fd = 0;
+  const char* fde = getenv("OFDFT_FD");  // 0: V-cycles on every grid, 1: whatever else is set
+  if (fde) c->fd = atoi(fde) != 0;
   const char* mf = getenv("OFDFT_MG_FUSE_NODES");  // levels of at least this many nodes take the fused passes
   if (mf) c->mg_fuse_nodes = atoll(mf);          // (-1: none)
   const char* fb = getenv("OFDFT_CG_FOLD_BYTES");  // CG working set above which the iterate update is folded
@@ -1987,6 +2013,7 @@ int ofdft_destroy(ofdft_ctx* c) {
   cudaFree(c->partials.p);
   for (auto& b : c->v) cudaFree(b.p);
   cudaFree(c->mgbuf.p);
+  for (auto& t : c->fdtab) cudaFree(t.dev);
   cudaFree(c->counter);
   cudaFree(c->sc);
   cudaFree(c->scal);

@@ -16,6 +16,7 @@
 #include <vector>
 
 #include "../../include/ofdft.h"
+#include "fastdiag.cuh"
 #include "kernels.cuh"
 
 
@@ -26,6 +27,16 @@ struct DevBuf {
 };
 
 using ofd::CgScalars;
+
+// Eigenvectors and eigenvalues of one axis of the fast diagonalisation (node
+// count n, stencil radius R, spacing 1), kept for the context's lifetime.
+struct FdTable {
+  int n = 0, R = 0;
+  void* dev = nullptr;
+  ofd::FdAxis ax;
+  const float *mu = nullptr, *mul = nullptr;  // eigenvalues, even modes first
+  const float *mx = nullptr, *mxl = nullptr;  // ... in the order of a scratch row
+};
 
 struct ofdft_ctx {
   int device = 0;
@@ -96,6 +107,8 @@ struct ofdft_ctx {
   int func_split_dots = 0;                     // G.d and G.s_old by a pass after the functional
   int mg_zstream = 0;                          // level smoothing passes as z-streaming radius-1 stencils
   long long mg_zstream_nodes = -1;             // ... on the levels of at least this many nodes (-1: none)
+  int fd = 1;                                  // fast diagonalisation on the grids it covers (else V-cycles)
+  std::vector<FdTable> fdtab;                  // its axis tables
   // the b_J tables in V_BTAB belong to this geometry (atoms, charges, grid,
   // sigma, r_c, stencil radius); empty: none kept
   std::vector<double> btab_key;
@@ -387,6 +400,15 @@ bool zvec_ok(const GridDev& g, const L& ld, const E& ep) {
   return true;
 }
 
+// Fast diagonalisation of one grid (kernels and the method: fastdiag.cuh).
+struct FdPlan {
+  bool on = false;
+  FdAxis ax[3];                       // x, y, z
+  const float *mu[3], *mul[3];        // eigenvalues of h^2 T, high and low parts
+  int pitch = 0;                      // floats of a scratch row
+  double ih2 = 0.0;
+};
+
 // Multigrid preconditioner of the Poisson CG (S3): the levels of a grid (kernels
 // and the cycle's steps: mg_* in kernels.cuh).
 constexpr int kMgCoarseNodes = 4096;  // levels from this size down run in one block
@@ -408,6 +430,7 @@ struct MgPlan {
   MgSlab slab[kMgMaxLevels];
   size_t csmem = 0;       // dynamic shared memory per block of the cluster kernel
   unsigned tail_off = 0;  // byte offset of block 0's coarse-end arrays
+  FdPlan fd;              // fd.on: z = M r by fast diagonalisation instead of the cycle
 };
 constexpr size_t kMgClusterSmem = 220 * 1024;  // dynamic shared memory per cluster block (of 227 KB)
 
@@ -484,6 +507,294 @@ cudaError_t launch_k(ofdft_ctx* c, void (*kern)(KArgs...), dim3 grid, dim3 block
   }
   kern<<<grid, block, smem, c->stream>>>(args...);
   return cudaGetLastError();
+}
+
+// ------------------------------------------------------ fast diagonalisation --
+// Eigenpairs of a symmetric m x m matrix a (row-major, destroyed): Householder
+// tridiagonalisation and the implicit symmetric QR iteration with Wilkinson's
+// shift (Golub and Van Loan, Matrix Computations, sec. 8.3).  On return d holds
+// the eigenvalues and row k of v the eigenvector of d[k].  Returns false when an
+// eigenvalue does not settle.
+inline bool sym_eigen(int m, std::vector<double>& a, std::vector<double>& d, std::vector<double>& v) {
+  d.assign(m, 0.0);
+  v.assign((size_t)m * m, 0.0);
+  for (int i = 0; i < m; ++i) v[(size_t)i * m + i] = 1.0;
+  std::vector<double> e(m, 0.0), h(m), p(m);
+  for (int k = 0; k + 2 < m; ++k) {  // reflect column k below the subdiagonal away
+    double nrm = 0.0;
+    for (int i = k + 1; i < m; ++i) nrm += a[(size_t)i * m + k] * a[(size_t)i * m + k];
+    nrm = sqrt(nrm);
+    if (nrm == 0.0) continue;
+    const double x0 = a[(size_t)(k + 1) * m + k], al = x0 > 0.0 ? -nrm : nrm;
+    for (int i = k + 1; i < m; ++i) h[i] = a[(size_t)i * m + k];
+    h[k + 1] -= al;
+    double hh = 0.0;
+    for (int i = k + 1; i < m; ++i) hh += h[i] * h[i];
+    const double be = 2.0 / hh;
+    double hp = 0.0;
+    for (int i = k + 1; i < m; ++i) {
+      double t = 0.0;
+      for (int j = k + 1; j < m; ++j) t += a[(size_t)i * m + j] * h[j];
+      p[i] = be * t;
+      hp += h[i] * p[i];
+    }
+    for (int i = k + 1; i < m; ++i) p[i] -= 0.5 * be * hp * h[i];
+    for (int i = k + 1; i < m; ++i)
+      for (int j = k + 1; j < m; ++j) a[(size_t)i * m + j] -= h[i] * p[j] + p[i] * h[j];
+    a[(size_t)(k + 1) * m + k] = a[(size_t)k * m + k + 1] = al;
+    std::fill(p.begin(), p.end(), 0.0);  // v = (I - be h h^T) v
+    for (int i = k + 1; i < m; ++i)
+      for (int j = 0; j < m; ++j) p[j] += h[i] * v[(size_t)i * m + j];
+    for (int i = k + 1; i < m; ++i)
+      for (int j = 0; j < m; ++j) v[(size_t)i * m + j] -= be * h[i] * p[j];
+  }
+  for (int i = 0; i < m; ++i) {
+    d[i] = a[(size_t)i * m + i];
+    if (i + 1 < m) e[i] = a[(size_t)(i + 1) * m + i];
+  }
+  int hi = m - 1, its = 0;
+  while (hi > 0) {
+    for (int k = 0; k < hi; ++k)
+      if (fabs(e[k]) <= 1.2e-16 * (fabs(d[k]) + fabs(d[k + 1]))) e[k] = 0.0;
+    if (e[hi - 1] == 0.0) {
+      --hi;
+      its = 0;
+      continue;
+    }
+    if (++its > 80) return false;
+    int lo = hi - 1;
+    while (lo > 0 && e[lo - 1] != 0.0) --lo;
+    const double g = 0.5 * (d[hi - 1] - d[hi]), q = e[hi - 1];
+    const double den = g + (g >= 0.0 ? 1.0 : -1.0) * hypot(g, q);
+    const double mu = d[hi] - q * q / den;
+    double x = d[lo] - mu, z = e[lo];
+    for (int k = lo; k < hi; ++k) {  // chase the bulge with plane rotations
+      const double r = hypot(x, z);
+      const double cs = r > 0.0 ? x / r : 1.0, sn = r > 0.0 ? z / r : 0.0;
+      if (k > lo) e[k - 1] = r;
+      const double dk = d[k], dn = d[k + 1], ek = e[k];
+      d[k] = cs * cs * dk + 2.0 * cs * sn * ek + sn * sn * dn;
+      d[k + 1] = sn * sn * dk - 2.0 * cs * sn * ek + cs * cs * dn;
+      e[k] = (cs * cs - sn * sn) * ek + cs * sn * (dn - dk);
+      if (k + 1 < hi) {
+        x = e[k];
+        z = sn * e[k + 1];
+        e[k + 1] *= cs;
+      }
+      double* v0 = &v[(size_t)k * m];
+      double* v1 = v0 + m;
+      for (int j = 0; j < m; ++j) {
+        const double t = v0[j];
+        v0[j] = cs * t + sn * v1[j];
+        v1[j] = cs * v1[j] - sn * t;
+      }
+    }
+  }
+  return true;
+}
+
+// The axis table of n nodes at stencil radius R, in host memory: `mat` holds
+// forwards high, low, backwards high, low (each the even half's ne x pe and the
+// odd half's no x po elements), `mu` the n eigenvalues at spacing 1 (even modes
+// first).  The half problems: in the basis (delta_i +- delta_{n-1-i}) / sqrt 2
+// (and the middle node of an odd axis) the Toeplitz matrix t(|i - j|) reads
+// t(|i - j|) +- t(n - 1 - i - j).
+inline bool fd_axis_host(int n, int R, FdAxis* ax, std::vector<float>* mat, std::vector<double>* mu) {
+  ax->n = n;
+  ax->ne = (n + 1) / 2;
+  ax->no = n / 2;
+  ax->pe = (ax->ne + kFdTile - 1) / kFdTile * kFdTile;
+  ax->po = (ax->no + kFdTile - 1) / kFdTile * kFdTile;
+  const size_t se = (size_t)ax->ne * ax->pe, so = (size_t)ax->no * ax->po, sz = se + so;
+  mat->assign(4 * sz, 0.0f);
+  mu->assign(n, 0.0);
+  const Weights<double> W = lap_weights(R, 1.0, -1.0);
+  auto t = [&](int q) { return q == 0 ? W.c / 3.0 : q <= R ? W.w[q] : 0.0; };
+  const double r2 = sqrt(0.5);
+  for (int odd = 0; odd < 2; ++odd) {
+    const int m = odd ? ax->no : ax->ne, wp = odd ? ax->po : ax->pe;
+    const bool mid = !odd && (n & 1);
+    std::vector<double> a((size_t)m * m), d, v;
+    for (int i = 0; i < m; ++i)
+      for (int j = 0; j < m; ++j) {
+        double x = t(abs(i - j));
+        const double y = t(n - 1 - i - j);
+        const int mids = (mid && i == m - 1) + (mid && j == m - 1);
+        if (mids == 0)
+          x += odd ? -y : y;
+        else if (mids == 1)
+          x = 2.0 * r2 * x;  // sqrt 2 t(|i - m|): both mirror images couple to the middle
+        a[(size_t)i * m + j] = x;
+      }
+    if (!sym_eigen(m, a, d, v)) return false;
+    for (int k = 0; k < m; ++k) (*mu)[(odd ? ax->ne : 0) + k] = d[k];
+    for (int k = 0; k < m; ++k)
+      for (int i = 0; i < m; ++i) {
+        const double x = v[(size_t)k * m + i] * ((mid && i == m - 1) ? 1.0 : r2);
+        const float h = (float)x, l = (float)(x - (double)h);
+        const size_t f = (odd ? se : 0) + (size_t)i * wp + k, b = (odd ? se : 0) + (size_t)k * wp + i;
+        (*mat)[f] = h;
+        (*mat)[sz + f] = l;
+        (*mat)[2 * sz + b] = h;
+        (*mat)[3 * sz + b] = l;
+      }
+  }
+  return true;
+}
+
+// The context's table for (n, R), built and copied to the device on first use.
+inline int fd_table(ofdft_ctx* c, int n, int R, const FdTable** out) {
+  for (const FdTable& t : c->fdtab)
+    if (t.n == n && t.R == R) {
+      *out = &t;
+      return OFDFT_OK;
+    }
+  FdTable t;
+  t.n = n;
+  t.R = R;
+  std::vector<float> mat;
+  std::vector<double> mu;
+  *out = nullptr;
+  if (!fd_axis_host(n, R, &t.ax, &mat, &mu)) return OFDFT_OK;  // not settled: the caller keeps the V-cycle
+  // the eigenvalues twice: in order (as the z axis uses them) and laid out as the
+  // scratch rows are (x), where the padding's ones only ever divide zeros
+  const size_t sz = mat.size() / 4, np = (size_t)n + 16;
+  mat.resize(4 * sz + 4 * np, 1.0f);
+  for (int k = 0; k < n; ++k) {
+    const float h = (float)mu[k], l = (float)(mu[k] - (double)h);
+    const size_t x = k < t.ax.ne ? k : fd_up4(t.ax.ne) + k - t.ax.ne;
+    mat[4 * sz + k] = h;
+    mat[4 * sz + np + k] = l;
+    mat[4 * sz + 2 * np + x] = h;
+    mat[4 * sz + 3 * np + x] = l;
+  }
+  CU(cudaMalloc(&t.dev, mat.size() * sizeof(float)));
+  const cudaError_t e = cudaMemcpyAsync(t.dev, mat.data(), mat.size() * sizeof(float), cudaMemcpyHostToDevice, c->stream);
+  if (e != cudaSuccess || cudaStreamSynchronize(c->stream) != cudaSuccess) {
+    cudaFree(t.dev);
+    return fail(c, OFDFT_ECUDA, "fast diagonalisation: copying an axis table failed");
+  }
+  const float* p = static_cast<const float*>(t.dev);
+  t.ax.fwd = p;
+  t.ax.fwdl = p + sz;
+  t.ax.inv = p + 2 * sz;
+  t.ax.invl = p + 3 * sz;
+  t.mu = p + 4 * sz;
+  t.mul = p + 4 * sz + np;
+  t.mx = p + 4 * sz + 2 * np;
+  t.mxl = p + 4 * sz + 3 * np;
+  c->fdtab.push_back(t);
+  *out = &c->fdtab.back();
+  return OFDFT_OK;
+}
+
+// Whether a grid takes the fast diagonalisation: every axis of kFdMinN to
+// kFdMaxN nodes.  Measured against the V-cycle on whole Poisson solves of a random
+// density, order 12 (us; FP64 to 1e-10, MIXED to 1e-8; V-cycle -> here):
+//   32^3       FP64   2,626 ->    242    MIXED   1,402 ->    398
+//   64^3              4,713 ->    257            2,105 ->    411
+//   512x48^2         12,602 ->    947            4,200 ->    671
+//   160^3            30,551 ->  1,786            7,787 ->  1,949
+//   512^2x64        143,156 -> 10,329           26,231 ->  8,768
+//   400^3           482,773 -> 91,501          103,551 -> 43,391
+// and to 1e-4 (the loosest a solve asks for) 3 to 9 times faster, so nothing
+// inside the limits goes to the V-cycle.  The upper limit is what one block's
+// panel holds; the work grows with n1 + n2 + n3 per node.  Below kFdMinN the
+// V-cycle keeps the iteration counts that callers who cap them see (a cap of a
+// few steps ends a 24^3 solve with OFDFT_ENOTCONV).
+inline bool fd_usable(const ofdft_ctx* c, const GridDev& g, int nmax = kFdMaxN) {
+  const int lo = std::min(g.n1, std::min(g.n2, g.n3)), hi = std::max(g.n1, std::max(g.n2, g.n3));
+  return c->fd && lo >= kFdMinN && hi <= nmax;
+}
+
+// Floats of a scratch row, and elements of the scratch array.
+inline int fd_pitch(int n1) { return fd_up4((n1 + 1) / 2) + fd_up4(n1 / 2); }
+inline long long fd_scratch(const GridDev& g) { return (long long)fd_pitch(g.n1) * g.n2 * g.n3; }
+
+inline int fd_plan(ofdft_ctx* c, const GridDev& g, int R, double h, FdPlan* P) {
+  *P = FdPlan{};
+  const int n[3] = {g.n1, g.n2, g.n3};
+  for (int d = 0; d < 3; ++d) {
+    const FdTable* t = nullptr;
+    TRY(fd_table(c, n[d], R, &t));
+    if (!t) return OFDFT_OK;
+    P->ax[d] = t->ax;
+    P->mu[d] = d == 0 ? t->mx : t->mu;
+    P->mul[d] = d == 0 ? t->mxl : t->mul;
+  }
+  P->pitch = fd_pitch(g.n1);
+  P->ih2 = 1.0 / (h * h);
+  P->on = true;
+  return OFDFT_OK;
+}
+
+// The job of pass p (0 .. 4: x, y, z, y, x) of z = M r.
+template <typename T>
+FdJob fd_job(const GridDev& g, const FdPlan& P, int p, const T* r, T* z, void* scratch, CgScalars* sc) {
+  FdJob J = {};
+  const int d = p == 2 ? 2 : (p == 1 || p == 3) ? 1 : 0;
+  J.ax = P.ax[d];
+  J.in = r;
+  J.out = z;
+  J.s = static_cast<float*>(scratch);
+  J.sl = J.s + fd_scratch(g);
+  J.pitch = P.pitch;
+  J.ncols = d == 0 ? (long long)g.n2 * g.n3 : d == 1 ? (long long)P.pitch * g.n3 : (long long)P.pitch * g.n2;
+  J.cw = d == 1 ? P.pitch : (int)((long long)P.pitch * g.n2);
+  J.is = d == 1 ? P.pitch : P.pitch * g.n2;
+  J.cs = (long long)P.pitch * g.n2;
+  J.mx = P.mu[0], J.my = P.mu[1], J.mz = P.mu[2];
+  J.mxl = P.mul[0], J.myl = P.mul[1], J.mzl = P.mul[2];
+  J.ih2 = P.ih2;
+  J.vec = g.n1 % 8 == 0 && (((uintptr_t)r | (uintptr_t)z) & 15u) == 0;
+  J.sc = sc;
+  return J;
+}
+
+template <typename T, bool XAX, int MODE, int CT, int TPW>
+int fd_launch(ofdft_ctx* c, FdJob J, int warps) {
+  constexpr int TC = 16 * CT;
+  const size_t smem = (size_t)fd_panel_floats(J.ax, XAX, TC) * sizeof(T) + (size_t)warps * fd_ring_floats<sizeof(T) == 8>() * sizeof(float);
+  static bool attr_dev[64] = {false};
+  if (c->device < 0 || c->device >= 64) return fail(c, OFDFT_EINVAL, "device index out of range");
+  if (!attr_dev[c->device]) {
+    CU(cudaFuncSetAttribute(fd_kernel<T, XAX, MODE, CT, TPW>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFdSmem));
+    attr_dev[c->device] = true;
+  }
+  const long long nb = (J.ncols + TC - 1) / TC;
+  if (MODE == FD_SOLVE) {
+    TRY(ensure_partials(c, nb, 1));
+    J.red = red(c);
+    J.nblocks = (int)nb;
+  }
+  ProfScope ps_(c, OFDFT_K_MG);
+  CU(launch_k(c, fd_kernel<T, XAX, MODE, CT, TPW>, dim3((unsigned)nb), dim3(warps * 32), smem, J));
+  return OFDFT_OK;
+}
+
+template <typename T, bool XAX, int MODE>
+int fd_pass(ofdft_ctx* c, const FdJob& J) {
+  const int tiles = J.ax.pe / kFdTile + J.ax.po / kFdTile;
+  const int tpw = tiles > 16 ? 2 : 1, warps = (tiles + tpw - 1) / tpw;
+  // FP32: panels of 64 columns, or of 32 where 64 would leave SMs without a block;
+  // float-float: 32 (its accumulators and its panel take twice the room)
+  const bool wide = sizeof(T) == 4 && J.ncols >= 128LL * c->sms;
+  if constexpr (sizeof(T) == 4) {
+    if (wide)
+      return tpw == 1 ? fd_launch<T, XAX, MODE, 4, 1>(c, J, warps) : fd_launch<T, XAX, MODE, 4, 2>(c, J, warps);
+  }
+  return tpw == 1 ? fd_launch<T, XAX, MODE, 2, 1>(c, J, warps) : fd_launch<T, XAX, MODE, 2, 2>(c, J, warps);
+}
+
+// z = M r by fast diagonalisation, with r.z and the PCG scalars as the V-cycle's
+// last pass forms them.  scratch: fd_scratch(g) elements of T.
+template <typename T>
+int fd_apply(ofdft_ctx* c, const GridDev& g, const FdPlan& P, const T* r, T* z, void* scratch, CgScalars* sc) {
+  TRY((fd_pass<T, true, FD_FWD>(c, fd_job<T>(g, P, 0, r, z, scratch, sc))));
+  TRY((fd_pass<T, false, FD_FWD>(c, fd_job<T>(g, P, 1, r, z, scratch, sc))));
+  TRY((fd_pass<T, false, FD_SOLVE>(c, fd_job<T>(g, P, 2, r, z, scratch, sc))));
+  TRY((fd_pass<T, false, FD_INV>(c, fd_job<T>(g, P, 3, r, z, scratch, sc))));
+  return fd_pass<T, true, FD_INV>(c, fd_job<T>(g, P, 4, r, z, scratch, sc));
 }
 
 template <typename T, int R, int V, class L, class E>

@@ -1,0 +1,117 @@
+"""Fast diagonalisation as the Poisson CG's preconditioner, through the C ABI, at
+the sizes where its panels, tiles and halves have edges.
+
+The right-hand side is the discrete operator applied to a known field (the
+oracle's stencil), so the solve must return that field.  Tolerance, from
+||phi - phi*|| <= ||A^-1|| ||r|| with ||r|| <= tol ||4 pi rho||: relative to
+||phi*|| at most tol times the operator's condition number, of which the largest
+and smallest eigenvalues are bounded by the symbol: lambda_max <= 12 / h^2 sum_p
+|w_p h^2| and lambda_min >= 3 (pi / (n_max + 1))^2 / h^2 / 2; FP32 results add
+their rounding (2^-24 a value, doubled).
+"""
+import os
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import oracle as O
+from paper_1405_6456_gb300 import build as B
+from paper_1405_6456_gb300 import ofdft as F
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+def _context(**env):
+    old = {k: os.environ.get(k) for k in env}
+    os.environ.update({k: str(v) for k, v in env.items()})
+    try:
+        return F.Context(0)
+    finally:
+        for k, v in old.items():
+            if v is None:
+                del os.environ[k]
+            else:
+                os.environ[k] = v
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    B.build()
+    c = F.Context(0)
+    yield c
+    c.close()
+
+
+# the shortest axis; odd halves, rows that are no whole vectors; one node past a
+# tile; two tiles a warp (more than 256 nodes) on each axis in turn; the longest
+SIZES = [((32, 32, 32), 12), ((33, 35, 34), 12), ((47, 40, 39), 2), ((64, 97, 36), 8), ((130, 33, 66), 6),
+         ((257, 32, 33), 12), ((32, 300, 34), 10), ((36, 32, 512), 12), ((512, 32, 32), 4)]
+
+
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+@pytest.mark.parametrize("dims,order", SIZES)
+def test_poisson_returns_the_known_field(ctx, dims, order, dtype):
+    g = F.make_grid(*dims, 0.5)
+    og = O.make_grid(*dims, 0.5, (0.0, 0.0, 0.0))
+    phi_m = np.random.default_rng(sum(dims)).standard_normal(g.shape)
+    rho = -O.laplacian(og, order // 2, phi_m) / (4.0 * np.pi)
+    if dtype == torch.float32:
+        rho = rho.astype(np.float32)
+    tol = 1e-10 if dtype == torch.float64 else 1e-8
+    phi = torch.zeros(g.shape, dtype=dtype, device=DEV)
+    ctx.reset_counters()
+    st = ctx.poisson(g, order, phi, rho=torch.as_tensor(rho, device=DEV), tol=tol)
+    cnt = ctx.counters()
+    assert st.rel_residual <= tol
+    assert cnt.kind_launches[F.K_MG] == 5 * cnt.kind_launches[F.K_CG_DIR_STENCIL]  # five passes a step
+    assert st.iterations <= 6  # V-cycles: 17 to 35
+    w = np.abs(O.lap_weights(order // 2, 1.0))
+    lam_max, lam_min = 12.0 * w[1:].sum(), 1.5 * (np.pi / (max(dims) + 1)) ** 2
+    cond = lam_max / lam_min
+    bound = tol * cond
+    if dtype == torch.float32:
+        # rho itself is rounded to FP32 (2^-25 a value), which A^-1 carries to phi
+        bound += 2.0**-25 * cond + 2.0**-23
+    err = np.linalg.norm(phi.double().cpu().numpy() - phi_m) / np.linalg.norm(phi_m)
+    assert err <= bound, (err, bound)
+
+
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+def test_unaligned_fields_and_the_vcycle_agree(ctx, dtype):
+    """Fields that start off a 16-byte boundary take the element-wise rows of the x
+    passes; the V-cycle (OFDFT_FD=0) reaches the same potential."""
+    dims, order = (48, 40, 36), 12
+    g = F.make_grid(*dims, 0.5)
+    rho = np.random.default_rng(4).standard_normal(g.shape)
+    tol = 1e-10 if dtype == torch.float64 else 1e-9
+    sols = []
+    cv = _context(OFDFT_FD=0)
+    for c, off in ((ctx, 0), (ctx, 1), (cv, 0)):
+        buf = torch.zeros(2, g.size + 1, dtype=dtype, device=DEV)
+        phi, r = (buf[k, off:off + g.size].view(g.shape) for k in (0, 1))
+        r.copy_(torch.as_tensor(rho))
+        st = c.poisson(g, order, phi, rho=r, tol=tol)
+        assert st.rel_residual <= tol
+        sols.append(phi.double().cpu().numpy())
+    cv.close()
+    # each is within tol * cond of the solution (cond <= 27 / 6.5e-3 at n = 48), FP32 ones with their rounding
+    bound = 2.0 * (tol * 4.2e3 + (0.0 if dtype == torch.float64 else 2.0**-23))
+    for s in sols[1:]:
+        assert np.linalg.norm(s - sols[0]) <= bound * np.linalg.norm(sols[0])
+
+
+def test_short_axes_keep_the_vcycle(ctx):
+    """One axis below 32 nodes: the multigrid launches of one iteration are not the
+    five passes."""
+    g = F.make_grid(31, 40, 40, 0.5)
+    rho = torch.as_tensor(np.random.default_rng(4).standard_normal(g.shape), device=DEV)
+    phi = torch.zeros(g.shape, dtype=torch.float64, device=DEV)
+    ctx.reset_counters()
+    st = ctx.poisson(g, 12, phi, rho=rho, tol=1e-10)
+    assert st.iterations > 6
+    assert ctx.counters().kind_launches[F.K_MG] > 5 * st.iterations
