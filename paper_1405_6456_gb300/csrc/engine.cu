@@ -232,6 +232,12 @@ int carve(ofdft_ctx* c, Slot<T>* S, int prec) {
     S->mgc = (T*)take(std::max<long long>(S->mg.elems, 1) * sizeof(T));
   }
   S->pc = (S->mg.ok && c->precond == OFDFT_PRECOND_MG) ? 1 : 0;
+  // the fast diagonalisation's scratch takes the place of the cycle's scratch and
+  // levels (adjacent pieces, together at least G (1 + 3/8) elements); eight warps
+  // of two tiles cover 256 nodes
+  if (S->pc && fd_usable(c, S->g, 256) &&
+      fd_scratch(S->g) * sizeof(T) <= (size_t)((char*)(S->mgc + S->mg.elems) - (char*)S->mt))
+    TRY(fd_plan(c, S->g, S->Rr, S->h, &S->mg.fd));
   if ((size_t)(p - (char*)S->mem) > S->bytes) return fail(c, OFDFT_EINVAL, "slot workspace carve overflow");
   CU(cudaMemsetAsync(S->counter, 0, 256, c->stream));
   return OFDFT_OK;
@@ -408,17 +414,67 @@ struct Engine {
     return OFDFT_OK;
   }
 
-  // z = M r for every preconditioned slot: one V-cycle per grid, each pass of
-  // the cycle shared by the grids that have that level (S3 + S11).
+  // One pass of the fast diagonalisation over the grids of `v`: a launch for the
+  // grids with one tile of outputs a warp on this axis, and one for those with two.
+  template <bool XAX, int MODE, class GetR, class GetSc>
+  int fd_pass_batch(const std::vector<Slot<T>*>& v, int pass, GetR getr, GetSc getsc) {
+    constexpr int CT = sizeof(T) == 4 ? 4 : 2;
+    for (int tpw = 1; tpw <= 2; ++tpw) {
+      std::vector<FdTile> tiles;
+      std::vector<FdJob> jobs;
+      size_t smem = 0;
+      for (Slot<T>* S : v) {
+        FdJob J = fd_job<T>(S->g, S->mg.fd, pass, getr(S), S->mz, S->mt, getsc(S));
+        if ((J.ax.pe + J.ax.po) / kFdTile > kFdBatchWarps ? tpw == 1 : tpw == 2) continue;
+        J.red = slot_red(S);
+        J.nblocks = (int)((J.ncols + 16 * CT - 1) / (16 * CT));
+        for (int k = 0; k < J.nblocks; ++k) tiles.push_back(FdTile{(int)jobs.size(), k});
+        jobs.push_back(J);
+        smem = std::max(smem, (size_t)fd_panel_floats(J.ax, XAX, 16 * CT) * sizeof(T));
+      }
+      if (tiles.empty()) continue;
+      smem += (size_t)kFdBatchWarps * fd_ring_floats<sizeof(T) == 8>() * sizeof(float);
+      const void *pt = nullptr, *pj = nullptr;
+      TRY(put(B->d_tiles, tiles, &pt));
+      TRY(put(B->d_ops, jobs, &pj));
+      static bool attr_dev[64] = {false};  // per instantiation and device
+      if (c->device < 0 || c->device >= 64) return fail(c, OFDFT_EINVAL, "device index out of range");
+      if (!attr_dev[c->device]) {
+        CU(cudaFuncSetAttribute(fd_batch_kernel<T, XAX, MODE, CT, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                kFdSmem));
+        CU(cudaFuncSetAttribute(fd_batch_kernel<T, XAX, MODE, CT, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                kFdSmem));
+        attr_dev[c->device] = true;
+      }
+      ProfScope ps_(c, OFDFT_K_MG);
+      const unsigned nb = (unsigned)tiles.size();
+      if (tpw == 1)
+        fd_batch_kernel<T, XAX, MODE, CT, 1><<<nb, kFdBatchWarps * 32, smem, c->stream>>>((const FdTile*)pt, (const FdJob*)pj);
+      else
+        fd_batch_kernel<T, XAX, MODE, CT, 2><<<nb, kFdBatchWarps * 32, smem, c->stream>>>((const FdTile*)pt, (const FdJob*)pj);
+      CU(cudaGetLastError());
+    }
+    return OFDFT_OK;
+  }
+
+  // z = M r for every preconditioned slot: by fast diagonalisation, or one V-cycle
+  // per grid, each pass shared by the grids that take it (S3 + S11).
   template <class GetR, class GetSc>
   int mg_cycle(const std::vector<Slot<T>*>& slots, GetR getr, GetSc getsc) {
-    std::vector<Slot<T>*> pcs;
+    std::vector<Slot<T>*> pcs, fds;
     int maxlc = 0;
     for (Slot<T>* S : slots)
-      if (S->pc) {
+      if (S->pc && S->mg.fd.on) {
+        fds.push_back(S);
+      } else if (S->pc) {
         pcs.push_back(S);
         maxlc = std::max(maxlc, S->mg.lc);
       }
+    TRY((fd_pass_batch<true, FD_FWD>(fds, 0, getr, getsc)));
+    TRY((fd_pass_batch<false, FD_FWD>(fds, 1, getr, getsc)));
+    TRY((fd_pass_batch<false, FD_SOLVE>(fds, 2, getr, getsc)));
+    TRY((fd_pass_batch<false, FD_INV>(fds, 3, getr, getsc)));
+    TRY((fd_pass_batch<true, FD_INV>(fds, 4, getr, getsc)));
     if (pcs.empty()) return OFDFT_OK;
     const T om = (T)c->mg_omega;
     auto nodes = [](Slot<T>* S, int l) { return mg_nodes(S->mg.d[l]); };
@@ -646,7 +702,7 @@ struct Engine {
       key.push_back((long long)getx(S));
       key.push_back((long long)getr(S));
       key.push_back((long long)getsc(S));
-      key.push_back(S->pc);
+      key.push_back(S->pc + (S->mg.fd.on ? 2 : 0));
       idx.push_back(S->index);
     }
     for (auto& e : B->graphs)
@@ -781,14 +837,23 @@ struct Engine {
       if (c->autotune) TRY(tune_zdepth(set, getr));
       TRY(cg_iteration(set, fold, getx, getr, getsc));  // also sets kernel attributes outside the capture
       B->eager_iters++;
-      cudaGraphExec_t exec = nullptr;
-      TRY(loop_graph(set, fold, getx, getr, getsc, &exec));
-      CU(cudaGraphLaunch(exec, c->stream));
-      B->graph_replays++;
-      TRY(read_scalars());
-      long long its = 0;
-      for (Slot<T>* S : slots) its = std::max<long long>(its, hostsc(S).iters);
-      B->graph_iters += its;
+      // one step of a directly inverted operator mostly ends its solve; the loop
+      // graph runs only while some solve of the set is left
+      bool left = true;
+      if (std::any_of(slots.begin(), slots.end(), [](Slot<T>* S) { return S->mg.fd.on; })) {
+        TRY(read_scalars());
+        left = std::any_of(slots.begin(), slots.end(), [&](Slot<T>* S) { return !hostsc(S).done; });
+      }
+      if (left) {
+        cudaGraphExec_t exec = nullptr;
+        TRY(loop_graph(set, fold, getx, getr, getsc, &exec));
+        CU(cudaGraphLaunch(exec, c->stream));
+        B->graph_replays++;
+        TRY(read_scalars());
+        long long its = 0;
+        for (Slot<T>* S : slots) its = std::max<long long>(its, hostsc(S).iters);
+        B->graph_iters += its;
+      }
       std::vector<Slot<T>*> still;
       for (Slot<T>* S : slots)
         if (!hostsc(S).done) still.push_back(S);

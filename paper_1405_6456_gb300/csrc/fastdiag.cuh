@@ -746,4 +746,21 @@ __global__ void __maxnreg__(TPW == 1 ? 80 : 128) fd_kernel(const __grid_constant
   fd_panel<T, XAX, MODE, CT, TPW>(J, (long long)blockIdx.x * (16 * CT), blockIdx.x, fd_sm);
 }
 
+// The same pass for several grids of a batch: block b takes panel tiles[b].panel
+// of job tiles[b].job, always with eight warps, so that a grid's sums do not
+// depend on the others.
+struct FdTile {
+  int job, panel;
+};
+constexpr int kFdBatchWarps = 8;
+template <typename T, bool XAX, int MODE, int CT, int TPW>
+__global__ void __maxnreg__(TPW == 1 ? 80 : 128)
+    fd_batch_kernel(const FdTile* __restrict__ tiles, const FdJob* __restrict__ jobs) {
+  extern __shared__ __align__(16) float fd_sm[];
+  const FdTile t = tiles[blockIdx.x];
+  const FdJob J = jobs[t.job];
+  if (J.sc->done) return;
+  fd_panel<T, XAX, MODE, CT, TPW>(J, (long long)t.panel * (16 * CT), t.panel, fd_sm);
+}
+
 }  // namespace ofd

@@ -115,3 +115,33 @@ def test_short_axes_keep_the_vcycle(ctx):
     st = ctx.poisson(g, 12, phi, rho=rho, tol=1e-10)
     assert st.iterations > 6
     assert ctx.counters().kind_launches[F.K_MG] > 5 * st.iterations
+
+
+@pytest.mark.parametrize("prec", [F.PREC_FP64, F.PREC_MIXED])
+def test_batched_passes_do_not_depend_on_the_mix(ctx, prec):
+    """Grids of one and of two output tiles a warp in one batch (one axis over 128
+    nodes), beside one that keeps the V-cycle: each result is the same alone, bit for
+    bit, and the single solve's within the solver's tolerance (E is second order in
+    what tol_inner leaves: 1e-8 Ha/atom, a tenth of the bound)."""
+    from paper_1405_6456_gb300 import workloads as W
+    c = W.tiny_cluster("dimer", h=0.6, fd_order=8)
+    p = F.default_params(fd_order=8, precision=prec, tol_E=1e-7, tol_inner=1e-8)
+    grids = []
+    for n in ((44, 34, 36), (140, 33, 34), (44, 30, 32)):
+        grids.append(F.make_grid(*n, 0.6, tuple(-0.3 * k for k in n)))
+    alone = []
+    for g in grids:
+        bt = F.Batch(ctx, prec, 1 << 32)
+        rid = bt.submit(c.R, c.Z, c.h, p, grid=g)
+        bt.run()
+        alone.append(bt.poll(rid))
+        bt.close()
+    bt = F.Batch(ctx, prec, 1 << 32)
+    ids = [bt.submit(c.R, c.Z, c.h, p, grid=g) for g in grids]
+    bt.run()
+    for g, rid, (Ea, Fa, _) in zip(grids, ids, alone):
+        E, Fv, st = bt.poll(rid)
+        assert st.converged and E == Ea and np.array_equal(Fv, Fa)
+        E1, _, _ = ctx.solve(c.R, c.Z, c.h, p, grid=g)
+        assert abs(E - E1) / c.M <= 1e-7
+    bt.close()
