@@ -1410,6 +1410,12 @@ int upload_atoms(ofdft_ctx* c, const double* R_host, const double* Z_host, int M
   A->oz = g ? g->origin[2] : 0.0;
   A->sigma = sigma;
   A->rc = rc;
+  A->rc2 = sq_threshold(rc);
+  if (!c->v[V_GTAB].p) {
+    TRY(ensure(c, c->v[V_GTAB], kGtabBytes));
+    CU(cudaMemcpyAsync(c->v[V_GTAB].p, gtab_host().data(), kGtabBytes, cudaMemcpyHostToDevice, c->stream));
+  }
+  A->gtab = vec<double>(c, V_GTAB);
   return OFDFT_OK;
 }
 
@@ -1449,8 +1455,8 @@ inline void atom_box_lo(const double* R_host, int a0, int na, const ofdft_grid* 
 }
 
 template <typename T, int R>
-int launch_force_boxes(ofdft_ctx* c, const AtomArgs& A, int a0, int na, int vdim, int bdim, const int* lo,
-                       const Weights<double>& W, double* vbox, double* bbox);
+int launch_force_boxes(ofdft_ctx* c, const GridDev& g, const AtomArgs& A, int a0, int na, int vdim, int bdim,
+                       const int* lo, const Weights<double>& W, double* vbox, double* bbox, double* es_out = nullptr);
 
 // Identity of the b_J tables of a geometry: everything they depend on.
 inline std::vector<double> btab_key(const ofdft_grid* gr, int R, const double* R_host, const double* Z_host, int M,
@@ -1489,19 +1495,17 @@ int pseudocharge_tables(ofdft_ctx* c, const ofdft_grid* gr, const GridDev& g, co
   double* bacc = multi ? vec<double>(c, V_BACC) : nullptr;
   std::vector<int> lo((size_t)3 * t.batch);
   const dim3 grid((g.n1 + AT - 1) / AT, (g.n2 + AT - 1) / AT, (g.n3 + AT - 1) / AT);
-  TRY(ensure_partials(c, (long long)grid.x * grid.y * grid.z, 1));
   CU(cudaMemsetAsync(es_dev, 0, sizeof(double), c->stream));
   for (int a0 = 0; a0 < M; a0 += t.batch) {
     const int na = std::min(t.batch, M - a0);
     double* bbox = keep ? btab + (size_t)a0 * t.bper : vbox + (size_t)t.batch * t.vper;
     atom_box_lo(R_host, a0, na, gr, t.rb, lo);
     CU(cudaMemcpyAsync(lo_dev, lo.data(), 3 * na * sizeof(int), cudaMemcpyHostToDevice, c->stream));
-    TRY((launch_force_boxes<T, R>(c, A, a0, na, t.vdim, t.bdim, lo_dev, W, vbox, bbox)));
+    TRY((launch_force_boxes<T, R>(c, g, A, a0, na, t.vdim, t.bdim, lo_dev, W, vbox, bbox, es_dev)));
     {
       ProfScope ps_(c, OFDFT_K_ATOMS);
       pseudocharge_gather_kernel<T><<<grid, dim3(AT, AT, AT), 0, c->stream>>>(
-          g, A, a0, na, t.box, t.bdim, t.vdim, R, lo_dev, vbox, bbox, bacc, a0 == 0 ? 1 : 0,
-          a0 + na >= M ? 1 : 0, b, es_dev, red(c));
+          g, A, a0, na, t.box, t.bdim, R, lo_dev, bbox, bacc, a0 == 0 ? 1 : 0, a0 + na >= M ? 1 : 0, b);
     }
     CU(cudaGetLastError());
   }
@@ -1544,9 +1548,31 @@ int device_guess(ofdft_ctx* c, const ofdft_grid* gr, const double* R_host, const
   const GridDev g = gdev(gr);
   dim3 grid((g.n1 + AT - 1) / AT, (g.n2 + AT - 1) / AT, (g.n3 + AT - 1) / AT);
   TRY(ensure_partials(c, (long long)grid.x * grid.y * grid.z, 1));
+  // axis tables over each atom's box (one node of slack), or over the whole grid
+  // where the boxes would be larger
+  const int nmax = std::max(g.n1, std::max(g.n2, g.n3));
+  const double rbd = ceil(gcut / gr->h) + 1.0;
+  const bool whole = !(2.0 * rbd + 1.0 < nmax);
+  const int rb = whole ? 0 : (int)rbd, m = whole ? nmax : 2 * rb + 1;
+  TRY(ensure(c, c->v[V_ATOM1], (size_t)M * 6 * m * sizeof(double)));
+  TRY(ensure(c, c->v[V_ATOM2], (size_t)M * 3 * sizeof(int)));
+  std::vector<int> lo((size_t)3 * M, 0);
+  for (int k = 0; k < 3 * M && !whole; ++k) {
+    const double q = floor((R_host[k] - gr->origin[k % 3]) / gr->h - 0.5);
+    lo[k] = (int)std::min(std::max(q, -1e9), 1e9) - rb + 1;
+  }
+  int* lo_dev = vec<int>(c, V_ATOM2);
+  double* gsq = vec<double>(c, V_ATOM1);
+  double* gex = gsq + (size_t)M * 3 * m;
+  CU(cudaMemcpyAsync(lo_dev, lo.data(), 3 * (size_t)M * sizeof(int), cudaMemcpyHostToDevice, c->stream));
   {
     ProfScope ps_(c, OFDFT_K_ATOMS);
-    guess_kernel<T><<<grid, dim3(AT, AT, AT), 0, c->stream>>>(g, A, gsig, gcut, u, c->scal + 21, red(c));
+    guess_axes_kernel<<<pointwise_blocks(c, (long long)M * 12 * m), 256, 0, c->stream>>>(A, gsig, m, lo_dev, gsq, gex);
+  }
+  CU(cudaGetLastError());
+  {
+    ProfScope ps_(c, OFDFT_K_ATOMS);
+    guess_kernel<T><<<grid, dim3(AT, AT, AT), 0, c->stream>>>(g, A, gcut, m, lo_dev, gsq, gex, u, c->scal + 21, red(c));
   }
   CU(cudaGetLastError());
   {
@@ -1558,23 +1584,38 @@ int device_guess(ofdft_ctx* c, const ofdft_grid* gr, const double* R_host, const
   return OFDFT_OK;
 }
 
+// Room for the potential's coefficients and the squared offsets of a box of up to
+// 1024 nodes a side (a per-device setting, cheap to repeat).
+inline int atom_smem_attr(ofdft_ctx* c, const void* kern) {
+  CU(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kGtabBytes + 3 * 1024 * (int)sizeof(double)));
+  return OFDFT_OK;
+}
+
 template <typename T, int R>
-int launch_force_boxes(ofdft_ctx* c, const AtomArgs& A, int a0, int na, int vdim, int bdim, const int* lo,
-                       const Weights<double>& W, double* vbox, double* bbox) {
+int launch_force_boxes(ofdft_ctx* c, const GridDev& g, const AtomArgs& A, int a0, int na, int vdim, int bdim,
+                       const int* lo, const Weights<double>& W, double* vbox, double* bbox, double* es_out) {
   // one block row per atom, about eight blocks per SM in total
   auto grid_for = [&](long long per) {
     const long long bx = std::max<long long>(1, std::min<long long>((per + 255) / 256, ((long long)c->sms * 8 + na - 1) / na));
     return dim3((unsigned)bx, (unsigned)na);
   };
+  TRY(atom_smem_attr(c, (const void*)force_vbox_kernel));
   {
     ProfScope ps_(c, OFDFT_K_ATOMS);
-    force_vbox_kernel<<<grid_for((long long)vdim * vdim * vdim), 256, 0, c->stream>>>(A, a0, vdim, R, lo, vbox);
+    force_vbox_kernel<<<grid_for((long long)vdim * vdim * vdim), 256, kGtabBytes + 3 * vdim * sizeof(double),
+                        c->stream>>>(A, a0, vdim, R, lo, vbox);
   }
   CU(cudaGetLastError());
-  {
+  const dim3 gb = grid_for((long long)bdim * bdim * bdim);
+  const size_t smem = 3 * bdim * sizeof(double);
+  if (es_out) {  // also the self energy's sum of b_J V_J
+    TRY(ensure_partials(c, (long long)gb.x * gb.y, 1));
     ProfScope ps_(c, OFDFT_K_ATOMS);
-    force_bbox_kernel<R><<<grid_for((long long)bdim * bdim * bdim), 256, 0, c->stream>>>(A, a0, vdim, bdim, lo, W,
-                                                                                        vbox, bbox);
+    force_bbox_kernel<R, true><<<gb, 256, smem, c->stream>>>(g, A, a0, vdim, bdim, lo, W, vbox, bbox, es_out, red(c));
+  } else {
+    ProfScope ps_(c, OFDFT_K_ATOMS);
+    force_bbox_kernel<R, false><<<gb, 256, smem, c->stream>>>(g, A, a0, vdim, bdim, lo, W, vbox, bbox, nullptr,
+                                                              RedBuf{});
   }
   CU(cudaGetLastError());
   return OFDFT_OK;
@@ -1584,9 +1625,10 @@ template <typename T, int R>
 int launch_force_ball(ofdft_ctx* c, const GridDev& g, const AtomArgs& A, int a0, int na, int bdim, int box,
                       const int* lo, const Weights<double>& W, const Weights<double>& Wt, const double* bbox,
                       const T* phi, int exact, double* partial, int nblk) {
+  TRY(atom_smem_attr(c, (const void*)force_ball_kernel<T, R>));
   {
     ProfScope ps_(c, OFDFT_K_ATOMS);
-    force_ball_kernel<T, R><<<dim3(nblk, na), 256, 0, c->stream>>>(g, A, a0, bdim, box, lo, W, Wt, bbox, phi, exact,
+    force_ball_kernel<T, R><<<dim3(nblk, na), 256, kGtabBytes + 3 * box * sizeof(double), c->stream>>>(g, A, a0, bdim, box, lo, W, Wt, bbox, phi, exact,
                                                                     partial);
   }
   CU(cudaGetLastError());
@@ -1611,7 +1653,10 @@ int device_forces(ofdft_ctx* c, const ofdft_grid* gr, int R, const double* R_hos
   int batch = (int)std::max<long long>(1, std::min<long long>(M, (256ll << 20) / ((vper + bper) * 8)));
   batch = std::min(batch, 16384);  // atoms of one launch (one block row each)
   if (exact) batch = std::min(M, 4096);
-  const int nblk = std::max(1, std::min(64, (int)((long long)box * box * box / 2048) + 1));
+  // blocks per atom: about eight per SM over all atoms (each loads the potential's
+  // coefficients), the same whatever the batch, so that an atom's sums are too
+  const int nblk = std::max(1, std::min(std::min(64, (int)((long long)box * box * box / 2048) + 1),
+                                        (8 * c->sms + M - 1) / M));
   // the b_J tables of this very geometry, kept by the solve's pseudocharge pass
   const bool kept = !exact && !c->btab_key.empty() && c->btab_key == btab_key(gr, R, R_host, Z_host, M, sigma, rc);
   if (kept) batch = std::min(M, 4096);
@@ -1634,12 +1679,12 @@ int device_forces(ofdft_ctx* c, const ofdft_grid* gr, int R, const double* R_hos
     if (kept) bbox = vec<double>(c, V_BTAB) + (size_t)a0 * bper;
     if (!exact && !kept) {
       switch (R) {
-        case 1: TRY((launch_force_boxes<T, 1>(c, A, a0, na, vdim, bdim, lo_dev, W, vbox, bbox))); break;
-        case 2: TRY((launch_force_boxes<T, 2>(c, A, a0, na, vdim, bdim, lo_dev, W, vbox, bbox))); break;
-        case 3: TRY((launch_force_boxes<T, 3>(c, A, a0, na, vdim, bdim, lo_dev, W, vbox, bbox))); break;
-        case 4: TRY((launch_force_boxes<T, 4>(c, A, a0, na, vdim, bdim, lo_dev, W, vbox, bbox))); break;
-        case 5: TRY((launch_force_boxes<T, 5>(c, A, a0, na, vdim, bdim, lo_dev, W, vbox, bbox))); break;
-        case 6: TRY((launch_force_boxes<T, 6>(c, A, a0, na, vdim, bdim, lo_dev, W, vbox, bbox))); break;
+        case 1: TRY((launch_force_boxes<T, 1>(c, g, A, a0, na, vdim, bdim, lo_dev, W, vbox, bbox))); break;
+        case 2: TRY((launch_force_boxes<T, 2>(c, g, A, a0, na, vdim, bdim, lo_dev, W, vbox, bbox))); break;
+        case 3: TRY((launch_force_boxes<T, 3>(c, g, A, a0, na, vdim, bdim, lo_dev, W, vbox, bbox))); break;
+        case 4: TRY((launch_force_boxes<T, 4>(c, g, A, a0, na, vdim, bdim, lo_dev, W, vbox, bbox))); break;
+        case 5: TRY((launch_force_boxes<T, 5>(c, g, A, a0, na, vdim, bdim, lo_dev, W, vbox, bbox))); break;
+        case 6: TRY((launch_force_boxes<T, 6>(c, g, A, a0, na, vdim, bdim, lo_dev, W, vbox, bbox))); break;
       }
     }
     switch (R) {

@@ -130,6 +130,7 @@ enum Vec {
   V_B2,                                // mixed: the FP64 pseudocharge as float-float pairs (residual pass)
   V_BTAB,                              // b_J tables of every atom, kept from the pseudocharge for the forces
   V_OC,                                // overlap correction: b, b~, V, V~ (FP64)
+  V_GTAB,                              // coefficients of the nuclear potential (gtab_v)
   V_COUNT
 };
 
@@ -972,6 +973,52 @@ inline void fill_energy(const EvalOut& o, double h, const ofdft_params* p, doubl
   e->rs = h3 * o.sums[7];
   e->rs_pc = e->rs;
   e->gnorm2 = h3 * o.sums[8];
+}
+
+// Coefficients of gtab_v, [power][interval]: the Taylor series of
+// g(s) = erf(sqrt s)/sqrt s around c = (middle of the interval of s + 1) - 1.  Up to
+// c = 3 from g's power series (2/sqrt pi) sum (-s)^j / (j! (2j + 1)); beyond from
+// 2 s g' + g = (2/sqrt pi) e^{-s}, whose recurrence for the coefficients,
+//   a_{k+1} = ((2/sqrt pi) e^{-c} (-1)^k / k! - (2k + 1) a_k) / (2 c (k + 1)),
+// is stable forwards there (a_k ~ c^{-k} is its dominant solution).
+inline const std::vector<double>& gtab_host() {
+  static const std::vector<double> tab = [] {
+    std::vector<double> t((size_t)kGtabN * kGtabC);
+    const long double tsp = 2.0L / sqrtl(acosl(-1.0L));
+    for (int i = 0; i < kGtabN; ++i) {
+      const long double c = ldexpl(1.0L + ((i % 64) + 0.5L) / 64.0L, i / 64) - 1.0L;
+      long double a[kGtabC];
+      if (c < 3.0L) {
+        for (int k = 0; k < kGtabC; ++k) {
+          long double s = 0.0L, f = 1.0L;  // f = C(j, k) c^{j-k} / j!, from j = k on
+          for (int m = 1; m <= k; ++m) f /= m;
+          for (int j = k; j < k + 60; ++j) {
+            s += ((j & 1) ? -f : f) / (2 * j + 1);
+            f *= c / (j + 1 - k);
+          }
+          a[k] = tsp * s;
+        }
+      } else {
+        a[0] = erfl(sqrtl(c)) / sqrtl(c);
+        long double f = tsp * expl(-c);
+        for (int k = 0; k + 1 < kGtabC; ++k) {
+          a[k + 1] = (f - (2 * k + 1) * a[k]) / (2.0L * c * (k + 1));
+          f *= -1.0L / (k + 1);
+        }
+      }
+      for (int k = 0; k < kGtabC; ++k) t[(size_t)k * kGtabN + i] = (double)a[k];
+    }
+    return t;
+  }();
+  return tab;
+}
+// The smallest d2 whose rounded square root is not below rc: r < rc is d2 < rc2
+// exactly, without a square root per node.
+inline double sq_threshold(double rc) {
+  double x = rc * rc;
+  while (sqrt(x) >= rc) x = nextafter(x, 0.0);
+  while (sqrt(x) < rc) x = nextafter(x, INFINITY);
+  return x;
 }
 
 // Routines of api.cu used by the batched engine (instantiated for double and float).

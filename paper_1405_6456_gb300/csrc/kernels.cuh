@@ -2792,22 +2792,72 @@ struct OpConvert {
 __device__ __forceinline__ double node_off(double origin, int i, double h, double Ra) {
   return __dsub_rn(__dadd_rn(origin, __dmul_rn(__dadd_rn((double)i, 0.5), h)), Ra);
 }
-__device__ __forceinline__ double dist3(double x, double y, double z) {
-  return __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(x, x), __dmul_rn(y, y)), __dmul_rn(z, z)));
+
+// Gaussian nucleus V(r) = -Z erf(r/sigma)/r (with its r -> 0 limit) without erf,
+// square root or division: V = -(Z/sigma) g(s), s = (r/sigma)^2, where
+// g(s) = erf(sqrt s)/sqrt s is an entire function of s, from Taylor polynomials of
+// degree 7 around the middles of intervals of s + 1 in [1, 512), 64 to an octave
+// (the top six mantissa bits pick one).  The remainder is below 1e-17 of g
+// (|t| <= (s + 1)/128), and V's rounding error, 7.3e-17 rms over a ball of 10 sigma,
+// below that of erf, root and quotient (8.1e-17).  14 FP64 operations a node
+// instead of about 130: FP64 issues two a clock and SM, and bounds these kernels.
+// Coefficients (gtab_host, host.cuh) lie [power][interval] in shared memory.
+constexpr int kGtabN = 9 * 64, kGtabC = 8;
+constexpr int kGtabBytes = kGtabN * kGtabC * (int)sizeof(double);
+__device__ __forceinline__ void gtab_load(double* sm, const double* __restrict__ tab) {
+  for (int i = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z); i < kGtabN * kGtabC;
+       i += blockDim.x * blockDim.y * blockDim.z)
+    sm[i] = tab[i];
 }
-__device__ __forceinline__ double dist3_sq(double x, double y, double z) {
-  return __dadd_rn(__dadd_rn(__dmul_rn(x, x), __dmul_rn(y, y)), __dmul_rn(z, z));
+// V at squared distance d2; is2 = 1/sigma^2, zs = -Z/sigma
+__device__ __forceinline__ double gtab_v(const double* tab, double d2, double is2, double zs, double sigma) {
+  const double u = fma(d2, is2, 1.0);
+  if (!(u < 512.0)) return zs * sigma / sqrt(d2);
+  const int hi = __double2hiint(u);
+  const int k = (hi >> 14) - (0x3ff00000 >> 14);
+  const double t = u - __hiloint2double((hi & ~0x3fff) | 0x2000, 0);
+  double g = tab[(kGtabC - 1) * kGtabN + k];
+#pragma unroll
+  for (int c = kGtabC - 2; c >= 1; --c) g = fma(g, t, tab[c * kGtabN + k]);
+  return fma(zs, tab[k], (zs * t) * g);  // one rounding at V's own size
 }
 
-// Gaussian nucleus V(r) = -Z erf(r/sigma)/r and its r -> 0 limit.  From
-// r = 6 sigma on, 1 - erf(r/sigma) = erfc(r/sigma) < 2.2e-17 is below half a
-// unit in the last place of 1.0 (2^-54), so erf rounds to exactly 1 and
-// V = -Z/r; that skips the erf on most of an atom's table (r up to r_c + n h).
-__device__ __forceinline__ double gauss_v(double Z, double inv_sigma, double r) {
-  if (r < 1e-12 / inv_sigma) return -2.0 * Z * inv_sigma * 0.56418958354775628;  // 1/sqrt(pi)
-  const double x = r * inv_sigma;
-  if (x >= 6.0) return -Z / r;
-  return -Z * erf(x) / r;
+// Squared node offsets of a box of m nodes a side from node lo, for one atom, by
+// uncontracted IEEE operations: q[axis m + i].
+__device__ __forceinline__ void box_squares(double* q, int m, const int* lo, const double* R, double h,
+                                            const double* origin) {
+  for (int e = threadIdx.x; e < 3 * m; e += blockDim.x) {
+    const int d = e / m, i = e - d * m;
+    const double x = node_off(origin[d], lo[d] + i, h, R[d]);
+    q[e] = __dmul_rn(x, x);
+  }
+}
+
+// Walks the n nodes of a range, a warp's 32 at a time, and calls work(e) with full
+// warps only: nodes that pass test(e) queue up in the warp's 64 slots of shared
+// memory.  FP64 instructions cost the same for one active lane as for 32, and a
+// ball fills 22 to 40% of its box.
+template <class Test, class Work>
+__device__ __forceinline__ void warp_compact(unsigned first, unsigned last, unsigned step, unsigned* qe,
+                                             Test test, Work work) {
+  const int lane = threadIdx.x & 31;
+  int cnt = 0;
+  for (unsigned e0 = first; e0 < last; e0 += step) {
+    const unsigned e = e0 + lane;
+    const bool ok = e < last && test(e);
+    const unsigned m = __ballot_sync(0xffffffffu, ok);
+    if (ok) qe[cnt + __popc(m & ((1u << lane) - 1u))] = e;
+    __syncwarp();
+    cnt += __popc(m);
+    if (cnt >= 32) {
+      const unsigned w = qe[cnt - 32 + lane];
+      __syncwarp();
+      cnt -= 32;
+      work(w);
+    }
+  }
+  if (lane < cnt) work(qe[lane]);
+  __syncwarp();
 }
 
 // Conservative FP32 screen of node-to-atom distances.  The offset of a box's
@@ -2837,6 +2887,8 @@ struct AtomArgs {
   int M;
   double h, ox, oy, oz;  // spacing and origin
   double sigma, rc;
+  const double* gtab = nullptr;  // Taylor coefficients of gtab_v
+  double rc2 = 0.0;              // smallest d2 whose rounded square root is >= rc: r < rc is d2 < rc2
 };
 
 constexpr int AT = 8;  // atom-kernel tile edge (AT^3 = 512 threads)
@@ -2850,10 +2902,13 @@ __device__ __forceinline__ int tile_atoms(const AtomArgs& A, int a0, double cx, 
   const int a = a0 + tid;
   bool hit = false;
   if (a < A.M) {
-    const double dx = fmax(fabs(A.R[3 * a] - cx) - half, 0.0);
-    const double dy = fmax(fabs(A.R[3 * a + 1] - cy) - half, 0.0);
-    const double dz = fmax(fabs(A.R[3 * a + 2] - cz) - half, 0.0);
-    hit = dx * dx + dy * dy + dz * dz < reach * reach;
+    // in FP32 from the offset to the tile's centre, with the screen's margin: an atom
+    // too many costs a test a node, and FP64 here took as long as the pairs themselves
+    const float hf = (float)half;
+    const float dx = fmaxf(fabsf((float)(A.R[3 * a] - cx)) - hf, 0.0f);
+    const float dy = fmaxf(fabsf((float)(A.R[3 * a + 1] - cy)) - hf, 0.0f);
+    const float dz = fmaxf(fabsf((float)(A.R[3 * a + 2] - cz)) - hf, 0.0f);
+    hit = dx * dx + dy * dy + dz * dz < screen_r2(reach);
   }
   const unsigned m = __ballot_sync(0xffffffffu, hit);
   if (lane == 0) warp_cnt[warp] = __popc(m);
@@ -2868,11 +2923,36 @@ __device__ __forceinline__ int tile_atoms(const AtomArgs& A, int a0, double cx, 
   return total;
 }
 
+// Axis tables of the starting guess: for atom J and axis d the squared offsets of
+// the m nodes from lo[3 J + d] on (uncontracted, as node_off) and the Gaussian
+// factors exp(-o^2/(2 s^2)); the z axis' carry Z_J (2 pi s^2)^{-3/2}.  One thread a
+// value.
+static __global__ void __launch_bounds__(256) guess_axes_kernel(AtomArgs A, double gsig, int m,
+                                                                const int* __restrict__ lo, double* sq, double* ex) {
+  const double norm = pow(2.0 * kPi * gsig * gsig, -1.5), i2s2 = -1.0 / (2.0 * gsig * gsig);
+  const long long total = (long long)A.M * 3 * m;
+  for (long long e = (long long)blockIdx.x * 256 + threadIdx.x; e < total; e += (long long)gridDim.x * 256) {
+    const int jd = (int)(e / m), i = (int)(e - (long long)jd * m), d = jd % 3;
+    const double o = node_off(d == 0 ? A.ox : d == 1 ? A.oy : A.oz, lo[jd] + i, A.h, A.R[jd]);
+    const double o2 = __dmul_rn(o, o);
+    sq[e] = o2;
+    ex[e] = exp(o2 * i2s2) * (d == 2 ? A.Z[jd / 3] * norm : 1.0);
+  }
+}
+
 // rho_0 = sum_J Z_J (2 pi s^2)^{-3/2} exp(-r^2/(2 s^2)) (r < cut); writes
-// sqrt(rho_0) and reduces sum rho_0 (starting guess, Sec. 4).
+// sqrt(rho_0) and reduces sum rho_0 (starting guess, Sec. 4).  The Gaussian is a
+// product over the axes, so a node takes it from the axis tables: two FP64
+// operations a pair instead of an exponential.  Nodes the FP32 distance (see
+// DistScreen) puts clearly inside the cut need no FP64 test; those near it take
+// the exact one.  Bound by the FP64 pipe (pairs, and the root of every node) and
+// the staging of the tables: 666 atoms at 128^3 in 320 us (2,304 us with an
+// exponential a pair).
 template <typename T>
-__global__ void __launch_bounds__(512) guess_kernel(GridDev g, AtomArgs A, double gsig, double gcut,
-                                                    T* u, double* sum_out, RedBuf red) {
+__global__ void __launch_bounds__(512) guess_kernel(GridDev g, AtomArgs A, double gcut, int m,
+                                                    const int* __restrict__ lo, const double* __restrict__ gsq,
+                                                    const double* __restrict__ gex, T* u, double* sum_out,
+                                                    RedBuf red) {
   __shared__ int list[512];
   __shared__ int warp_cnt[16];
   __shared__ double smem[512 / 32];
@@ -2883,25 +2963,41 @@ __global__ void __launch_bounds__(512) guess_kernel(GridDev g, AtomArgs A, doubl
   const double half = 0.5 * AT * A.h;
   const double cx = A.ox + (blockIdx.x * AT) * A.h + half, cy = A.oy + (blockIdx.y * AT) * A.h + half,
                cz = A.oz + (blockIdx.z * AT) * A.h + half;
-  const double norm = pow(2.0 * kPi * gsig * gsig, -1.5);
-  // FP32 screen of the node's distance to each listed atom (see DistScreen):
-  // node x sits at ox + (x + 1/2) h
-  const float fx = (float)(A.ox + (x + 0.5) * A.h), fy = (float)(A.oy + (y + 0.5) * A.h),
-              fz = (float)(A.oz + (z + 0.5) * A.h);
+  // (relative to the tile's centre, so that wherever the box lies FP32 resolves them)
+  const float fx = (float)(A.ox + (x + 0.5) * A.h - cx), fy = (float)(A.oy + (y + 0.5) * A.h - cy),
+              fz = (float)(A.oz + (z + 0.5) * A.h - cz);
+  // the screen's error stays below 1e-4 r + 1e-3 either way
   const float cut2 = screen_r2(gcut);
+  const float sure = fmaxf((float)(gcut * (1.0 - 1e-4) - 1e-3), 0.0f), sure2 = sure * sure;
+  const double gcut2 = __dmul_rn(gcut, gcut);
+  constexpr int GA = 21;  // atoms staged at once: 24 values each, a thread a value
+  __shared__ double sq[GA][3][AT], ex[GA][3][AT];
+  __shared__ float fr[GA][3];
   double rho = 0.0;
   for (int a0 = 0; a0 < A.M; a0 += 512) {
     const int cnt = tile_atoms(A, a0, cx, cy, cz, half, gcut + A.h, list, warp_cnt);
-    if (inside) {
-      for (int t = 0; t < cnt; ++t) {
-        const int J = list[t];
-        const float dx = fx - (float)A.R[3 * J], dy = fy - (float)A.R[3 * J + 1], dz = fz - (float)A.R[3 * J + 2];
-        if (dx * dx + dy * dy + dz * dz > cut2) continue;
-        const double rx = node_off(A.ox, x, A.h, A.R[3 * J]), ry = node_off(A.oy, y, A.h, A.R[3 * J + 1]),
-                     rz = node_off(A.oz, z, A.h, A.R[3 * J + 2]);
-        const double r2 = dist3_sq(rx, ry, rz);
-        if (r2 < __dmul_rn(gcut, gcut)) rho += A.Z[J] * norm * exp(-r2 / (2.0 * gsig * gsig));
+    for (int t0 = 0; t0 < cnt; t0 += GA) {
+      const int na = min(GA, cnt - t0);
+      if (tid < na * 3 * AT) {
+        const int t = tid / (3 * AT), d = (tid / AT) % 3, i = tid % AT, jd = 3 * list[t0 + t] + d;
+        const int k = (d == 0 ? blockIdx.x : d == 1 ? blockIdx.y : blockIdx.z) * AT + i - lo[jd];
+        const bool in = k >= 0 && k < m;  // outside the table the offset alone exceeds the cut
+        sq[t][d][i] = in ? gsq[(size_t)jd * m + k] : 2.0 * gcut2;
+        ex[t][d][i] = in ? gex[(size_t)jd * m + k] : 0.0;
+        if (i == 0) fr[t][d] = (float)(A.R[jd] - (d == 0 ? cx : d == 1 ? cy : cz));
       }
+      __syncthreads();
+      if (inside)
+        for (int t = 0; t < na; ++t) {
+          const float dx = fx - fr[t][0], dy = fy - fr[t][1], dz = fz - fr[t][2];
+          const float f2 = dx * dx + dy * dy + dz * dz;
+          if (f2 > cut2) continue;
+          if (!(f2 < sure2) &&
+              !(__dadd_rn(__dadd_rn(sq[t][0][threadIdx.x], sq[t][1][threadIdx.y]), sq[t][2][threadIdx.z]) < gcut2))
+            continue;
+          rho = fma(ex[t][0][threadIdx.x] * ex[t][1][threadIdx.y], ex[t][2][threadIdx.z], rho);
+        }
+      __syncthreads();
     }
     __syncthreads();
   }
@@ -2925,50 +3021,61 @@ struct AtomBox {
 // V_J tabulated on the atom's box grown by 2R: vbox[a][...], one block row per
 // atom (blockIdx.y).  Only nodes within r_c + R h of the atom are ever read
 // (the stencil neighbours of the nodes of its ball, where b_J is nonzero), so
-// V_J is evaluated there only and the rest of the cube holds 0.
+// V_J is evaluated there only and the rest of the cube holds 0.  Bound by the FP64
+// pipe (14 operations a node of the ball, 33,500 nodes at h = 0.5, 12th order): 512
+// atoms in 415 us, 0.38 ms at the pipe's rate; with erf, root and quotient 3,590 us.
 static __global__ void __launch_bounds__(256) force_vbox_kernel(AtomArgs A, int a0, int vdim, int R,
                                                          const int* __restrict__ lo, double* vbox) {
+  extern __shared__ __align__(16) double atom_sm[];  // coefficients, squared offsets
+  __shared__ unsigned queue[8][64];
   const int a = blockIdx.y;
   const int J = a0 + a;
   const unsigned per = (unsigned)vdim * vdim * vdim;
   const double reach = A.rc + R * A.h + 1e-9 * (A.rc + A.h);
-  const int bx = lo[3 * a] - 2 * R, by = lo[3 * a + 1] - 2 * R, bz = lo[3 * a + 2] - 2 * R;
-  const double Rx = A.R[3 * J], Ry = A.R[3 * J + 1], Rz = A.R[3 * J + 2];
-  const DistScreen sc{(float)node_off(A.ox, bx, A.h, Rx), (float)node_off(A.oy, by, A.h, Ry),
-                      (float)node_off(A.oz, bz, A.h, Rz), (float)A.h, screen_r2(reach)};
+  const int bl[3] = {lo[3 * a] - 2 * R, lo[3 * a + 1] - 2 * R, lo[3 * a + 2] - 2 * R};
+  const double Rj[3] = {A.R[3 * J], A.R[3 * J + 1], A.R[3 * J + 2]}, og[3] = {A.ox, A.oy, A.oz};
+  const DistScreen sc{(float)node_off(A.ox, bl[0], A.h, Rj[0]), (float)node_off(A.oy, bl[1], A.h, Rj[1]),
+                      (float)node_off(A.oz, bl[2], A.h, Rj[2]), (float)A.h, screen_r2(reach)};
+  double* q = atom_sm + kGtabN * kGtabC;
+  gtab_load(atom_sm, A.gtab);
+  box_squares(q, vdim, bl, Rj, A.h, og);
+  __syncthreads();
+  const double is2 = 1.0 / (A.sigma * A.sigma), zs = -A.Z[J] / A.sigma;
   double* out = vbox + (size_t)a * per;
-  for (unsigned e = blockIdx.x * 256 + threadIdx.x; e < per; e += gridDim.x * 256) {
+  auto ijk = [&](unsigned e, int& i, int& j, int& k) {
     const unsigned jk = e / (unsigned)vdim;
-    const int i = (int)(e - jk * (unsigned)vdim);
-    const int k = (int)(jk / (unsigned)vdim);
-    const int j = (int)(jk - (unsigned)k * (unsigned)vdim);
-    double v = 0.0;
-    if (sc.maybe_within(i, j, k)) {
-      const double r = dist3(node_off(A.ox, bx + i, A.h, Rx), node_off(A.oy, by + j, A.h, Ry),
-                             node_off(A.oz, bz + k, A.h, Rz));
-      if (r <= reach) v = gauss_v(A.Z[J], 1.0 / A.sigma, r);
-    }
-    out[e] = v;
-  }
+    i = (int)(e - jk * (unsigned)vdim);
+    k = (int)(jk / (unsigned)vdim);
+    j = (int)(jk - (unsigned)k * (unsigned)vdim);
+  };
+  warp_compact(blockIdx.x * 256 + (threadIdx.x & ~31u), per, gridDim.x * 256, queue[threadIdx.x >> 5],
+               [&](unsigned e) {
+                 int i, j, k;
+                 ijk(e, i, j, k);
+                 const bool in = sc.maybe_within(i, j, k);
+                 if (!in) out[e] = 0.0;
+                 return in;
+               },
+               [&](unsigned e) {
+                 int i, j, k;
+                 ijk(e, i, j, k);
+                 const double d2 = __dadd_rn(__dadd_rn(q[i], q[vdim + j]), q[2 * vdim + k]);
+                 out[e] = gtab_v(atom_sm, d2, is2, zs, A.sigma);
+               });
 }
 
 // Pseudocharge from the atoms' tables (S1): for every node of a tile, the atoms
 // of [a0, a0 + na) (na <= 512) whose ball can reach the tile, in atom order,
 // add b_J (bbox, -(1/4 pi) L_h V_J inside r_c, 0 outside) to the node's running
-// FP64 sum (bacc, carried across launches of successive atom ranges) and
-// b_J V_J to the self-energy sum (added into es_out[0]).  The last range writes
-// b in the field type.
+// FP64 sum (bacc, carried across launches of successive atom ranges).  The last
+// range writes b in the field type.  Bound by the latency of the table reads.
 template <typename T>
 __global__ void __launch_bounds__(512) pseudocharge_gather_kernel(GridDev g, AtomArgs A, int a0, int na, int box,
-                                                                  int bdim, int vdim, int R,
-                                                                  const int* __restrict__ lo,
-                                                                  const double* __restrict__ vbox,
+                                                                  int bdim, int R, const int* __restrict__ lo,
                                                                   const double* __restrict__ bbox, double* bacc,
-                                                                  int first, int last, T* b, double* es_out,
-                                                                  RedBuf red) {
+                                                                  int first, int last, T* b) {
   __shared__ int list[512];
   __shared__ int warp_cnt[16];
-  __shared__ double smem[512 / 32];
   const int x = blockIdx.x * AT + threadIdx.x, y = blockIdx.y * AT + threadIdx.y,
             z = blockIdx.z * AT + threadIdx.z;
   const int tid = threadIdx.x + AT * (threadIdx.y + AT * threadIdx.z);
@@ -2979,69 +3086,114 @@ __global__ void __launch_bounds__(512) pseudocharge_gather_kernel(GridDev g, Ato
   AtomArgs Ar = A;
   Ar.M = a0 + na;  // the list covers this range only
   const int cnt = tile_atoms(Ar, a0, cx, cy, cz, half, A.rc + A.h, list, warp_cnt);
-  const long long bper = (long long)bdim * bdim * bdim, vper = (long long)vdim * vdim * vdim;
-  double es = 0.0;
+  const long long bper = (long long)bdim * bdim * bdim;
+  // the listed atoms' box starts and, for the FP32 screen of the node's distance
+  // (DistScreen), their positions
+  __shared__ int slo[512][3];
+  __shared__ float sfr[512][3];
+  for (int e = tid; e < 3 * cnt; e += 512) {
+    const int t = e / 3, d = e - 3 * t;
+    slo[t][d] = lo[3 * (list[t] - a0) + d];
+    sfr[t][d] = (float)(A.R[3 * list[t] + d] - (d == 0 ? cx : d == 1 ? cy : cz));
+  }
+  __syncthreads();
+  // (relative to the tile's centre, so that wherever the box lies FP32 resolves them)
+  const float fx = (float)(A.ox + (x + 0.5) * A.h - cx), fy = (float)(A.oy + (y + 0.5) * A.h - cy),
+              fz = (float)(A.oz + (z + 0.5) * A.h - cz);
+  const float rc2 = screen_r2(A.rc);
   if (inside) {
     const long long node = lin(g, x, y, z);
     double bsum = first ? 0.0 : bacc[node];
-    for (int t = 0; t < cnt; ++t) {
-      const int a = list[t] - a0;
-      const int ix = x - lo[3 * a], iy = y - lo[3 * a + 1], iz = z - lo[3 * a + 2];
-      if (ix < 0 || iy < 0 || iz < 0 || ix >= box || iy >= box || iz >= box) continue;
-      const double bj = bbox[a * bper + (ix + R) + (long long)bdim * ((iy + R) + (long long)bdim * (iz + R))];
-      if (bj == 0.0) continue;
-      bsum += bj;
-      es += bj * vbox[a * vper + (ix + 2 * R) + (long long)vdim * ((iy + 2 * R) + (long long)vdim * (iz + 2 * R))];
+    // four atoms at a time, so that their table reads are in flight together
+    for (int t0 = 0; t0 < cnt; t0 += 4) {
+      double bj[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int t = min(t0 + k, cnt - 1);
+        const float dx = fx - sfr[t][0], dy = fy - sfr[t][1], dz = fz - sfr[t][2];
+        const int a = list[t] - a0, ix = x - slo[t][0], iy = y - slo[t][1], iz = z - slo[t][2];
+        const bool in = t0 + k < cnt && dx * dx + dy * dy + dz * dz <= rc2 && ix >= 0 && iy >= 0 && iz >= 0 &&
+                        ix < box && iy < box && iz < box;
+        bj[k] = in ? __ldg(bbox + a * bper + (ix + R) + (long long)bdim * ((iy + R) + (long long)bdim * (iz + R))) : 0.0;
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (bj[k] != 0.0) bsum += bj[k];
     }
     if (last)
       b[node] = (T)bsum;
     else
       bacc[node] = bsum;
   }
-  double acc[1] = {es};
-  struct Fin {
-    double* out;
-    __device__ void operator()(double* t) const { out[0] += t[0]; }
-  } fin{es_out};
-  const int nb = gridDim.x * gridDim.y * gridDim.z;
-  const int bid = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
-  grid_sum<1, 512>(acc, smem, red, nb, bid, tid, fin);
 }
 
 // b_J on the atom's box grown by R: -(1/4 pi) L_h V_J inside r_c, 0 outside;
-// one block row per atom (blockIdx.y).
-template <int R>
-__global__ void __launch_bounds__(256) force_bbox_kernel(AtomArgs A, int a0, int vdim, int bdim,
+// one block row per atom (blockIdx.y).  Bound by the FP64 pipe (6 R + 4 operations
+// a node of the ball): 409 atoms at h = 0.5, 12th order, in 469 us, 0.31 ms at the
+// pipe's rate (512 atoms took 1,679 us with a root a node and rows as warps).
+// With ES it also adds the sum of b_J V_J over the grid's nodes to es_out.
+template <int R, bool ES>
+__global__ void __launch_bounds__(256) force_bbox_kernel(GridDev g, AtomArgs A, int a0, int vdim, int bdim,
                                                          const int* __restrict__ lo, Weights<double> W,
-                                                         const double* __restrict__ vbox, double* bbox) {
+                                                         const double* __restrict__ vbox, double* bbox,
+                                                         double* es_out, RedBuf red) {
+  extern __shared__ __align__(16) double atom_sm[];  // squared offsets
+  __shared__ double smem[256 / 32];
+  double es[1] = {0.0};
+  __shared__ unsigned queue[8][64];
   const int a = blockIdx.y;
   const int J = a0 + a;
   const unsigned per = (unsigned)bdim * bdim * bdim;
   const size_t vper = (size_t)vdim * vdim * vdim;
-  const int bx = lo[3 * a] - R, by = lo[3 * a + 1] - R, bz = lo[3 * a + 2] - R;
-  const double Rx = A.R[3 * J], Ry = A.R[3 * J + 1], Rz = A.R[3 * J + 2];
-  const DistScreen sc{(float)node_off(A.ox, bx, A.h, Rx), (float)node_off(A.oy, by, A.h, Ry),
-                      (float)node_off(A.oz, bz, A.h, Rz), (float)A.h, screen_r2(A.rc)};
+  const int bl[3] = {lo[3 * a] - R, lo[3 * a + 1] - R, lo[3 * a + 2] - R};
+  const double Rj[3] = {A.R[3 * J], A.R[3 * J + 1], A.R[3 * J + 2]}, og[3] = {A.ox, A.oy, A.oz};
+  const DistScreen sc{(float)node_off(A.ox, bl[0], A.h, Rj[0]), (float)node_off(A.oy, bl[1], A.h, Rj[1]),
+                      (float)node_off(A.oz, bl[2], A.h, Rj[2]), (float)A.h, screen_r2(A.rc)};
+  box_squares(atom_sm, bdim, bl, Rj, A.h, og);
+  __syncthreads();
   const double* v = vbox + (size_t)a * vper;
   double* out = bbox + (size_t)a * per;
   const long long sy = vdim, sz = (long long)vdim * vdim;
-  for (unsigned e = blockIdx.x * 256 + threadIdx.x; e < per; e += gridDim.x * 256) {
+  constexpr double scale = -1.0 / (4.0 * kPi);
+  auto ijk = [&](unsigned e, int& i, int& j, int& k) {
     const unsigned jk = e / (unsigned)bdim;
-    const int i = (int)(e - jk * (unsigned)bdim);
-    const int k = (int)(jk / (unsigned)bdim);
-    const int j = (int)(jk - (unsigned)k * (unsigned)bdim);
-    double val = 0.0;
-    if (sc.maybe_within(i, j, k) &&
-        dist3(node_off(A.ox, bx + i, A.h, Rx), node_off(A.oy, by + j, A.h, Ry), node_off(A.oz, bz + k, A.h, Rz)) <
-            A.rc) {
-      const long long c = (long long)(i + R) + sy * (j + R) + sz * (k + R);
-      double lap = W.c * v[c];
+    i = (int)(e - jk * (unsigned)bdim);
+    k = (int)(jk / (unsigned)bdim);
+    j = (int)(jk - (unsigned)k * (unsigned)bdim);
+  };
+  warp_compact(blockIdx.x * 256 + (threadIdx.x & ~31u), per, gridDim.x * 256, queue[threadIdx.x >> 5],
+               [&](unsigned e) {
+                 int i, j, k;
+                 ijk(e, i, j, k);
+                 const bool in = sc.maybe_within(i, j, k);
+                 if (!in) out[e] = 0.0;
+                 return in;
+               },
+               [&](unsigned e) {
+                 int i, j, k;
+                 ijk(e, i, j, k);
+                 const double d2 = __dadd_rn(__dadd_rn(atom_sm[i], atom_sm[bdim + j]), atom_sm[2 * bdim + k]);
+                 double val = 0.0;
+                 if (d2 < A.rc2) {
+                   const double* c = v + ((i + R) + sy * (j + R) + sz * (k + R));
+                   double lap = W.c * c[0];
 #pragma unroll
-      for (int p = 1; p <= R; ++p)
-        lap = fma(W.w[p], ((v[c + p] + v[c - p]) + (v[c + p * sy] + v[c - p * sy])) + (v[c + p * sz] + v[c - p * sz]), lap);
-      val = -lap / (4.0 * kPi);
-    }
-    out[e] = val;
+                   for (int p = 1; p <= R; ++p)
+                     lap = fma(W.w[p], ((c[p] + c[-p]) + (c[p * sy] + c[-p * sy])) + (c[p * sz] + c[-p * sz]), lap);
+                   val = lap * scale;
+                   if constexpr (ES) {
+                     const int x = bl[0] + i, y = bl[1] + j, z = bl[2] + k;
+                     if (x >= 0 && y >= 0 && z >= 0 && x < g.n1 && y < g.n2 && z < g.n3) es[0] = fma(val, c[0], es[0]);
+                   }
+                 }
+                 out[e] = val;
+               });
+  if constexpr (ES) {
+    struct Fin {
+      double* out;
+      __device__ void operator()(double* t) const { out[0] += t[0]; }
+    } fin{es_out};
+    grid_sum<1, 256>(es, smem, red, gridDim.x * gridDim.y, blockIdx.y * gridDim.x + blockIdx.x, threadIdx.x, fin);
   }
 }
 
@@ -3056,7 +3208,9 @@ __global__ void __launch_bounds__(256) force_ball_kernel(GridDev g, AtomArgs A, 
                                                          const double* __restrict__ bbox,
                                                          const T* __restrict__ phi, int exact,
                                                          double* partial) {
+  extern __shared__ __align__(16) double atom_sm[];  // coefficients, squared offsets
   __shared__ double smem[3 * (256 / 32)];
+  __shared__ unsigned queue[8][64];
   const int a = blockIdx.y;
   const int J = a0 + a;
   const long long per = (long long)box * box * box;
@@ -3065,21 +3219,32 @@ __global__ void __launch_bounds__(256) force_ball_kernel(GridDev g, AtomArgs A, 
   const DistScreen sc{(float)node_off(A.ox, lo[3 * a], A.h, A.R[3 * J]),
                       (float)node_off(A.oy, lo[3 * a + 1], A.h, A.R[3 * J + 1]),
                       (float)node_off(A.oz, lo[3 * a + 2], A.h, A.R[3 * J + 2]), (float)A.h, screen_r2(A.rc)};
+  const double Rj[3] = {A.R[3 * J], A.R[3 * J + 1], A.R[3 * J + 2]}, og[3] = {A.ox, A.oy, A.oz};
+  double* qd = atom_sm + kGtabN * kGtabC;
+  gtab_load(atom_sm, A.gtab);
+  box_squares(qd, box, lo + 3 * a, Rj, A.h, og);
+  __syncthreads();
+  const double is2 = 1.0 / (A.sigma * A.sigma), zs = -A.Z[J] / A.sigma;
   double acc[3] = {0.0, 0.0, 0.0};
-  for (unsigned t = blockIdx.x * 256 + threadIdx.x; t < (unsigned)per; t += gridDim.x * 256) {
+  auto ijk = [&](unsigned t, int& i, int& j, int& k) {
     const unsigned jk = t / (unsigned)box;
-    const int i = (int)(t - jk * (unsigned)box);
-    const int k = (int)(jk / (unsigned)box);
-    const int j = (int)(jk - (unsigned)k * (unsigned)box);
+    i = (int)(t - jk * (unsigned)box);
+    k = (int)(jk / (unsigned)box);
+    j = (int)(jk - (unsigned)k * (unsigned)box);
+  };
+  auto test = [&](unsigned t) {
+    int i, j, k;
+    ijk(t, i, j, k);
     const int gi = lo[3 * a] + i, gj = lo[3 * a + 1] + j, gk = lo[3 * a + 2] + k;
-    if (gi < 0 || gj < 0 || gk < 0 || gi >= g.n1 || gj >= g.n2 || gk >= g.n3) continue;
-    if (!sc.maybe_within(i, j, k)) continue;
-    const double rx = node_off(A.ox, gi, A.h, A.R[3 * J]);
-    const double ry = node_off(A.oy, gj, A.h, A.R[3 * J + 1]);
-    const double rz = node_off(A.oz, gk, A.h, A.R[3 * J + 2]);
-    const double r = dist3(rx, ry, rz);
-    if (!(r < A.rc)) continue;
-    const double pv = (double)phi[lin(g, gi, gj, gk)] - gauss_v(A.Z[J], inv_s, r);
+    return gi >= 0 && gj >= 0 && gk >= 0 && gi < g.n1 && gj < g.n2 && gk < g.n3 && sc.maybe_within(i, j, k);
+  };
+  auto work = [&](unsigned t) {
+    int i, j, k;
+    ijk(t, i, j, k);
+    const int gi = lo[3 * a] + i, gj = lo[3 * a + 1] + j, gk = lo[3 * a + 2] + k;
+    const double d2 = __dadd_rn(__dadd_rn(qd[i], qd[box + j]), qd[2 * box + k]);
+    if (!(d2 < A.rc2)) return;
+    const double pv = (double)phi[lin(g, gi, gj, gk)] - gtab_v(atom_sm, d2, is2, zs, A.sigma);
     double gx = 0.0, gy = 0.0, gz = 0.0;
     if (!exact) {
       const double* bb = bbox + (long long)a * bper;
@@ -3093,6 +3258,8 @@ __global__ void __launch_bounds__(256) force_ball_kernel(GridDev g, AtomArgs A, 
       }
     } else {
       // -(1/4 pi) L_h grad V_J with grad V analytic: dV/dr = Z erf(r/s)/r^2 - Z (2/(s sqrt pi)) e^{-r^2/s^2}/r
+      const double rx = node_off(A.ox, gi, A.h, Rj[0]), ry = node_off(A.oy, gj, A.h, Rj[1]),
+                   rz = node_off(A.oz, gk, A.h, Rj[2]);
       double lx = 0.0, ly = 0.0, lz = 0.0;
       for (int p = -R; p <= R; ++p) {
         for (int ax = 0; ax < 3; ++ax) {
@@ -3123,7 +3290,9 @@ __global__ void __launch_bounds__(256) force_ball_kernel(GridDev g, AtomArgs A, 
     acc[0] = fma(gx, pv, acc[0]);
     acc[1] = fma(gy, pv, acc[1]);
     acc[2] = fma(gz, pv, acc[2]);
-  }
+  };
+  warp_compact(blockIdx.x * 256 + (threadIdx.x & ~31u), (unsigned)per, gridDim.x * 256, queue[threadIdx.x >> 5], test,
+               work);
   block_sum<3, 256>(acc, smem, threadIdx.x);
   if (threadIdx.x == 0) {
     const long long o = ((long long)a * gridDim.x + blockIdx.x) * 3;

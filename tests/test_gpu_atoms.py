@@ -1,0 +1,68 @@
+"""The atom kernels against the oracle where their tables and queues have edges:
+nuclear widths and radii whose squared arguments cross the interval table's octaves
+and leave it, boxes larger and smaller than the grid, atoms near and outside the
+box's faces, every stencil radius."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import oracle as O
+from paper_1405_6456_gb300 import build as B
+from paper_1405_6456_gb300 import ofdft as F
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    B.build()
+    c = F.Context(0)
+    yield c
+    c.close()
+
+
+def _case(dims, h, seed):
+    g = F.make_grid(*dims, h, tuple(-0.5 * n * h for n in dims))
+    rng = np.random.default_rng(seed)
+    half = 0.5 * h * np.array(dims)
+    R = rng.uniform(-1.0, 1.0, (5, 3)) * half * 0.6
+    R[1] = half - 0.1                      # at a corner
+    R[2] = [half[0] + 1.0, 0.0, 0.2]       # outside the box
+    R[3] = [-half[0] + 0.5 * h, 0.5 * h - half[1], 0.5 * h - half[2]]  # on a node
+    return g, O.make_grid(*dims, h, tuple(g.origin)), R, np.array([3.0, 1.0, 2.0, 3.0, 0.5])
+
+
+# (sigma, rc): the default; a wide nucleus inside one octave; a narrow one whose
+# argument reaches 512 and leaves the table; a ball larger than the grid
+@pytest.mark.parametrize("sigma,rc", [(1.0, 7.0), (2.5, 4.0), (0.25, 5.0), (0.9, 9.5)])
+@pytest.mark.parametrize("dims,h,order", [((26, 21, 33), 0.6, 12), ((19, 24, 17), 0.8, 2), ((22, 30, 20), 0.7, 8)])
+def test_pseudocharge_and_forces_match_oracle(ctx, sigma, rc, dims, h, order):
+    g, og, R, Z = _case(dims, h, order)
+    n = order // 2
+    b = torch.empty(g.shape, dtype=torch.float64, device=DEV)
+    es = ctx.pseudocharge(g, order, R, Z, b, sigma=sigma, rc=rc)
+    b_ref, es_ref = O.pseudocharge(og, n, R, Z, sigma, rc)
+    # b_J is a sum of 6n + 1 values of V / h^2 that cancel: rounding of V's scale
+    scale = np.abs(O.lap_weights(n, h)).sum() * 6.0 * 3.0 * 2.0 / (sigma * np.sqrt(np.pi)) / (4.0 * np.pi)
+    assert np.abs(b.cpu().numpy() - b_ref).max() <= 5 * 4e-16 * scale
+    assert es == pytest.approx(es_ref, rel=1e-12)
+    phi = 0.01 * np.random.default_rng(3).standard_normal(g.shape)
+    for variant in (F.FORCE_PAPER, F.FORCE_EXACT):
+        Fd = ctx.forces(g, order, R, Z, torch.as_tensor(phi, device=DEV), sigma=sigma, rc=rc, variant=variant)
+        Fo = O.forces(og, n, R, Z, phi, sigma=sigma, rc=rc, exact=(variant == F.FORCE_EXACT))
+        np.testing.assert_allclose(Fd, Fo, rtol=1e-10, atol=1e-11 * np.abs(Fo).max())
+
+
+@pytest.mark.parametrize("gs,cut", [(2.0, 8.0), (0.7, 2.3), (5.0, 60.0)])
+@pytest.mark.parametrize("dims,h", [((26, 21, 33), 0.6), ((64, 9, 8), 0.5)])
+def test_initial_guess_matches_oracle(ctx, gs, cut, dims, h):
+    g, og, R, Z = _case(dims, h, 7)
+    u = torch.empty(g.shape, dtype=torch.float64, device=DEV)
+    ctx.initial_guess(g, R, Z, u, guess_sigma=gs, guess_cut=cut)
+    u_ref = O.initial_guess(og, R, Z, gs, cut)
+    # three exponentials multiplied against one of the sum: a few units of 2^-53
+    assert np.abs(u.cpu().numpy() - u_ref).max() <= 1e-14 * np.abs(u_ref).max()
