@@ -787,21 +787,42 @@ int poisson_fp64(ofdft_ctx* c, int R, const GridDev& g, double h, const double* 
   return OFDFT_OK;
 }
 
-// Mixed Poisson solve (S3 + S10): FP32 CG with residual replacement.  The
-// potential phi64 stays FP64; r, p, q = A p and the correction e of the current
-// round are FP32.  Each round folds e into phi64 and computes the FP64 true
-// residual r64 = 4 pi (u^2 + b64) + L_h phi64 with the FP64 stencil; the solve
-// ends when it meets tol.  Otherwise r64 replaces the FP32 residual (plain CG
-// keeps the search direction after the first round, so no Krylov information is
-// lost; preconditioned CG restarts from p = z) and FP32 iterations run until the FP32 residual falls by mixed_inner_tol (1e-4,
-// or less when the FP64 test needs less) or refine_every steps.  At the end
-// phi32 = (float) phi64.  rho32 (optional) replaces u^2 + b.  b2_valid
-// (optional): the caller's flag that V_B2 already holds b64 as float-float
-// pairs (the pseudocharge is fixed for a whole ground state, so a solve splits
-// it once); set here after a split.
+// Where a mixed Poisson solve takes its starting potential and its pseudocharge
+// from, when it does not find them in phi64 and b64: phi32 (FP32 fields of a caller),
+// or phi64 extrapolated along a line search by t (from64 - line0), from64 being
+// another buffer.  b32: the pseudocharge in FP32.
+struct MixedStart {
+  bool fp32 = false;              // phi64 = (double) phi32 on entry
+  const double* from64 = nullptr; // NULL: phi64 itself
+  const double* line0 = nullptr;  // potential at the line search's origin (t != 0)
+  double t = 0.0;
+  const float* b32 = nullptr;
+};
+
+// Mixed Poisson solve (S3 + S10): FP32 corrections of an FP64 potential.  Each round
+// forms the residual 4 pi (u^2 + b) + L_h phi64 in float-float arithmetic (or with
+// the FP64 stencil) and the solve ends when it meets tol.
+//
+// Where the fast diagonalisation covers the grid a round's correction is M r itself
+// (M inverts -L_h up to FP32 rounding, so a CG step's alpha would be 1 up to the
+// same): the residual pass writes r in FP32, and the last of the five passes adds z
+// to phi64 and rewrites the pairs and the FP32 field beside it.  No CG vectors, no
+// scalars but the residual pass's own (192^3, 12th order, from zero to 1e-8: 1,775 us
+// with a CG step in each of the two rounds, 1,241 us so).  A round that does not at least halve the
+// residual (the rounding floor, or an M that is off) hands over to the CG form.
+//
+// Otherwise r, p, q = A p and the correction e of the round are FP32; the FP64
+// residual replaces the FP32 one (plain CG keeps the search direction after the
+// first round, so no Krylov information is lost; preconditioned CG restarts from
+// p = z) and FP32 iterations run until the FP32 residual falls by mixed_inner_tol
+// (1e-4, or less when the FP64 test needs less) or refine_every steps.  At the end
+// phi32 = (float) phi64.  rho32 (optional) replaces u^2 + b.  b2_valid (optional):
+// the caller's flag that V_B2 already holds b64 as float-float pairs (the
+// pseudocharge is fixed for a whole ground state, so a solve splits it once); set
+// here after a split.
 int poisson_mixed(ofdft_ctx* c, int R, const GridDev& g, double h, const float* rho32, const float* u,
                   const double* b64, double* phi64, float* phi32, double tol, int max_it, int refine_every,
-                  ofdft_cg_stats* st, int* b2_valid = nullptr) {
+                  ofdft_cg_stats* st, int* b2_valid = nullptr, const MixedStart& from = MixedStart{}) {
   TRY(ensure_cg_vectors(c, g.G, sizeof(float), true));
   const Weights<double> W = lap_weights(R, h, 1.0), Wneg = lap_weights(R, h, -1.0);
   double* r64 = vec<double>(c, V_R64);
@@ -813,13 +834,13 @@ int poisson_mixed(ofdft_ctx* c, int R, const GridDev& g, double h, const float* 
   int total = 0, rc = OFDFT_OK;
   CgScalars hs, hs32;
   const int max_rounds = 60;
-  CU(cudaMemsetAsync(e32, 0, g.G * sizeof(float), c->stream));
   // float-float residual pass: the potential and the pseudocharge as float-float
-  // pairs (phi2, b2), split once here and phi2 kept in step by every fold; the
-  // residual itself is written as pairs (r2, in the r64 buffer)
+  // pairs (phi2, b2), split once here and phi2 kept in step by every correction
   float2 *phi2 = nullptr, *b2 = nullptr;
   float2* r2 = reinterpret_cast<float2*>(r64);
   c->mixed_ff = c->ff_residual != 0;
+  // (contexts that stage by TMA keep the CG form, whose stencil pass is what they stage)
+  bool direct = mg.fd.on && c->mixed_ff && !c->tma;
   if (c->mixed_ff) {
     TRY(ensure(c, c->v[V_PHI2], g.G * sizeof(float2)));
     phi2 = vec<float2>(c, V_PHI2);
@@ -830,19 +851,44 @@ int poisson_mixed(ofdft_ctx* c, int R, const GridDev& g, double h, const float* 
     const bool split_b = b2 && !(b2_valid && *b2_valid);
     {
       ProfScope ps_(c, OFDFT_K_VECTOR);
-      ff_split_kernel<<<pb, 256, 0, c->stream>>>(g.G, phi2, phi64, split_b ? b2 : nullptr, b64);
+      ff_prepare_kernel<<<pb, 256, 0, c->stream>>>(g.G, from.from64 ? from.from64 : phi64, from.line0, from.t,
+                                                   from.fp32 ? phi32 : nullptr, phi64, phi2,
+                                                   (direct && !from.fp32) ? phi32 : nullptr,
+                                                   split_b ? b2 : nullptr, b64, from.b32);
     }
     CU(cudaGetLastError());
     if (split_b && b2_valid) *b2_valid = 1;
+  } else {
+    if (from.fp32) {
+      ProfScope ps_(c, OFDFT_K_VECTOR);
+      convert_kernel<float, double><<<pb, 256, 0, c->stream>>>(g.G, phi64, phi32);
+    } else if (from.from64) {
+      CU(cudaMemcpyAsync(phi64, from.from64, g.G * sizeof(double), cudaMemcpyDeviceToDevice, c->stream));
+    }
+    if (from.line0) {
+      ProfScope ps_(c, OFDFT_K_VECTOR);
+      extrap_kernel<<<pb, 256, 0, c->stream>>>(g.G, phi64, from.line0, from.t);
+    }
+    CU(cudaGetLastError());
   }
+  if (from.b32 && !rho32) {  // the FP64 copy that the FP64 residual and the functional read
+    if (!c->mixed_ff) {
+      ProfScope ps_(c, OFDFT_K_VECTOR);
+      convert_kernel<float, double><<<pb, 256, 0, c->stream>>>(g.G, const_cast<double*>(b64), from.b32);
+    }
+    CU(cudaGetLastError());
+  }
+  if (!direct) CU(cudaMemsetAsync(e32, 0, g.G * sizeof(float), c->stream));
   const float2 fourpi = ff_of(4.0 * kPi);
+  double rr_old = -1.0;
   for (int round = 0; round <= max_rounds; ++round) {
-    if (round > 0) {
+    if (round > 0 && !direct) {
       ProfScope ps_(c, OFDFT_K_VECTOR);
       fold_kernel<<<pb, 256, 0, c->stream>>>(g.G, phi64, e32, phi2);
     }
     if (c->mixed_ff) {
-      const EpiResidualFF ep{rho32, rho32 ? nullptr : u, b2, r2, c->sc, tol, max_it, 0, fourpi};
+      const EpiResidualFF ep{rho32, rho32 ? nullptr : u, b2, direct ? nullptr : r2, direct ? r32 : nullptr, c->sc, tol,
+                             max_it, 0, fourpi};
       TRY(launch_z_r<float2>(c, R, g, W, LoadPlain<float2>{phi2}, ep, OFDFT_K_RESIDUAL));
     } else {
       const EpiResidual<double, float, double> ep =
@@ -862,6 +908,18 @@ int poisson_mixed(ofdft_ctx* c, int R, const GridDev& g, double h, const float* 
       rc = fail(c, OFDFT_ENOTCONV, "mixed Poisson reached %d FP32 iterations at relative residual %.3e", total,
                 sqrt(hs.rr / bb));
       break;
+    }
+    if (direct) {
+      if (rr_old >= 0.0 && hs.rr > 0.25 * rr_old) {  // not halved: go on with CG (from a residual in pairs)
+        direct = false;
+        CU(cudaMemsetAsync(e32, 0, g.G * sizeof(float), c->stream));
+        continue;
+      }
+      rr_old = hs.rr;
+      if (c->trace) fprintf(stderr, "[ofdft] mixed round %d rel64=%.3e direct\n", round, sqrt(hs.rr / bb));
+      TRY(fd_correction(c, g, mg.fd, r32, c->v[V_T].p, phi64, phi2, phi32));
+      total += 1;
+      continue;
     }
     const int budget = std::min(refine_every, max_it - total);
     TRY(ensure_partials(c, pb, 1));
@@ -889,7 +947,7 @@ int poisson_mixed(ofdft_ctx* c, int R, const GridDev& g, double h, const float* 
               hs32.pc);
     total += std::max(hs32.iters - before, 1);
   }
-  {
+  if (!direct) {
     ProfScope ps_(c, OFDFT_K_VECTOR);
     convert_kernel<double, float><<<pb, 256, 0, c->stream>>>(g.G, phi32, phi64);
   }
@@ -1040,6 +1098,8 @@ struct Solver {
   ofdft_solve_stats* stats;
   ofdft_energy e;  // at the current point
   int trace = 0;   // OFDFT_TRACE=1: one line per evaluation on stderr
+  MixedStart from;          // mixed: where the next Poisson solve starts
+  double pend_gamma = 0.0;  // rank-one correction (with V_W) still to be applied to the last evaluation's s
   int b2_valid = 0;  // mixed: V_B2 holds b64 as float-float pairs (split by the first Poisson solve)
 
   int eval(const T* at, T* Gout, T* sout, const T* dd, const T* s_old, double eta, double mu, ofdft_energy* out) {
@@ -1063,7 +1123,8 @@ struct Solver {
                           &cs);
       else
         rc = poisson_mixed(c, R, g, h, nullptr, (const float*)at, b64, phi64, (float*)phi, tol_p, p->max_cg,
-                           std::max(p->refine_every, 1), &cs, &b2_valid);
+                           std::max(p->refine_every, 1), &cs, &b2_valid, from);
+      from = MixedStart{};
       if (rc != OFDFT_OK) return rc;
       stats->stencil_apps += cs.iterations + 1;
       stats->cg_iters += cs.iterations;
@@ -1091,11 +1152,7 @@ struct Solver {
       // exact inverse of diag + (4 h^3/mu) u u^T (Sherman-Morrison) applied to r = -G
       const double cpen = 4.0 * h * h * h / mu;
       const double gamma = cpen * o.sums[10] / (1.0 + cpen * o.sums[11]);
-      {
-        ProfScope ps_(c, OFDFT_K_VECTOR);
-        rank1_kernel<T><<<pointwise_blocks(c, g.G), 256, 0, c->stream>>>(g.G, sout, winv, gamma);
-      }
-      CU(cudaGetLastError());
+      pend_gamma = gamma;  // applied to sout by nlcg_direction, if sout becomes the current residual
       out->rs_pc -= h * h * h * gamma * o.sums[10];
     }
     out->poisson = cs;
@@ -1107,13 +1164,26 @@ struct Solver {
   // than phi_l alone.  line_start records phi0 at the origin; line_guess(a)
   // rewrites the FP64 potential (phi_l, from the solve at position l) in place.
   double* master() { return mixed ? phi64 : reinterpret_cast<double*>(phi); }
+  // In MIXED nothing is copied or extrapolated here: line_start exchanges the two
+  // buffers, and the next solve's preparing pass (MixedStart) reads the origin's
+  // potential, extrapolates and writes.
   int line_start() {
-    CU(cudaMemcpyAsync(phi0, master(), g.G * sizeof(double), cudaMemcpyDeviceToDevice, c->stream));
     line_l = 0.0;
+    if (mixed) {
+      if (p->terms & OFDFT_TERM_ES) {
+        std::swap(phi64, phi0);
+        from.from64 = phi0;
+      }
+      return OFDFT_OK;
+    }
+    CU(cudaMemcpyAsync(phi0, master(), g.G * sizeof(double), cudaMemcpyDeviceToDevice, c->stream));
     return OFDFT_OK;
   }
   int line_guess(double a) {
-    if (line_l != 0.0 && (p->terms & OFDFT_TERM_ES)) {
+    if (line_l != 0.0 && mixed && (p->terms & OFDFT_TERM_ES)) {
+      from.line0 = phi0;
+      from.t = a / line_l - 1.0;
+    } else if (line_l != 0.0 && (p->terms & OFDFT_TERM_ES)) {
       ProfScope ps_(c, OFDFT_K_VECTOR);
       extrap_kernel<<<pointwise_blocks(c, g.G), 256, 0, c->stream>>>(g.G, master(), phi0, a / line_l - 1.0);
     }
@@ -1152,6 +1222,22 @@ struct Solver {
     return OFDFT_OK;
   }
 
+  // The direction d = s + beta d with the pending correction of s, and G.d and d.d
+  // for the line search (in c->scal + 16; read by nlcg_dots).
+  int nlcg_direction(double beta) {
+    const int pb = pointwise_blocks(c, g.G);
+    TRY(ensure_partials(c, pb, 2));
+    {
+      ProfScope ps_(c, OFDFT_K_VECTOR);
+      nlcg_direction_kernel<T><<<pb, 256, 0, c->stream>>>(g.G, d, s, p->precond_rank1 ? vec<T>(c, V_W) : nullptr, G,
+                                                          pend_gamma, beta, c->scal + 16, red(c));
+    }
+    CU(cudaGetLastError());
+    pend_gamma = 0.0;
+    return OFDFT_OK;
+  }
+  int nlcg_dots(double* r2) { return sync_scalars(c, c->scal + 16, 2 * sizeof(double), r2); }
+
   // Polak-Ribiere nonlinear CG with a secant line search and the Jacobi
   // preconditioner, u <- |u| after every update (Sec. 4), on L(., eta, mu).
   int nlcg(double eta, double mu, int* converged) {
@@ -1159,7 +1245,7 @@ struct Solver {
     const double h3 = h * h * h;
     const double tol_in = p->tol_inner * M;
     TRY(eval(u, G, s, nullptr, nullptr, eta, mu, &e));
-    TRY(direction(0.0));  // d = s
+    TRY(nlcg_direction(0.0));  // d = s
     double delta_new = e.rs_pc;
     int k = 0;
     for (int it = 0; it < p->max_nlcg; ++it) {
@@ -1172,13 +1258,13 @@ struct Solver {
       stats->nlcg_iters++;
       T* s_old = s;
       double gdd[2];
-      TRY(dots(G, d, d, d, gdd));
+      TRY(nlcg_dots(gdd));
       double g0 = h3 * gdd[0];
       double dd = h3 * gdd[1];
       if (!(g0 < 0.0)) {  // not a descent direction: restart along s
-        TRY(direction(0.0));
+        TRY(nlcg_direction(0.0));
         k = 0;
-        TRY(dots(G, d, d, d, gdd));
+        TRY(nlcg_dots(gdd));
         g0 = h3 * gdd[0];
         dd = h3 * gdd[1];
       }
@@ -1238,10 +1324,10 @@ struct Solver {
       if (trace) fprintf(stderr, "[ofdft] nlcg beta=%.6e delta_old=%.6e delta_new=%.6e delta_mid=%.6e\n", beta,
                          delta_old, delta_new, delta_mid);
       if (k >= p->restart_every || !(beta > 0.0) || !std::isfinite(beta)) {
-        TRY(direction(0.0));
+        TRY(nlcg_direction(0.0));
         k = 0;
       } else {
-        TRY(direction(beta));
+        TRY(nlcg_direction(beta));
       }
     }
     if (!*converged && e.rs < tol_in) *converged = 1;
@@ -2253,20 +2339,13 @@ int ofdft_poisson(ofdft_ctx* c, const ofdft_grid* g, int fd_order, int prec, con
   // mixed: FP64 copies of b and phi live in the context for the call
   TRY(ensure(c, c->v[V_PHI64], gd.G * sizeof(double)));
   TRY(ensure(c, c->v[V_B64], gd.G * sizeof(double)));
-  const int pb = pointwise_blocks(c, gd.G);
-  {
-    ProfScope ps_(c, OFDFT_K_VECTOR);
-    convert_kernel<float, double><<<pb, 256, 0, c->stream>>>(gd.G, vec<double>(c, V_PHI64), (const float*)phi);
-  }
-  if (!rho) {
-    ProfScope ps_(c, OFDFT_K_VECTOR);
-    convert_kernel<float, double><<<pb, 256, 0, c->stream>>>(gd.G, vec<double>(c, V_B64), (const float*)b);
-  }
-  CU(cudaGetLastError());
+  MixedStart from;
+  from.fp32 = true;
+  from.b32 = rho ? nullptr : (const float*)b;
   ofdft_params dp;
   ofdft_default_params(&dp);
   const int rc = poisson_mixed(c, fd_order / 2, gd, g->h, (const float*)rho, (const float*)u, vec<double>(c, V_B64),
-                               vec<double>(c, V_PHI64), (float*)phi, tol, max_it, dp.refine_every, st);
+                               vec<double>(c, V_PHI64), (float*)phi, tol, max_it, dp.refine_every, st, nullptr, from);
   TRY(zstream_fault_check(c));
   return rc;
 }
@@ -2299,19 +2378,12 @@ int ofdft_energy_grad(ofdft_ctx* c, const ofdft_grid* g, const ofdft_params* p, 
     } else {
       TRY(ensure(c, c->v[V_PHI64], gd.G * sizeof(double)));
       TRY(ensure(c, c->v[V_B64], gd.G * sizeof(double)));
-      const int pb = pointwise_blocks(c, gd.G);
-      {
-        ProfScope ps_(c, OFDFT_K_VECTOR);
-        convert_kernel<float, double><<<pb, 256, 0, c->stream>>>(gd.G, vec<double>(c, V_PHI64), (const float*)phi);
-      }
-      {
-        ProfScope ps_(c, OFDFT_K_VECTOR);
-        convert_kernel<float, double><<<pb, 256, 0, c->stream>>>(gd.G, vec<double>(c, V_B64), (const float*)b);
-      }
-      CU(cudaGetLastError());
+      MixedStart from;
+      from.fp32 = true;
+      from.b32 = (const float*)b;
       int rc = poisson_mixed(c, R, gd, g->h, nullptr, (const float*)u, vec<double>(c, V_B64), vec<double>(c, V_PHI64),
                              (float*)phi, p->tol_poisson, solve_poisson ? p->max_cg : 0, std::max(p->refine_every, 1),
-                             &cs);
+                             &cs, nullptr, from);
       if (rc != OFDFT_OK && !(rc == OFDFT_ENOTCONV && !solve_poisson)) return rc;
       c->err.clear();
     }

@@ -60,7 +60,10 @@ enum { FD_FWD = 0, FD_INV = 1, FD_SOLVE = 2 };
 struct FdJob {
   FdAxis ax;
   const void* in;   // x forwards: r
-  void* out;        // x backwards: z
+  void* out;        // x backwards: z, or (corrections of a mixed solve) NULL and
+  double* phi64;    // phi64 += z,
+  float2* phi2;     // with its pairs (may be NULL)
+  float* phi32;     // and its FP32 rounding
   float* s;         // scratch, high parts
   float* sl;        // scratch, low parts (float-float)
   long long ncols;
@@ -71,7 +74,7 @@ struct FdJob {
   const float *mx, *my, *mz;     // eigenvalues of h^2 T by axis
   const float *mxl, *myl, *mzl;  // ... low parts
   double ih2;       // 1 / h^2
-  CgScalars* sc;
+  CgScalars* sc;    // the CG this serves (NULL: none; r.z is then not formed)
   RedBuf red;       // z: r.z
   int nblocks;
 };
@@ -313,6 +316,33 @@ __device__ __forceinline__ void fd_store4(float* p, const float (&v)[4]) { *rein
 __device__ __forceinline__ void fd_store4(double* p, const double (&v)[4]) {
   *reinterpret_cast<double2*>(p) = make_double2(v[0], v[1]);
   *(reinterpret_cast<double2*>(p) + 1) = make_double2(v[2], v[3]);
+}
+
+// phi64 += z with the potential's other forms.
+template <typename T>
+__device__ __forceinline__ void fd_correct(const FdJob& J, long long i, T z) {
+  const double v = J.phi64[i] + (sizeof(T) == 4 ? double_of_float((float)z) : (double)z);
+  const float2 p = ff_of_double(v);
+  J.phi64[i] = v;
+  if (J.phi2) J.phi2[i] = p;
+  J.phi32[i] = ff_nearest(p);
+}
+template <typename T>
+__device__ __forceinline__ void fd_correct4(const FdJob& J, long long i, const T (&z)[4]) {
+  double v[4];
+  fd_load4(J.phi64 + i, v);
+  float2 p[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    v[k] += sizeof(T) == 4 ? double_of_float((float)z[k]) : (double)z[k];
+    p[k] = ff_of_double(v[k]);
+  }
+  fd_store4(J.phi64 + i, v);
+  if (J.phi2) {
+    *reinterpret_cast<float4*>(J.phi2 + i) = f4(p[0].x, p[0].y, p[1].x, p[1].y);
+    *reinterpret_cast<float4*>(J.phi2 + i + 2) = f4(p[2].x, p[2].y, p[3].x, p[3].y);
+  }
+  *reinterpret_cast<float4*>(J.phi32 + i) = f4(ff_nearest(p[0]), ff_nearest(p[1]), ff_nearest(p[2]), ff_nearest(p[3]));
 }
 
 // One block's panel of a pass: columns [c0, c0 + TC) of the job.  T is the field
@@ -621,21 +651,23 @@ __device__ __forceinline__ void fd_panel(const FdJob& J, long long c0, int bid, 
     // as the V-cycle's last pass does
     __shared__ double dsm[16];
     __shared__ bool last;
-    const double v = fd_block_sum(dot.value(), dsm, tid, nt);
-    if (tid == 0) {
-      J.red.partials[bid] = v;
-      __threadfence();
-      last = atomicAdd(J.red.counter, 1u) == (unsigned)(J.nblocks - 1);
-    }
-    __syncthreads();
-    if (last) {
-      __threadfence();
-      double s = 0.0;
-      for (int b = tid; b < J.nblocks; b += nt) s += __ldcg(&J.red.partials[b]);
-      s = fd_block_sum(s, dsm, tid, nt);
+    if (J.sc) {
+      const double v = fd_block_sum(dot.value(), dsm, tid, nt);
       if (tid == 0) {
-        MgFin{J.sc}(&s);
-        *J.red.counter = 0u;
+        J.red.partials[bid] = v;
+        __threadfence();
+        last = atomicAdd(J.red.counter, 1u) == (unsigned)(J.nblocks - 1);
+      }
+      __syncthreads();
+      if (last) {
+        __threadfence();
+        double s = 0.0;
+        for (int b = tid; b < J.nblocks; b += nt) s += __ldcg(&J.red.partials[b]);
+        s = fd_block_sum(s, dsm, tid, nt);
+        if (tid == 0) {
+          MgFin{J.sc}(&s);
+          *J.red.counter = 0u;
+        }
       }
     }
   }
@@ -674,14 +706,19 @@ __device__ __forceinline__ void fd_panel(const FdJob& J, long long c0, int bid, 
                          value(e.w, el.w, d.w, dl.w)};
         const T dn[4] = {value(e.w, el.w, -d.w, -dl.w), value(e.z, el.z, -d.z, -dl.z),
                          value(e.y, el.y, -d.y, -dl.y), value(e.x, el.x, -d.x, -dl.x)};
-        T* z = out + (c0 + c) * n;
-        fd_store4(z + x, up);
-        fd_store4(z + n - 4 - x, dn);
+        const long long o = (c0 + c) * n;
+        if (!out) {
+          fd_correct4(J, o + x, up);
+          fd_correct4(J, o + n - 4 - x, dn);
+          continue;
+        }
+        fd_store4(out + o + x, up);
+        fd_store4(out + o + n - 4 - x, dn);
       }
     } else {
       for (int c = warp; c < TC; c += nw) {
         if (c0 + c >= J.ncols) break;
-        T* z = out + (c0 + c) * n;
+        const long long o = (c0 + c) * n;
 #pragma unroll 4
         for (int x = lane; x < n; x += 32) {
           const int i = x < ne ? x : n - 1 - x;
@@ -692,7 +729,11 @@ __device__ __forceinline__ void fd_panel(const FdJob& J, long long c0, int bid, 
             el = pl[c * P + i];
             dl = i < no ? sg * pl[c * P + oo + i] : 0.0f;
           }
-          z[x] = value(ph[c * P + i], el, d, dl);
+          const T v = value(ph[c * P + i], el, d, dl);
+          if (out)
+            out[o + x] = v;
+          else
+            fd_correct(J, o + x, v);
         }
       }
     }
@@ -742,7 +783,7 @@ template <typename T, bool XAX, int MODE, int CT, int TPW>
 __global__ void __maxnreg__(TPW == 1 ? 80 : 128) fd_kernel(const __grid_constant__ FdJob J) {
   pdl_enter();
   extern __shared__ __align__(16) float fd_sm[];
-  if (J.sc->done) return;
+  if (J.sc && J.sc->done) return;
   fd_panel<T, XAX, MODE, CT, TPW>(J, (long long)blockIdx.x * (16 * CT), blockIdx.x, fd_sm);
 }
 
@@ -759,7 +800,7 @@ __global__ void __maxnreg__(TPW == 1 ? 80 : 128)
   extern __shared__ __align__(16) float fd_sm[];
   const FdTile t = tiles[blockIdx.x];
   const FdJob J = jobs[t.job];
-  if (J.sc->done) return;
+  if (J.sc && J.sc->done) return;
   fd_panel<T, XAX, MODE, CT, TPW>(J, (long long)t.panel * (16 * CT), t.panel, fd_sm);
 }
 

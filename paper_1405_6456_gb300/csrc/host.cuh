@@ -763,7 +763,7 @@ int fd_launch(ofdft_ctx* c, FdJob J, int warps) {
     attr_dev[c->device] = true;
   }
   const long long nb = (J.ncols + TC - 1) / TC;
-  if (MODE == FD_SOLVE) {
+  if (MODE == FD_SOLVE && J.sc) {
     TRY(ensure_partials(c, nb, 1));
     J.red = red(c);
     J.nblocks = (int)nb;
@@ -787,15 +787,37 @@ int fd_pass(ofdft_ctx* c, const FdJob& J) {
   return tpw == 1 ? fd_launch<T, XAX, MODE, 2, 1>(c, J, warps) : fd_launch<T, XAX, MODE, 2, 2>(c, J, warps);
 }
 
+// The five passes: z = M r, or (phi64 given) phi64 += M r with its other forms.
+template <typename T>
+int fd_passes(ofdft_ctx* c, const GridDev& g, const FdPlan& P, const T* r, T* z, void* scratch, CgScalars* sc,
+              double* phi64 = nullptr, float2* phi2 = nullptr, float* phi32 = nullptr) {
+  auto job = [&](int p) {
+    FdJob J = fd_job<T>(g, P, p, r, z, scratch, sc);
+    J.phi64 = phi64;
+    J.phi2 = phi2;
+    J.phi32 = phi32;
+    if (phi64 && (((uintptr_t)phi64 | (uintptr_t)phi2 | (uintptr_t)phi32) & 15u)) J.vec = 0;
+    return J;
+  };
+  TRY((fd_pass<T, true, FD_FWD>(c, job(0))));
+  TRY((fd_pass<T, false, FD_FWD>(c, job(1))));
+  TRY((fd_pass<T, false, FD_SOLVE>(c, job(2))));
+  TRY((fd_pass<T, false, FD_INV>(c, job(3))));
+  return fd_pass<T, true, FD_INV>(c, job(4));
+}
+
 // z = M r by fast diagonalisation, with r.z and the PCG scalars as the V-cycle's
 // last pass forms them.  scratch: fd_scratch(g) elements of T.
 template <typename T>
 int fd_apply(ofdft_ctx* c, const GridDev& g, const FdPlan& P, const T* r, T* z, void* scratch, CgScalars* sc) {
-  TRY((fd_pass<T, true, FD_FWD>(c, fd_job<T>(g, P, 0, r, z, scratch, sc))));
-  TRY((fd_pass<T, false, FD_FWD>(c, fd_job<T>(g, P, 1, r, z, scratch, sc))));
-  TRY((fd_pass<T, false, FD_SOLVE>(c, fd_job<T>(g, P, 2, r, z, scratch, sc))));
-  TRY((fd_pass<T, false, FD_INV>(c, fd_job<T>(g, P, 3, r, z, scratch, sc))));
-  return fd_pass<T, true, FD_INV>(c, fd_job<T>(g, P, 4, r, z, scratch, sc));
+  return fd_passes<T>(c, g, P, r, z, scratch, sc);
+}
+
+// One correction of a mixed Poisson solve: phi64 += M r, with its pairs and its FP32
+// rounding, in the last pass.
+inline int fd_correction(ofdft_ctx* c, const GridDev& g, const FdPlan& P, const float* r, void* scratch,
+                         double* phi64, float2* phi2, float* phi32) {
+  return fd_passes<float>(c, g, P, r, nullptr, scratch, nullptr, phi64, phi2, phi32);
 }
 
 template <typename T, int R, int V, class L, class E>

@@ -74,6 +74,32 @@ __device__ __forceinline__ float2 ff_mul_lazy(float2 w, float2 a) {
   return make_float2(p, fmaf(w.x, a.y, fmaf(w.y, a.x, e)));
 }
 
+// A double as a float pair, and a float as a double, on the integer and FP32 pipes:
+// conversions between the two widths issue at the FP64 rate here (1/64 of FP32),
+// and the passes over the FP64 potential did little else.  ff_of_double truncates
+// hi to the double's leading 24 bits and keeps the next 24 of the other 29 in lo
+// (an error below 2^-47 of v); values outside +-[2^-70, 2^127), zero among them,
+// take the plain conversions.
+__device__ __forceinline__ float2 ff_of_double(double v) {
+  const unsigned h = (unsigned)__double2hiint(v), l = (unsigned)__double2loint(v);
+  const unsigned e = (h >> 20) & 0x7ffu;
+  if (e - 953u < 197u) {  // 2^-70 <= |v| < 2^127
+    const unsigned sign = h & 0x80000000u;
+    const float hi = __uint_as_float((((h << 3) | (l >> 29)) ^ 0x40000000u) & 0x7fffffffu | sign);
+    const float sc = __uint_as_float(((e - 948u) << 23) | sign);  // +-2^(e - 1075): the unit of l
+    return make_float2(hi, (float)(l & 0x1fffffffu) * sc);
+  }
+  const float hi = (float)v;
+  return make_float2(hi, isfinite(hi) ? (float)(v - (double)hi) : 0.0f);
+}
+__device__ __forceinline__ double double_of_float(float f) {
+  const unsigned b = __float_as_uint(f), e = (b >> 23) & 0xffu;
+  if (e - 1u < 254u) return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
+  return (double)f;
+}
+// The float nearest a pair's value.
+__device__ __forceinline__ float ff_nearest(float2 a) { return a.x + a.y; }
+
 template <typename T>
 __host__ __device__ __forceinline__ T zero_of() { return T(0); }
 template <>
@@ -1008,7 +1034,8 @@ struct EpiResidualFF {
   const float* rho;  // explicit density, or NULL for u^2 + b
   const float* u;
   const float2* b2;
-  float2* r2;
+  float2* r2;  // the residual as pairs, or
+  float* r1;   // rounded to FP32 (where it only feeds an FP32 correction); the other is NULL
   CgScalars* sc;
   double tol;
   int max_it;
@@ -1030,15 +1057,17 @@ struct EpiResidualFF {
     }
     const float2 rh = ff_mul(fourpi, rr);
     const float2 r = ff_add(rh, lap);
-    r2[i] = r;
+    if (r1)
+      r1[i] = r.x;
+    else
+      r2[i] = r;
     acc[1].add(rh.x, rh.x);
     acc[2].add(r.x, r.x);
+    // the products' low parts are 2^-24 of them: one FMA each into the sums' low parts
     acc[3].add(rr.x, ph.x);
-    acc[3].add(rr.x, ph.y);
-    acc[3].add(rr.y, ph.x);
+    acc[3].lo = fmaf(rr.x, ph.y, fmaf(rr.y, ph.x, acc[3].lo));
     acc[4].add(ph.x, r.x);
-    acc[4].add(ph.x, r.y);
-    acc[4].add(ph.y, r.x);
+    acc[4].lo = fmaf(ph.x, r.y, fmaf(ph.y, r.x, acc[4].lo));
   }
   __device__ __forceinline__ void operator()(double* t) const {
     sc->sum_uu = t[0];
@@ -1060,18 +1089,52 @@ struct EpiResidualFF {
   }
 };
 
-// phi2 = phi64 and b2 = b64 (if b2 is not NULL) split into float-float pairs
-// (hi = nearest float, lo = nearest float of the remainder).
-static __global__ void __launch_bounds__(256) ff_split_kernel(long long G, float2* phi2, const double* phi64,
-                                                              float2* b2, const double* b64) {
-  for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < G; i += (long long)gridDim.x * 256) {
-    const double v = phi64[i];
-    const float hi = (float)v;
-    phi2[i] = make_float2(hi, (float)(v - (double)hi));
-    if (b2) {
-      const double w = b64[i];
-      const float bh = (float)w;
-      b2[i] = make_float2(bh, (float)(w - (double)bh));
+// The potential a mixed Poisson solve starts from, in its three forms: phi64 (from
+// in64, extrapolated along a line search by t (in64 - in0) when in0 is given, or
+// from the FP32 field in32), the pairs phi2 the residual pass reads, and the FP32
+// field out32 (when given).  b2: the pseudocharge as pairs, from b64 or b32 (when
+// given).  One pass where there were a copy, an extrapolation, a split and, at the
+// end of the solve, a conversion (together 53 us at 128^3); bound by HBM (28 to 36
+// bytes a node).
+static __global__ void __launch_bounds__(256) ff_prepare_kernel(long long G, const double* in64, const double* in0,
+                                                                double t, const float* in32, double* phi64,
+                                                                float2* phi2, float* out32, float2* b2,
+                                                                const double* b64, const float* b32) {
+  const long long step = (long long)gridDim.x * 256;
+  const bool write64 = in32 || in0 || phi64 != in64;
+  for (long long i0 = (long long)blockIdx.x * 256 + threadIdx.x; i0 < G; i0 += 4 * step) {
+    double v[4], o[4], bv[4];
+    float f[4], bf[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const long long i = i0 + k * step;
+      v[k] = o[k] = bv[k] = 0.0;
+      f[k] = bf[k] = 0.0f;
+      if (i >= G) continue;
+      if (in32)
+        f[k] = in32[i];
+      else
+        v[k] = in64[i];
+      if (in0) o[k] = in0[i];
+      if (b2 && b32) bf[k] = b32[i];
+      if (b2 && !b32) bv[k] = b64[i];
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const long long i = i0 + k * step;
+      if (i >= G) continue;
+      float2 p;
+      if (in32) {
+        v[k] = double_of_float(f[k]);
+        p = make_float2(f[k], 0.0f);
+      } else {
+        if (in0) v[k] = fma(t, v[k] - o[k], v[k]);
+        p = ff_of_double(v[k]);
+      }
+      if (write64) phi64[i] = v[k];
+      phi2[i] = p;
+      if (out32) out32[i] = ff_nearest(p);
+      if (b2) b2[i] = b32 ? make_float2(bf[k], 0.0f) : ff_of_double(bv[k]);
     }
   }
 }
@@ -2322,6 +2385,57 @@ __global__ void __launch_bounds__(256) axpy_abs_kernel(long long G, T* out, cons
   const T al = (T)alpha;
   for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < G; i += (long long)gridDim.x * 256)
     out[i] = fabs(fma(al, b[i], a[i]));
+}
+
+// The Polak-Ribiere direction of the NLCG with everything that belongs to it in one
+// pass: s -= gamma w (the rank-one correction of the evaluation's preconditioned
+// residual; gamma == 0: none), d = s + beta d (d = s when beta == 0), and
+// out[0] = G.d, out[1] = d.d for the line search.  Three passes before, and the
+// correction was applied to trial points whose residual nobody used (48 us an
+// iteration at 128^3 in FP32); bound by HBM.
+template <typename T>
+__global__ void __launch_bounds__(256) nlcg_direction_kernel(long long G, T* __restrict__ d, T* __restrict__ s,
+                                                             const T* __restrict__ w, const T* __restrict__ gr,
+                                                             double gamma, double beta, double* out, RedBuf red) {
+  __shared__ double smem[2 * (256 / 32)];
+  const T be = (T)beta, ga = (T)gamma;
+  const bool corr = gamma != 0.0, old = beta != 0.0;
+  DotAcc<T> a0, a1;
+  const long long step = (long long)gridDim.x * 256;
+  for (long long i0 = (long long)blockIdx.x * 256 + threadIdx.x; i0 < G; i0 += 4 * step) {
+    T sv[4], wv[4], dv[4], gv[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const long long i = i0 + k * step;
+      if (i >= G) continue;
+      sv[k] = s[i];
+      wv[k] = corr ? w[i] : T(0);
+      dv[k] = old ? d[i] : T(0);
+      gv[k] = gr[i];
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const long long i = i0 + k * step;
+      if (i >= G) continue;
+      if (corr) {
+        sv[k] = fma(-ga, wv[k], sv[k]);
+        s[i] = sv[k];
+      }
+      const T di = old ? fma(be, dv[k], sv[k]) : sv[k];
+      d[i] = di;
+      a0.add(gv[k], di);
+      a1.add(di, di);
+    }
+  }
+  double acc[2] = {a0.value(), a1.value()};
+  struct Fin {
+    double* out;
+    __device__ void operator()(double* t) const {
+      out[0] = t[0];
+      out[1] = t[1];
+    }
+  } fin{out};
+  grid_sum<2, 256>(acc, smem, red, gridDim.x, blockIdx.x, threadIdx.x, fin);
 }
 
 // d = s + beta d (Polak-Ribiere direction), or d = s when beta == 0.
