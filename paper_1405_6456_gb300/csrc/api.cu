@@ -341,7 +341,7 @@ int tune_cg_split(ofdft_ctx* c, int R, const GridDev& g, const Weights<double>& 
   for (auto& t : c->ztuned)
     if (t == tkey) return OFDFT_OK;
   const std::vector<int> cand = {0, 1, 2, 3, 4, 5, 6, 7, 8, 10, 12, 14, 16, 20, 24, 32, 48, 64};
-  TRY(ensure_partials(c, zshape<T>(c, g, R, 1, 64).nblocks, 1));  // largest candidate
+  TRY(ensure_partials(c, zshape<T>(c, g, 1, 64).nblocks, 1));  // largest candidate
   CU(cudaMalloc(&pv, g.G * sizeof(T)));
   if (cudaMalloc(&qv, g.G * sizeof(T)) != cudaSuccess) {
     cudaFree(pv);
@@ -669,8 +669,9 @@ int cg_iterate(ofdft_ctx* c, int R, const GridDev& g, double h, const Weights<do
   }
   const int pb = pointwise_blocks(c, g.G);
   TRY(ensure_partials(c, pb, 1));
-  TRY(ensure_partials(c, zshape<T>(c, g, R, 32).nblocks, 1));
-  TRY(tune_cg_split<T>(c, R, g, Wneg, r, reinterpret_cast<T*>(x)));
+  TRY(ensure_partials(c, zshape<T>(c, g, 1, g.n3).nblocks, 1));
+  // (a directly inverted operator needs a step or two: not worth a tuning run)
+  if (!mg.fd.on) TRY(tune_cg_split<T>(c, R, g, Wneg, r, reinterpret_cast<T*>(x)));
   const bool full_timed = (c->prof & (1 << OFDFT_K_CG_UPDATE)) != 0;
   const bool sampled = !full_timed && (c->prof & (1 << OFDFT_K_CG_DIR_STENCIL)) != 0;
   const int nmg = mg_launches(c, mg);  // V-cycle launches per iteration

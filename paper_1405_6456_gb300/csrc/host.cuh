@@ -13,6 +13,7 @@
 
 #include <algorithm>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/ofdft.h"
@@ -323,10 +324,6 @@ inline int pointwise_blocks(ofdft_ctx* c, long long G) {
   return (int)std::max<long long>(1, std::min<long long>(b, (long long)c->sms * c->pw_per_sm));
 }
 
-// z-streaming launch shape: BX x BY columns; z split so that the grid fills
-// the resident block slots (SMs x blocks per SM) in whole waves: a grid just
-// above a wave would leave a nearly empty second wave.  z-chunks are at least
-// 2R planes deep unless the grid is too small to fill the GPU at all.
 // Poisson tolerance inside a solve's NLCG at a point with h^3 r.s = rs (see
 // ofdft_params.poisson_adapt): the gradient's error from an inexact potential
 // only has to stay small against the gradient itself.
@@ -361,6 +358,7 @@ inline double mixed_inner_tol(double rr, double bb, double tol) {
   return std::max(1e-4, std::min(want, 0.5));
 }
 
+// z-streaming launch shape: tiles of columns times chunks of z planes.
 struct ZShape {
   dim3 grid;
   int zchunk;
@@ -368,19 +366,44 @@ struct ZShape {
 };
 
 template <typename T>
-ZShape zshape(ofdft_ctx* c, const GridDev& g, int R, int blocks_per_sm = 4, int force_nz = 0) {
+ZShape zshape(ofdft_ctx* c, const GridDev& g, int blocks_per_sm = 2, int force_nz = 0) {
   ZShape s;
   const int gx = (g.n1 + BX - 1) / BX, gy = (g.n2 + ZCfg<T>::TY - 1) / ZCfg<T>::TY;
   const long long tiles = (long long)gx * gy;
-  const long long slots = (long long)c->sms * std::max(blocks_per_sm, 1);
-  int nz = (int)std::max<long long>(1, slots / tiles);  // one wave when tiles <= slots
-  nz = std::min(nz, std::max(1, g.n3 / std::max(2 * R, 4)));
-  if (force_nz > 0) nz = std::min(force_nz, g.n3);
-  int zc = (g.n3 + nz - 1) / nz;
-  nz = (g.n3 + zc - 1) / zc;
+  const int per_sm = std::max(blocks_per_sm, 1);
+  int best = 1;
+  if (force_nz > 0) {
+    best = std::min(force_nz, g.n3);
+  } else {
+    // a block's chunk of zc planes costs zc + c0 plane times, k blocks on an SM
+    // slow each other down to 1 + a (k - 1) of that: FP64 passes share a pipe that
+    // one block fills (a = 0.95, c0 = 0.7), FP32 and float-float ones mostly wait
+    // (a = 0.45, c0 = 2.3).  Fitted to sweeps of 1 to 64 chunks on 48^3 to 192^3;
+    // the chosen split is within 4% of the best measured one, where the former rule
+    // (one wave, chunks of at least 2 R planes) lost 10 to 75% below 160^3
+    // (functional, us: FP64 48^3 245 -> 61, 80^3 283 -> 173; FP32 64^3 68 -> 33,
+    // 128^3 92 -> 71) and nothing above.
+    const double a = sizeof(T) == 8 && std::is_same<T, double>::value ? 0.95 : 0.45;
+    const double c0 = std::is_same<T, double>::value ? 0.7 : 2.3;
+    double least = 1e300;
+    for (int zc = g.n3; zc >= 1; --zc) {
+      const int nz = (g.n3 + zc - 1) / zc;
+            const long long blocks = tiles * nz, wave = (long long)c->sms * per_sm;
+      const long long last = blocks % wave;
+      double cost = (double)(blocks / wave) * (1.0 + a * (per_sm - 1));
+      if (last) cost += 1.0 + a * (double)((last + c->sms - 1) / c->sms - 1);
+      cost *= zc + c0;
+      if (cost < least * (1.0 - 1e-9)) {
+        least = cost;
+        best = nz;
+      }
+    }
+  }
+  const int zc = (g.n3 + best - 1) / best;
+  const int nz = (g.n3 + zc - 1) / zc;
   s.grid = dim3(gx, gy, nz);
   s.zchunk = zc;
-  s.nblocks = (long long)gx * gy * nz;
+  s.nblocks = tiles * nz;
   return s;
 }
 
@@ -846,7 +869,7 @@ int launch_zv(ofdft_ctx* c, const GridDev& g, const Weights<double>& W, L ld, E 
       }
   }
   c->last_zkey = key;
-  const ZShape s = zshape<T>(c, g, R, per_sm, nz);
+  const ZShape s = zshape<T>(c, g, per_sm, nz);
   if (E::K > 0) TRY(ensure_partials(c, s.nblocks, E::K));
   {
     ProfScope ps_(c, kind);
@@ -927,7 +950,7 @@ int launch_zv_tma(ofdft_ctx* c, const GridDev& g, const Weights<double>& W, L ld
         }
     }
     c->last_zkey = key;
-    const ZShape s = zshape<T>(c, g, R, per_sm, nz);
+    const ZShape s = zshape<T>(c, g, per_sm, nz);
     if (E::K > 0) TRY(ensure_partials(c, s.nblocks, E::K));
     {
       ProfScope ps_(c, kind);
@@ -967,8 +990,12 @@ int launch_z_r(ofdft_ctx* c, int R, const GridDev& g, const Weights<double>& W, 
 
 
 inline int sync_scalars(ofdft_ctx* c, const void* dev, size_t bytes, void* host) {
-  CU(cudaMemcpyAsync(host, dev, bytes, cudaMemcpyDeviceToHost, c->stream));
+  // through the context's pinned block: a copy to pageable memory is staged by the
+  // driver (5 us more a call)
+  void* to = bytes <= 64 * sizeof(double) ? (void*)c->host_scal : host;
+  CU(cudaMemcpyAsync(to, dev, bytes, cudaMemcpyDeviceToHost, c->stream));
   CU(cudaStreamSynchronize(c->stream));
+  if (to != host) memcpy(host, to, bytes);
   if (!c->pending.empty()) harvest(c);
   return OFDFT_OK;
 }
