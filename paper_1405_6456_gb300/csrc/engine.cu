@@ -103,6 +103,9 @@ struct Slot {
   double ev_tol = 0.0;             // Poisson tolerance of the pending evaluation
   // Poisson phase (within a round)
   int pphase = 0, ptotal = 0;
+  bool direct = false;   // mixed: this solve's corrections are M r themselves (as poisson_mixed)
+  bool fresh32 = false;  // ... and phi already holds phi64's rounding
+  double rr_old = -1.0;
   ofdft_cg_stats pstats;
 };
 
@@ -254,15 +257,14 @@ void grid_tiles(const GridDev& g, int slot, int rows, int zc, std::vector<ZTile>
   *count = bid;
 }
 
-void grid_segs(const GridDev& g, int slot, std::vector<PSeg>& out, int* count) {
-  const long long L = 16384;
-  int bid = 0;
-  for (long long b = 0; b < g.G; b += L) out.push_back(PSeg{slot, bid++, b, std::min(b + L, g.G)});
-  *count = bid;
-}
+// Elements of a segment of a pointwise pass over n elements: 2,048 (eight a thread)
+// up to 4 M elements, 16,384 beyond, where the GPU is full anyway and the work lists
+// would grow.  (With 16,384 throughout, six grids of 48^3 to 80^3 made 64 blocks and
+// each of their passes took 20 to 50 us.)
+long long seg_len(long long n) { return n <= (4LL << 20) ? 2048 : 16384; }
 
 void count_segs(long long n, int slot, std::vector<PSeg>& out, int* count) {
-  const long long L = 16384;
+  const long long L = seg_len(n);
   int bid = 0;
   for (long long b = 0; b < n; b += L) out.push_back(PSeg{slot, bid++, b, std::min(b + L, n)});
   *count = bid;
@@ -374,9 +376,7 @@ struct Engine {
     for (Slot<T>* S : slots) {
       int cnt = 0;
       const int si = (int)ops.size();
-      std::vector<PSeg> tmp;
-      grid_segs(S->g, si, tmp, &cnt);
-      segs.insert(segs.end(), tmp.begin(), tmp.end());
+      count_segs(S->g.G, si, segs, &cnt);
       ops.push_back(make(S, cnt));
     }
     if (segs.empty()) return OFDFT_OK;
@@ -416,8 +416,9 @@ struct Engine {
 
   // One pass of the fast diagonalisation over the grids of `v`: a launch for the
   // grids with one tile of outputs a warp on this axis, and one for those with two.
+  // `correct`: the passes of a direct correction (phi64 += M r64), not of z = M r.
   template <bool XAX, int MODE, class GetR, class GetSc>
-  int fd_pass_batch(const std::vector<Slot<T>*>& v, int pass, GetR getr, GetSc getsc) {
+  int fd_pass_batch(const std::vector<Slot<T>*>& v, int pass, GetR getr, GetSc getsc, bool correct = false) {
     constexpr int CT = sizeof(T) == 4 ? 4 : 2;
     for (int tpw = 1; tpw <= 2; ++tpw) {
       std::vector<FdTile> tiles;
@@ -425,6 +426,13 @@ struct Engine {
       size_t smem = 0;
       for (Slot<T>* S : v) {
         FdJob J = fd_job<T>(S->g, S->mg.fd, pass, getr(S), S->mz, S->mt, getsc(S));
+        if (correct) {
+          J.in64 = S->r64;
+          J.out = nullptr;
+          J.phi64 = S->phi64;
+          J.phi32 = (float*)S->phi;
+          J.sc = nullptr;
+        }
         if ((J.ax.pe + J.ax.po) / kFdTile > kFdBatchWarps ? tpw == 1 : tpw == 2) continue;
         J.red = slot_red(S);
         J.nblocks = (int)((J.ncols + 16 * CT - 1) / (16 * CT));
@@ -455,6 +463,17 @@ struct Engine {
       CU(cudaGetLastError());
     }
     return OFDFT_OK;
+  }
+
+  // phi64 += M r64, with its FP32 rounding, for slots on the fast diagonalisation.
+  int fd_correction_batch(const std::vector<Slot<T>*>& v) {
+    auto getr = [](Slot<T>* S) -> const T* { return S->r; };
+    auto getsc = [&](Slot<T>* S) { return B->sc + S->index; };
+    TRY((fd_pass_batch<true, FD_FWD>(v, 0, getr, getsc, true)));
+    TRY((fd_pass_batch<false, FD_FWD>(v, 1, getr, getsc, true)));
+    TRY((fd_pass_batch<false, FD_SOLVE>(v, 2, getr, getsc, true)));
+    TRY((fd_pass_batch<false, FD_INV>(v, 3, getr, getsc, true)));
+    return fd_pass_batch<true, FD_INV>(v, 4, getr, getsc, true);
   }
 
   // z = M r for every preconditioned slot: by fast diagonalisation, or one V-cycle
@@ -711,7 +730,8 @@ struct Engine {
         return OFDFT_OK;
       }
     // the graph's own arena for the work lists its launches read
-    const size_t arena = (size_t)16 << 20;
+    size_t arena = (size_t)16 << 20;
+    for (Slot<T>* S : slots) arena += 8 * sizeof(PSeg) * (size_t)(S->g.G / seg_len(S->g.G) + 32);
     void* dev = nullptr;
     CU(cudaMalloc(&dev, arena));
     cudaGraph_t graph = nullptr;
@@ -896,16 +916,21 @@ struct Engine {
       }
       return OFDFT_OK;
     }
-    // mixed: FP32 CG with residual replacement (per slot), as poisson_mixed
+    // mixed, as poisson_mixed: direct corrections for the slots on the fast
+    // diagonalisation, FP32 CG with residual replacement for the others
+    if (c->autotune && c->use_graphs && c->cond_graphs)
+      TRY(tune_zdepth(ev, [](Slot<T>* S) -> const T* { return S->r; }));
     for (Slot<T>* S : ev) {
       S->ptotal = 0;
       S->pphase = 1;  // 1: the next replacement restarts the FP32 CG
+      S->direct = S->pc && S->mg.fd.on;
+      S->fresh32 = false;
+      S->rr_old = -1.0;
+      if (!S->direct) CU(cudaMemsetAsync(S->e32, 0, S->g.G * sizeof(float), c->stream));
     }
-    std::vector<Slot<T>*> resid = ev;
-    for (Slot<T>* S : ev) CU(cudaMemsetAsync(S->e32, 0, S->g.G * sizeof(float), c->stream));
+    std::vector<Slot<T>*> resid = ev, fold;  // fold: slots with a CG correction to add
     for (int round = 0; round <= 60 && !resid.empty(); ++round) {
-      if (round > 0)
-        TRY((ppass<OpFold>(resid, OFDFT_K_VECTOR, [&](Slot<T>* S, int) { return OpFold{S->phi64, S->e32}; })));
+      TRY((ppass<OpFold>(fold, OFDFT_K_VECTOR, [&](Slot<T>* S, int) { return OpFold{S->phi64, S->e32}; })));
       TRY((zpass<double, LoadPlain<double>, EpiResidual<double, float, double>>(
           resid, OFDFT_K_RESIDUAL, 1.0, [&](Slot<T>* S) {
             return std::make_pair(LoadPlain<double>{S->phi64},
@@ -914,16 +939,30 @@ struct Engine {
                                                                      1});
           })));
       TRY(read_scalars());
-      std::vector<Slot<T>*> corr;
+      std::vector<Slot<T>*> dir, corr, next;
       for (Slot<T>* S : resid) {
         const CgScalars& h = B->h_sc[S->index];
         const double bb = h.bb > 0 ? h.bb : 1.0;
         S->pstats.iterations = S->ptotal;
         S->pstats.rel_residual = sqrt(h.rr / bb);
         if (h.rr <= S->ev_tol * S->ev_tol * bb || S->ptotal >= S->p.max_cg || !isfinite(h.rr)) continue;
-        corr.push_back(S);
+        next.push_back(S);
+        if (S->direct && S->rr_old >= 0.0 && h.rr > 0.25 * S->rr_old) {  // not halved: go on with CG
+          S->direct = S->fresh32 = false;
+          CU(cudaMemsetAsync(S->e32, 0, S->g.G * sizeof(float), c->stream));
+        }
+        S->rr_old = h.rr;
+        (S->direct ? dir : corr).push_back(S);
       }
-      if (corr.empty()) break;
+      resid.swap(next);
+      if (resid.empty()) break;
+      TRY(fd_correction_batch(dir));
+      for (Slot<T>* S : dir) {
+        S->ptotal += 1;
+        S->fresh32 = true;
+      }
+      fold = corr;
+      if (corr.empty()) continue;
       TRY((ppass<OpRefineReplace>(corr, OFDFT_K_VECTOR, [&](Slot<T>* S, int nb) {
         const int budget = std::min(std::max(S->p.refine_every, 1), S->p.max_cg - S->ptotal);
         const CgScalars& h = B->h_sc[S->index];
@@ -940,15 +979,21 @@ struct Engine {
         before[S->index] = B->h_sc32[S->index].iters;
         if (!B->h_sc32[S->index].done) run.push_back(S);
       }
+      // the loop's graph is captured for the round's CG slots (see cg_loop)
+      std::vector<Slot<T>*> set;
+      for (Slot<T>* S : ev)
+        if (!S->direct) set.push_back(S);
       TRY(cg_loop(
-          run, ev, [](Slot<T>* S) { return (T*)S->e32; }, [](Slot<T>* S) { return S->r; },
+          run, set, [](Slot<T>* S) { return (T*)S->e32; }, [](Slot<T>* S) { return S->r; },
           [&](Slot<T>* S) { return B->sc32 + S->index; },
           [&](Slot<T>* S) -> CgScalars& { return B->h_sc32[S->index]; }));
       for (Slot<T>* S : corr) S->ptotal += std::max(B->h_sc32[S->index].iters - before[S->index], 1);
-      resid.swap(corr);
     }
     // FP32 potential (the gradient and the forces take it)
-    TRY((ppass<OpConvert<double, float>>(ev, OFDFT_K_VECTOR, [&](Slot<T>* S, int) {
+    std::vector<Slot<T>*> conv;
+    for (Slot<T>* S : ev)
+      if (!S->fresh32) conv.push_back(S);
+    TRY((ppass<OpConvert<double, float>>(conv, OFDFT_K_VECTOR, [&](Slot<T>* S, int) {
       return OpConvert<double, float>{(float*)S->phi, S->phi64};
     })));
     return OFDFT_OK;

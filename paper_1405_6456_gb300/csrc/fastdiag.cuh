@@ -59,7 +59,8 @@ enum { FD_FWD = 0, FD_INV = 1, FD_SOLVE = 2 };
 // is a row of n contiguous nodes.
 struct FdJob {
   FdAxis ax;
-  const void* in;   // x forwards: r
+  const void* in;   // x forwards: r,
+  const double* in64;  // or in FP64 for an FP32 transform (in is then not read)
   void* out;        // x backwards: z, or (corrections of a mixed solve) NULL and
   double* phi64;    // phi64 += z,
   float2* phi2;     // with its pairs (may be NULL)
@@ -380,8 +381,19 @@ __device__ __forceinline__ void fd_panel(const FdJob& J, long long c0, int bid, 
         const long long row = c0 + c;
         T a[4] = {T(0), T(0), T(0), T(0)}, b[4] = {T(0), T(0), T(0), T(0)};
         if (row < J.ncols) {
-          fd_load4(src + row * n + x, a);
-          fd_load4(src + row * n + n - 4 - x, b);
+          if (sizeof(T) == 4 && J.in64) {
+            double a8[4], b8[4];
+            fd_load4(J.in64 + row * n + x, a8);
+            fd_load4(J.in64 + row * n + n - 4 - x, b8);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              a[k] = (T)ff_nearest(ff_of_double(a8[k]));
+              b[k] = (T)ff_nearest(ff_of_double(b8[k]));
+            }
+          } else {
+            fd_load4(src + row * n + x, a);
+            fd_load4(src + row * n + n - 4 - x, b);
+          }
         }
         float2 s[4], d[4];
 #pragma unroll
@@ -406,12 +418,16 @@ __device__ __forceinline__ void fd_panel(const FdJob& J, long long c0, int bid, 
       for (int c = warp; c < TC; c += nw) {
         const long long row = c0 + c;
         const bool ok = row < J.ncols;
-        const T* f = src + (ok ? row : 0) * n;
+        const long long o = (ok ? row : 0) * n;
+        auto at = [&](int x) -> T {
+          if (sizeof(T) == 4 && J.in64) return (T)ff_nearest(ff_of_double(J.in64[o + x]));
+          return src[o + x];
+        };
 #pragma unroll 4
         for (int x = lane; x < oo; x += 32) {
           T a = T(0), b = T(0);
-          if (ok && x < ne) a = f[x];
-          if (ok && x < no) b = f[n - 1 - x];
+          if (ok && x < ne) a = at(x);
+          if (ok && x < no) b = at(n - 1 - x);
           float2 s, d;
           if constexpr (FF) {
             const float2 fa = fd_ff_of(a), fb = fd_ff_of(b);
