@@ -852,7 +852,8 @@ int poisson_mixed(ofdft_ctx* c, int R, const GridDev& g, double h, const float* 
     const bool split_b = b2 && !(b2_valid && *b2_valid);
     {
       ProfScope ps_(c, OFDFT_K_VECTOR);
-      ff_prepare_kernel<<<pb, 256, 0, c->stream>>>(g.G, from.from64 ? from.from64 : phi64, from.line0, from.t,
+      const int nb = (int)std::min<long long>((g.G + 1023) / 1024, 8LL * c->sms);
+      ff_prepare_kernel<<<nb, 256, 0, c->stream>>>(g.G, from.from64 ? from.from64 : phi64, from.line0, from.t,
                                                    from.fp32 ? phi32 : nullptr, phi64, phi2,
                                                    (direct && !from.fp32) ? phi32 : nullptr,
                                                    split_b ? b2 : nullptr, b64, from.b32);

@@ -103,6 +103,9 @@ struct Slot {
   double ev_tol = 0.0;             // Poisson tolerance of the pending evaluation
   // Poisson phase (within a round)
   int pphase = 0, ptotal = 0;
+  // mixed on the fast diagonalisation: the residual in float-float arithmetic, as
+  // ofdft_solve's; b64 then holds the pseudocharge as pairs and r64 the potential's
+  bool ff = false;
   bool direct = false;   // mixed: this solve's corrections are M r themselves (as poisson_mixed)
   bool fresh32 = false;  // ... and phi already holds phi64's rounding
   double rr_old = -1.0;
@@ -300,6 +303,24 @@ struct Engine {
     return OFDFT_OK;
   }
 
+  // Two work lists of one launch in a single copy (ordinary launches).
+  std::vector<char> both;
+  template <typename V1, typename V2>
+  int put2(const std::vector<V1>& v1, const std::vector<V2>& v2, const void** p1, const void** p2) {
+    if (B->capturing) {
+      TRY(put(B->d_tiles, v1, p1));
+      return put(B->d_desc, v2, p2);
+    }
+    const size_t b1 = v1.size() * sizeof(V1), off = (b1 + 255) & ~(size_t)255, b2 = v2.size() * sizeof(V2);
+    both.resize(off + b2);
+    memcpy(both.data(), v1.data(), b1);
+    memcpy(both.data() + off, v2.data(), b2);
+    TRY(upload(c, B->d_tiles, both));
+    *p1 = B->d_tiles.p;
+    *p2 = (const char*)B->d_tiles.p + off;
+    return OFDFT_OK;
+  }
+
   template <typename TT, int R, int V, class L, class E>
   int launch_zb(int kind, unsigned nb, const ZTile* dt, const ZSlot<TT, L, E>* ds) {
     constexpr int smem = zsmem_bytes<TT, R, V, E>();
@@ -346,8 +367,7 @@ struct Engine {
         }
         if (tiles.empty()) continue;
         const void *pt = nullptr, *pd = nullptr;
-        TRY(put(B->d_tiles, tiles, &pt));
-        TRY(put(B->d_desc, desc, &pd));
+        TRY(put2(tiles, desc, &pt, &pd));
         const ZTile* dt = (const ZTile*)pt;
         const ZSlot<TT, L, E>* ds = (const ZSlot<TT, L, E>*)pd;
         const unsigned nb = (unsigned)tiles.size();
@@ -381,8 +401,7 @@ struct Engine {
     }
     if (segs.empty()) return OFDFT_OK;
     const void *ps = nullptr, *po = nullptr;
-    TRY(put(B->d_segs, segs, &ps));
-    TRY(put(B->d_ops, ops, &po));
+    TRY(put2(segs, ops, &ps, &po));
     {
       ProfScope ps_(c, kind);
       pbatch_kernel<Op><<<(unsigned)segs.size(), 256, 0, c->stream>>>((const PSeg*)ps, (const Op*)po);
@@ -404,8 +423,7 @@ struct Engine {
     }
     if (segs.empty()) return OFDFT_OK;
     const void *ps = nullptr, *po = nullptr;
-    TRY(put(B->d_segs, segs, &ps));
-    TRY(put(B->d_ops, ops, &po));
+    TRY(put2(segs, ops, &ps, &po));
     {
       ProfScope ps_(c, kind);
       pbatch_kernel<Op><<<(unsigned)segs.size(), 256, 0, c->stream>>>((const PSeg*)ps, (const Op*)po);
@@ -416,7 +434,7 @@ struct Engine {
 
   // One pass of the fast diagonalisation over the grids of `v`: a launch for the
   // grids with one tile of outputs a warp on this axis, and one for those with two.
-  // `correct`: the passes of a direct correction (phi64 += M r64), not of z = M r.
+  // `correct`: the passes of a direct correction (phi64 += M r), not of z = M r.
   template <bool XAX, int MODE, class GetR, class GetSc>
   int fd_pass_batch(const std::vector<Slot<T>*>& v, int pass, GetR getr, GetSc getsc, bool correct = false) {
     constexpr int CT = sizeof(T) == 4 ? 4 : 2;
@@ -427,9 +445,9 @@ struct Engine {
       for (Slot<T>* S : v) {
         FdJob J = fd_job<T>(S->g, S->mg.fd, pass, getr(S), S->mz, S->mt, getsc(S));
         if (correct) {
-          J.in64 = S->r64;
           J.out = nullptr;
           J.phi64 = S->phi64;
+          J.phi2 = S->ff ? (float2*)S->r64 : nullptr;
           J.phi32 = (float*)S->phi;
           J.sc = nullptr;
         }
@@ -443,8 +461,7 @@ struct Engine {
       if (tiles.empty()) continue;
       smem += (size_t)kFdBatchWarps * fd_ring_floats<sizeof(T) == 8>() * sizeof(float);
       const void *pt = nullptr, *pj = nullptr;
-      TRY(put(B->d_tiles, tiles, &pt));
-      TRY(put(B->d_ops, jobs, &pj));
+      TRY(put2(tiles, jobs, &pt, &pj));
       static bool attr_dev[64] = {false};  // per instantiation and device
       if (c->device < 0 || c->device >= 64) return fail(c, OFDFT_EINVAL, "device index out of range");
       if (!attr_dev[c->device]) {
@@ -465,7 +482,8 @@ struct Engine {
     return OFDFT_OK;
   }
 
-  // phi64 += M r64, with its FP32 rounding, for slots on the fast diagonalisation.
+  // phi64 += M r (the FP64 residual's FP32 rounding), for slots on the fast
+  // diagonalisation.
   int fd_correction_batch(const std::vector<Slot<T>*>& v) {
     auto getr = [](Slot<T>* S) -> const T* { return S->r; };
     auto getsc = [&](Slot<T>* S) { return B->sc + S->index; };
@@ -928,15 +946,32 @@ struct Engine {
       S->rr_old = -1.0;
       if (!S->direct) CU(cudaMemsetAsync(S->e32, 0, S->g.G * sizeof(float), c->stream));
     }
+    std::vector<Slot<T>*> ffs;
+    for (Slot<T>* S : ev)
+      if (S->ff) {
+        ffs.push_back(S);
+        S->fresh32 = true;
+      }
+    TRY((ppass<OpPairs>(ffs, OFDFT_K_VECTOR, [&](Slot<T>* S, int) {
+      return OpPairs{S->phi64, (float2*)S->r64, (float*)S->phi};
+    })));
     std::vector<Slot<T>*> resid = ev, fold;  // fold: slots with a CG correction to add
     for (int round = 0; round <= 60 && !resid.empty(); ++round) {
       TRY((ppass<OpFold>(fold, OFDFT_K_VECTOR, [&](Slot<T>* S, int) { return OpFold{S->phi64, S->e32}; })));
+      std::vector<Slot<T>*> rff, r64s;
+      for (Slot<T>* S : resid) (S->ff ? rff : r64s).push_back(S);
+      TRY((zpass<float2, LoadPlain<float2>, EpiResidualFF>(rff, OFDFT_K_RESIDUAL, 1.0, [&](Slot<T>* S) {
+        return std::make_pair(LoadPlain<float2>{(const float2*)S->r64},
+                              EpiResidualFF{nullptr, (const float*)S->ev_at, (const float2*)S->b64, nullptr,
+                                            (float*)S->r, B->sc + S->index, S->ev_tol, S->p.max_cg, 0,
+                                            ff_of(4.0 * kPi)});
+      })));
       TRY((zpass<double, LoadPlain<double>, EpiResidual<double, float, double>>(
-          resid, OFDFT_K_RESIDUAL, 1.0, [&](Slot<T>* S) {
+          r64s, OFDFT_K_RESIDUAL, 1.0, [&](Slot<T>* S) {
             return std::make_pair(LoadPlain<double>{S->phi64},
                                   EpiResidual<double, float, double>{nullptr, (const float*)S->ev_at, S->b64, S->r64,
                                                                      B->sc + S->index, S->ev_tol, S->p.max_cg,
-                                                                     1});
+                                                                     1, 0, S->direct ? (float*)S->r : nullptr});
           })));
       TRY(read_scalars());
       std::vector<Slot<T>*> dir, corr, next;
@@ -946,8 +981,10 @@ struct Engine {
         S->pstats.iterations = S->ptotal;
         S->pstats.rel_residual = sqrt(h.rr / bb);
         if (h.rr <= S->ev_tol * S->ev_tol * bb || S->ptotal >= S->p.max_cg || !isfinite(h.rr)) continue;
+        const bool stalled = S->direct && S->rr_old >= 0.0 && h.rr > 0.25 * S->rr_old;
+        if (stalled && S->ff) continue;  // the rounding floor of the residual itself
         next.push_back(S);
-        if (S->direct && S->rr_old >= 0.0 && h.rr > 0.25 * S->rr_old) {  // not halved: go on with CG
+        if (stalled) {  // not halved: go on with CG
           S->direct = S->fresh32 = false;
           CU(cudaMemsetAsync(S->e32, 0, S->g.G * sizeof(float), c->stream));
         }
@@ -1017,7 +1054,9 @@ struct Engine {
       EpiFunctional<T> ep{es ? S->phi : nullptr, S->b, (es && !mixed) ? S->r : nullptr, S->ev_d, S->ev_sold,
                           S->ev_G, S->ev_s, (S->p.precond_rank1 && S->ev_s) ? S->w : nullptr,
                           &B->sc[S->index].sum_uu, f, B->out + 16 * S->index};
-      if (es && mixed) {  // FP64 potential, pseudocharge and residual (as the single-solve path)
+      if (es && mixed && S->ff) {
+        ep.es_sums = B->sc + S->index;  // from the residual pass
+      } else if (es && mixed) {  // FP64 potential, pseudocharge and residual (as the single-solve path)
         ep.phi64 = S->phi64;
         ep.b64 = S->b64;
         ep.r64 = S->r64;
@@ -1366,6 +1405,11 @@ struct Engine {
       TRY((ppass<OpConvert<double, float>>(one, OFDFT_K_VECTOR, [&](Slot<T>* X, int) {
         return OpConvert<double, float>{(float*)X->b, X->b64};
       })));
+      S->ff = S->pc && S->mg.fd.on && c->ff_residual;
+      if (S->ff)
+        TRY((ppass<OpPairs>(one, OFDFT_K_VECTOR, [&](Slot<T>* X, int) {
+          return OpPairs{X->b64, (float2*)X->b64, nullptr};
+        })));
       CU(cudaMemsetAsync(S->phi64, 0, S->g.G * sizeof(double), c->stream));
     }
     TRY(device_guess<T>(c, gr, S->R.data(), S->Z.data(), S->M, S->p.guess_sigma, S->p.guess_cut, S->N, S->u));

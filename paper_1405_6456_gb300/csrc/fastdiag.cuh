@@ -59,8 +59,7 @@ enum { FD_FWD = 0, FD_INV = 1, FD_SOLVE = 2 };
 // is a row of n contiguous nodes.
 struct FdJob {
   FdAxis ax;
-  const void* in;   // x forwards: r,
-  const double* in64;  // or in FP64 for an FP32 transform (in is then not read)
+  const void* in;   // x forwards: r
   void* out;        // x backwards: z, or (corrections of a mixed solve) NULL and
   double* phi64;    // phi64 += z,
   float2* phi2;     // with its pairs (may be NULL)
@@ -107,21 +106,25 @@ template <>
 struct FdAcc<false> {
   float2 h;
   __device__ __forceinline__ void zero() { h = make_float2(0.0f, 0.0f); }
-  __device__ __forceinline__ void add(float2 w, float2, float2 f, float2) { h = __ffma2_rn(w, f, h); }
+  __device__ __forceinline__ void add(float2 w, float2, float2 f, float2, float2) { h = __ffma2_rn(w, f, h); }
   __device__ __forceinline__ void finish() {}
 };
 template <>
 struct FdAcc<true> {
   float2 h, l;
   __device__ __forceinline__ void zero() { h = l = make_float2(0.0f, 0.0f); }
-  __device__ __forceinline__ void add(float2 w, float2 wl, float2 f, float2 fl) {
-    const float2 p = __fmul2_rn(w, f);
-    const float2 e = __ffma2_rn(w, f, fd_neg(p));  // exact rounding error of the product
-    const float2 s = __fadd2_rn(h, p);             // TwoSum
-    const float2 b = fd_sub(s, h);
-    const float2 t = __fadd2_rn(fd_sub(h, fd_sub(s, b)), fd_sub(p, b));
+  // (the packed instructions have no operand signs: a difference a - b is the FMA
+  // b (-1) + a, and the product enters with its sign turned through f, nf = -f)
+  __device__ __forceinline__ void add(float2 w, float2 wl, float2 f, float2 fl, float2 nf) {
+    const float2 m1 = make_float2(-1.0f, -1.0f);
+    const float2 np = __fmul2_rn(w, nf);        // -p
+    const float2 e = __ffma2_rn(w, f, np);      // exact rounding error of the product
+    const float2 s = __ffma2_rn(np, m1, h);     // TwoSum(h, p)
+    const float2 b = __ffma2_rn(h, m1, s);
+    const float2 t = __ffma2_rn(__ffma2_rn(b, m1, s), m1, h);
+    const float2 u = __ffma2_rn(__fadd2_rn(np, b), m1, t);
     h = s;
-    l = __fadd2_rn(l, __fadd2_rn(t, e));
+    l = __fadd2_rn(l, __fadd2_rn(u, e));
     l = __ffma2_rn(w, fl, l);
     l = __ffma2_rn(wl, f, l);
   }
@@ -195,10 +198,10 @@ __device__ __forceinline__ void fd_contract(FdAcc<FF> (&acc)[4][CT], const FdRin
 #pragma unroll
     for (int c = 0; c < CT; ++c) {
       const float2 fv = make_float2(f[c], f[c]);
-      float2 flv = make_float2(0.0f, 0.0f);
-      if constexpr (FF) flv = make_float2(fl[c], fl[c]);
+      float2 flv = make_float2(0.0f, 0.0f), nfv = flv;
+      if constexpr (FF) flv = make_float2(fl[c], fl[c]), nfv = make_float2(-f[c], -f[c]);
 #pragma unroll
-      for (int q = 0; q < 4; ++q) acc[q][c].add(wv[q], wlv[q], fv, flv);
+      for (int q = 0; q < 4; ++q) acc[q][c].add(wv[q], wlv[q], fv, flv, nfv);
     }
   };
   auto node = [&](const float* wr, int i) {  // node-major
@@ -277,10 +280,6 @@ __device__ __forceinline__ float2 fd_ff_add(float2 a, float2 b) {
   const float2 s = ff_two_sum(a.x, b.x);
   return ff_fast_two_sum(s.x, s.y + (a.y + b.y));
 }
-__device__ __forceinline__ float2 fd_ff_of(double v) {
-  const float h = (float)v;
-  return make_float2(h, (float)(v - (double)h));
-}
 // 1 / d for a positive pair: one Newton step from the FP32 reciprocal, the
 // residual 1 - d y formed exactly
 __device__ __forceinline__ float2 fd_ff_rcp(float2 d) {
@@ -304,22 +303,26 @@ __host__ __device__ __forceinline__ int fd_panel_floats(const FdAxis& ax, bool x
 
 __device__ __forceinline__ float4 f4(float a, float b, float c, float d) { return make_float4(a, b, c, d); }
 
-// Four consecutive elements, 16-byte aligned.
-__device__ __forceinline__ void fd_load4(const float* p, float (&v)[4]) {
+// 16 aligned bytes of a field, and the same number of elements of a panel.
+__device__ __forceinline__ void fd_load16(const float* p, float (&v)[4]) {
   const float4 a = *reinterpret_cast<const float4*>(p);
   v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w;
 }
-__device__ __forceinline__ void fd_load4(const double* p, double (&v)[4]) {
-  const double2 a = *reinterpret_cast<const double2*>(p), b = *(reinterpret_cast<const double2*>(p) + 1);
-  v[0] = a.x, v[1] = a.y, v[2] = b.x, v[3] = b.y;
+__device__ __forceinline__ void fd_load16(const double* p, double (&v)[2]) {
+  const double2 a = *reinterpret_cast<const double2*>(p);
+  v[0] = a.x, v[1] = a.y;
 }
-__device__ __forceinline__ void fd_store4(float* p, const float (&v)[4]) { *reinterpret_cast<float4*>(p) = f4(v[0], v[1], v[2], v[3]); }
-__device__ __forceinline__ void fd_store4(double* p, const double (&v)[4]) {
-  *reinterpret_cast<double2*>(p) = make_double2(v[0], v[1]);
-  *(reinterpret_cast<double2*>(p) + 1) = make_double2(v[2], v[3]);
+__device__ __forceinline__ void fd_store16(float* p, const float (&v)[4]) { *reinterpret_cast<float4*>(p) = f4(v[0], v[1], v[2], v[3]); }
+__device__ __forceinline__ void fd_store16(double* p, const double (&v)[2]) { *reinterpret_cast<double2*>(p) = make_double2(v[0], v[1]); }
+__device__ __forceinline__ void fd_put(float* p, const float (&v)[4]) { *reinterpret_cast<float4*>(p) = f4(v[0], v[1], v[2], v[3]); }
+__device__ __forceinline__ void fd_put(float* p, const float (&v)[2]) { *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1]); }
+__device__ __forceinline__ void fd_get(const float* p, float (&v)[4]) { fd_load16(p, v); }
+__device__ __forceinline__ void fd_get(const float* p, float (&v)[2]) {
+  const float2 a = *reinterpret_cast<const float2*>(p);
+  v[0] = a.x, v[1] = a.y;
 }
 
-// phi64 += z with the potential's other forms.
+// phi64 += z with the potential's other forms (v: phi64's old values).
 template <typename T>
 __device__ __forceinline__ void fd_correct(const FdJob& J, long long i, T z) {
   const double v = J.phi64[i] + (sizeof(T) == 4 ? double_of_float((float)z) : (double)z);
@@ -329,21 +332,13 @@ __device__ __forceinline__ void fd_correct(const FdJob& J, long long i, T z) {
   J.phi32[i] = ff_nearest(p);
 }
 template <typename T>
-__device__ __forceinline__ void fd_correct4(const FdJob& J, long long i, const T (&z)[4]) {
-  double v[4];
-  fd_load4(J.phi64 + i, v);
-  float2 p[4];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    v[k] += sizeof(T) == 4 ? double_of_float((float)z[k]) : (double)z[k];
-    p[k] = ff_of_double(v[k]);
-  }
-  fd_store4(J.phi64 + i, v);
-  if (J.phi2) {
-    *reinterpret_cast<float4*>(J.phi2 + i) = f4(p[0].x, p[0].y, p[1].x, p[1].y);
-    *reinterpret_cast<float4*>(J.phi2 + i + 2) = f4(p[2].x, p[2].y, p[3].x, p[3].y);
-  }
-  *reinterpret_cast<float4*>(J.phi32 + i) = f4(ff_nearest(p[0]), ff_nearest(p[1]), ff_nearest(p[2]), ff_nearest(p[3]));
+__device__ __forceinline__ void fd_correct2(const FdJob& J, long long i, double2 v, const T (&z)[2]) {
+  v.x += sizeof(T) == 4 ? double_of_float((float)z[0]) : (double)z[0];
+  v.y += sizeof(T) == 4 ? double_of_float((float)z[1]) : (double)z[1];
+  const float2 p = ff_of_double(v.x), q = ff_of_double(v.y);
+  *reinterpret_cast<double2*>(J.phi64 + i) = v;
+  if (J.phi2) *reinterpret_cast<float4*>(J.phi2 + i) = f4(p.x, p.y, q.x, q.y);
+  *reinterpret_cast<float2*>(J.phi32 + i) = make_float2(ff_nearest(p), ff_nearest(q));
 }
 
 // One block's panel of a pass: columns [c0, c0 + TC) of the job.  T is the field
@@ -374,44 +369,34 @@ __device__ __forceinline__ void fd_panel(const FdJob& J, long long c0, int bid, 
   if constexpr (XAX && MODE == FD_FWD) {
     const T* src = static_cast<const T*>(J.in);
     if (J.vec) {
-      const int gr = ne / 4;  // groups of four of a half row
+      constexpr int GS = 16 / (int)sizeof(T);  // elements of a lane's 16 bytes
+      const int gr = ne / GS;                  // groups of a half row
 #pragma unroll 4
       for (int q = tid; q < TC * gr; q += nt) {
-        const int c = q / gr, x = (q - c * gr) * 4;
+        const int c = q / gr, x = (q - c * gr) * GS;
         const long long row = c0 + c;
-        T a[4] = {T(0), T(0), T(0), T(0)}, b[4] = {T(0), T(0), T(0), T(0)};
+        T a[GS] = {}, b[GS] = {};
         if (row < J.ncols) {
-          if (sizeof(T) == 4 && J.in64) {
-            double a8[4], b8[4];
-            fd_load4(J.in64 + row * n + x, a8);
-            fd_load4(J.in64 + row * n + n - 4 - x, b8);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              a[k] = (T)ff_nearest(ff_of_double(a8[k]));
-              b[k] = (T)ff_nearest(ff_of_double(b8[k]));
-            }
-          } else {
-            fd_load4(src + row * n + x, a);
-            fd_load4(src + row * n + n - 4 - x, b);
-          }
+          fd_load16(src + row * n + x, a);
+          fd_load16(src + row * n + n - GS - x, b);
         }
-        float2 s[4], d[4];
+        float s[GS], d[GS], sl[GS], dl[GS];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
+        for (int k = 0; k < GS; ++k) {
           if constexpr (FF) {
-            const float2 fa = fd_ff_of(a[k]), fb = fd_ff_of(b[3 - k]);
-            s[k] = fd_ff_add(fa, fb);
-            d[k] = fd_ff_add(fa, fd_neg(fb));
+            const float2 fa = ff_of_double(a[k]), fb = ff_of_double(b[GS - 1 - k]);
+            const float2 sv = fd_ff_add(fa, fb), dv = fd_ff_add(fa, fd_neg(fb));
+            s[k] = sv.x, sl[k] = sv.y, d[k] = dv.x, dl[k] = dv.y;
           } else {
-            s[k] = make_float2(a[k] + b[3 - k], 0.0f);
-            d[k] = make_float2(a[k] - b[3 - k], 0.0f);
+            s[k] = a[k] + b[GS - 1 - k];
+            d[k] = a[k] - b[GS - 1 - k];
           }
         }
-        *reinterpret_cast<float4*>(ph + c * P + x) = f4(s[0].x, s[1].x, s[2].x, s[3].x);
-        *reinterpret_cast<float4*>(ph + c * P + oo + x) = f4(d[0].x, d[1].x, d[2].x, d[3].x);
+        fd_put(ph + c * P + x, s);
+        fd_put(ph + c * P + oo + x, d);
         if constexpr (FF) {
-          *reinterpret_cast<float4*>(pl + c * P + x) = f4(s[0].y, s[1].y, s[2].y, s[3].y);
-          *reinterpret_cast<float4*>(pl + c * P + oo + x) = f4(d[0].y, d[1].y, d[2].y, d[3].y);
+          fd_put(pl + c * P + x, sl);
+          fd_put(pl + c * P + oo + x, dl);
         }
       }
     } else {
@@ -419,18 +404,14 @@ __device__ __forceinline__ void fd_panel(const FdJob& J, long long c0, int bid, 
         const long long row = c0 + c;
         const bool ok = row < J.ncols;
         const long long o = (ok ? row : 0) * n;
-        auto at = [&](int x) -> T {
-          if (sizeof(T) == 4 && J.in64) return (T)ff_nearest(ff_of_double(J.in64[o + x]));
-          return src[o + x];
-        };
 #pragma unroll 4
         for (int x = lane; x < oo; x += 32) {
           T a = T(0), b = T(0);
-          if (ok && x < ne) a = at(x);
-          if (ok && x < no) b = at(n - 1 - x);
+          if (ok && x < ne) a = src[o + x];
+          if (ok && x < no) b = src[o + n - 1 - x];
           float2 s, d;
           if constexpr (FF) {
-            const float2 fa = fd_ff_of(a), fb = fd_ff_of(b);
+            const float2 fa = ff_of_double(a), fb = ff_of_double(b);
             s = fd_ff_add(fa, fb);
             d = fd_ff_add(fa, fd_neg(fb));
           } else {
@@ -621,7 +602,8 @@ __device__ __forceinline__ void fd_panel(const FdJob& J, long long c0, int bid, 
     const long long col = c0 + cl;
     const bool ok = col < J.ncols;
     const int kx = ok ? (int)(col % J.pitch) : 0, ky = ok ? (int)(col / J.pitch) : 0;
-    const float2 h2 = fd_ff_of(1.0 / J.ih2);
+    const double hh = 1.0 / J.ih2;
+    const float2 h2 = make_float2((float)hh, (float)(hh - (double)(float)hh));
     DotAcc<float> dot;
 #pragma unroll
     for (int t = 0; t < TPW; ++t) {
@@ -706,30 +688,62 @@ __device__ __forceinline__ void fd_panel(const FdJob& J, long long c0, int bid, 
       }
     };
     if (J.vec) {
-      const int gr = ne / 4;
-#pragma unroll 2
-      for (int q = tid; q < TC * gr; q += nt) {
-        const int c = q / gr, x = (q - c * gr) * 4;
-        if (c0 + c >= J.ncols) break;
-        const float4 e = *reinterpret_cast<const float4*>(ph + c * P + x);
-        const float4 d = *reinterpret_cast<const float4*>(ph + c * P + oo + x);
-        float4 el = f4(0.f, 0.f, 0.f, 0.f), dl = el;
+      // a lane stores 16 bytes of its widest array at a time (with 32 the sectors of a
+      // store are half filled: 98 against 45 us for the correcting pass at 192^3)
+      const int cols = (int)min((long long)TC, J.ncols - c0);
+      auto halves = [&](auto gs, int c, int x, T* up, T* dn) {
+        constexpr int GS = decltype(gs)::value;
+        float e[GS], d[GS], el[GS] = {}, dl[GS] = {};
+        fd_get(ph + c * P + x, e);
+        fd_get(ph + c * P + oo + x, d);
         if constexpr (FF) {
-          el = *reinterpret_cast<const float4*>(pl + c * P + x);
-          dl = *reinterpret_cast<const float4*>(pl + c * P + oo + x);
+          fd_get(pl + c * P + x, el);
+          fd_get(pl + c * P + oo + x, dl);
         }
-        const T up[4] = {value(e.x, el.x, d.x, dl.x), value(e.y, el.y, d.y, dl.y), value(e.z, el.z, d.z, dl.z),
-                         value(e.w, el.w, d.w, dl.w)};
-        const T dn[4] = {value(e.w, el.w, -d.w, -dl.w), value(e.z, el.z, -d.z, -dl.z),
-                         value(e.y, el.y, -d.y, -dl.y), value(e.x, el.x, -d.x, -dl.x)};
-        const long long o = (c0 + c) * n;
-        if (!out) {
-          fd_correct4(J, o + x, up);
-          fd_correct4(J, o + n - 4 - x, dn);
-          continue;
+#pragma unroll
+        for (int k = 0; k < GS; ++k) {
+          up[k] = value(e[k], el[k], d[k], dl[k]);
+          dn[GS - 1 - k] = value(e[k], el[k], -d[k], -dl[k]);
         }
-        fd_store4(out + o + x, up);
-        fd_store4(out + o + n - 4 - x, dn);
+      };
+      if (out) {
+        constexpr int GS = 16 / (int)sizeof(T);
+        const int gr = ne / GS, items = cols * gr;
+#pragma unroll 2
+        for (int q = tid; q < items; q += nt) {
+          const int c = q / gr, x = (q - c * gr) * GS;
+          T up[GS], dn[GS];
+          halves(std::integral_constant<int, GS>{}, c, x, up, dn);
+          const long long o = (c0 + c) * n;
+          fd_store16(out + o + x, up);
+          fd_store16(out + o + n - GS - x, dn);
+        }
+      } else {
+        // the potential's old values of four items in flight together
+        const int gr = ne / 2, items = cols * gr;
+        for (int q0 = tid; q0 < items; q0 += 4 * nt) {
+          double2 pu[4], pd[4];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const int q = q0 + k * nt, c = q / gr, x = (q - c * gr) * 2;
+            const long long o = (c0 + c) * n;
+            if (q < items) {
+              pu[k] = *reinterpret_cast<const double2*>(J.phi64 + o + x);
+              pd[k] = *reinterpret_cast<const double2*>(J.phi64 + o + n - 2 - x);
+            }
+          }
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const int q = q0 + k * nt, c = q / gr, x = (q - c * gr) * 2;
+            const long long o = (c0 + c) * n;
+            if (q < items) {
+              T up[2], dn[2];
+              halves(std::integral_constant<int, 2>{}, c, x, up, dn);
+              fd_correct2(J, o + x, pu[k], up);
+              fd_correct2(J, o + n - 2 - x, pd[k], dn);
+            }
+          }
+        }
       }
     } else {
       for (int c = warp; c < TC; c += nw) {

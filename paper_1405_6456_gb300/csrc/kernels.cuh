@@ -9,6 +9,8 @@
 
 #include <cooperative_groups.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace ofd {
@@ -184,7 +186,10 @@ struct CgScalars {
 // Epi:    static constexpr int K (number of FP64 partial sums), bool skip(),
 //         void apply(idx, centre, lap, acc[K]), and fin(sums[K]) run once by
 //         the last block.
+//         Pre prefetch(idx) loads, ahead of the stencil's arithmetic, what apply
+//         reads at the node from arrays the pipeline does not stage.
 // Epilogue accumulators: plain doubles, or DotAcc (compensated for FP32).
+struct NoPre {};
 __device__ __forceinline__ double to_double(double v) { return v; }
 template <typename T>
 __device__ __forceinline__ double to_double(const DotAcc<T>& a) { return a.value(); }
@@ -527,6 +532,15 @@ __device__ __forceinline__ void zstream_tile(const GridDev& g, const Weights<T>&
       cp_async_wait<ZD - 1>();  // planes <= k + R have landed (this thread's copies)
       __syncthreads();          // ... and every other thread's
     }
+    // values the epilogue reads at its own nodes from elsewhere are asked for here,
+    // ahead of the stencil's arithmetic
+    const long long base = plane * k + (long long)g.n1 * y0 + x0;
+    typename Epi::Pre pre[RY][CX];
+#pragma unroll
+    for (int i = 0; i < RY; ++i)
+#pragma unroll
+      for (int l = 0; l < CX; ++l)
+        if ((node_ok >> (i * CX + l)) & 1u) pre[i][l] = ep.prefetch(base + (long long)g.n1 * i + l);
     const T* pk = ring[sk] + cb;  // (row offset m, first column) of plane k at pk[m * SX]
 #pragma unroll
     for (int i = 0; i < RY; ++i) q[i][2 * R] = L::ld(ring[sf] + cb + (i + R) * SX);
@@ -549,6 +563,21 @@ __device__ __forceinline__ void zstream_tile(const GridDev& g, const Weights<T>&
 #pragma unroll
         for (int l = 0; l < CX; ++l) win[c + l] = L::lane(t, l);
       }
+      if constexpr (std::is_same<T, float2>::value) {
+        // float-float: a product and a sum cost 12 operations against 8 for an add,
+        // so the six neighbours at a distance are added first (316 operations a node
+        // at R = 6 against 364 with a chain per axis)
+        VT s = L::mul(W.w[1], L::add(L::add(L::add(L::make(win + RE + 1), L::make(win + RE - 1)),
+                                            L::add(ycol(i + R + 1), ycol(i + R - 1))),
+                                     L::add(q[i][R + 1], q[i][R - 1])));
+#pragma unroll
+        for (int p = 2; p <= R; ++p)
+          s = L::fma(W.w[p], L::add(L::add(L::add(L::make(win + RE + p), L::make(win + RE - p)),
+                                           L::add(ycol(i + R + p), ycol(i + R - p))),
+                                    L::add(q[i][R + p], q[i][R - p])), s);
+        lap[i] = L::add(lap[i], s);
+        continue;
+      }
       // one weighted sum per axis: three independent FMA chains per row
       VT ax = L::mul(W.w[1], L::add(L::make(win + RE + 1), L::make(win + RE - 1)));
       VT ay = L::mul(W.w[1], L::add(ycol(i + R + 1), ycol(i + R - 1)));
@@ -561,7 +590,6 @@ __device__ __forceinline__ void zstream_tile(const GridDev& g, const Weights<T>&
       }
       lap[i] = L::add(L::add(L::add(lap[i], ax), ay), az);
     }
-    const long long base = plane * k + (long long)g.n1 * y0 + x0;
 #pragma unroll
     for (int i = 0; i < RY; ++i)
 #pragma unroll
@@ -570,7 +598,7 @@ __device__ __forceinline__ void zstream_tile(const GridDev& g, const Weights<T>&
           T vin[NIN > 0 ? NIN : 1];
 #pragma unroll
           for (int j = 0; j < NIN; ++j) vin[j] = pin[ik][j][(ty * RY + i) * BX + CX * tx + l];
-          ep.apply(base + (long long)g.n1 * i + l, L::lane(q[i][R], l), L::lane(lap[i], l), vin, acc);
+          ep.apply(base + (long long)g.n1 * i + l, L::lane(q[i][R], l), L::lane(lap[i], l), vin, pre[i][l], acc);
         }
       }
 #pragma unroll
@@ -619,10 +647,12 @@ struct EpiCgAv {
   T* q;
   int first_;
   T beta_;
+  using Pre = NoPre;
+  __device__ __forceinline__ Pre prefetch(long long) const { return {}; }
   __device__ __forceinline__ bool skip() const { return false; }
   __device__ __forceinline__ void load() {}
   __host__ __device__ __forceinline__ const T* input(int j) const { return j == 0 ? p : q; }
-  __device__ __forceinline__ void apply(long long i, T rc, T ar, const T* vin, Acc* acc) const {
+  __device__ __forceinline__ void apply(long long i, T rc, T ar, const T* vin, const Pre&, Acc* acc) const {
     T pc, qc;
     if (first_) {
       pc = rc;
@@ -865,10 +895,12 @@ struct EpiStore {
   static constexpr int NIN = 0;
   using Acc = double;
   T* out;
+  using Pre = NoPre;
+  __device__ __forceinline__ Pre prefetch(long long) const { return {}; }
   __device__ __forceinline__ bool skip() const { return false; }
   __device__ __forceinline__ void load() {}
   __host__ __device__ __forceinline__ const T* input(int) const { return nullptr; }
-  __device__ __forceinline__ void apply(long long i, T, T lap, const T*, Acc*) const { out[i] = lap; }
+  __device__ __forceinline__ void apply(long long i, T, T lap, const T*, const Pre&, Acc*) const { out[i] = lap; }
   __device__ __forceinline__ void operator()(double*) const {}
 };
 
@@ -887,13 +919,15 @@ struct EpiCgA {
   CgScalars* sc;
   int first_ = 0;  // copies of the CG scalars, read once per block by load()
   T beta_ = T(0);
+  using Pre = NoPre;
+  __device__ __forceinline__ Pre prefetch(long long) const { return {}; }
   __device__ __forceinline__ bool skip() const { return sc->done != 0; }
   __device__ __forceinline__ void load() {
     first_ = sc->first;
     beta_ = (T)sc->beta;
   }
   __host__ __device__ __forceinline__ const T* input(int j) const { return j == 0 ? p : q; }
-  __device__ __forceinline__ void apply(long long i, T rc, T ar, const T* vin, Acc* acc) const {
+  __device__ __forceinline__ void apply(long long i, T rc, T ar, const T* vin, const Pre&, Acc* acc) const {
     T pc, qc;
     if (first_) {
       pc = rc;
@@ -929,6 +963,8 @@ struct EpiCgAX {
   CgScalars* sc;
   int first_ = 0, xd_ = 0;
   T beta_ = T(0), alpha_ = T(0);
+  using Pre = NoPre;
+  __device__ __forceinline__ Pre prefetch(long long) const { return {}; }
   __device__ __forceinline__ bool skip() const { return sc->done != 0; }
   __device__ __forceinline__ void load() {
     first_ = sc->first;
@@ -937,7 +973,7 @@ struct EpiCgAX {
     alpha_ = (T)sc->alpha;
   }
   __host__ __device__ __forceinline__ const T* input(int j) const { return j == 0 ? p : (j == 1 ? q : x); }
-  __device__ __forceinline__ void apply(long long i, T rc, T ar, const T* vin, Acc* acc) const {
+  __device__ __forceinline__ void apply(long long i, T rc, T ar, const T* vin, const Pre&, Acc* acc) const {
     if (xd_) x[i] = fma(alpha_, vin[0], vin[2]);
     T pc, qc;
     if (first_) {
@@ -976,20 +1012,29 @@ struct EpiResidual {
   int max_it;
   int want_r;
   int pc = 0;  // the CG that follows is preconditioned
+  float* r32 = nullptr;  // optional: the residual's FP32 rounding (for an FP32 correction)
+  struct Pre {
+    U u, rho;
+    V b;
+  };
+  __device__ __forceinline__ Pre prefetch(long long i) const {
+    return {u ? u[i] : U(0), (want_r && rho) ? rho[i] : U(0), (want_r && !rho) ? b[i] : V(0)};
+  }
   __device__ __forceinline__ bool skip() const { return false; }
   __device__ __forceinline__ void load() {}
   __host__ __device__ __forceinline__ const T* input(int) const { return nullptr; }
-  __device__ __forceinline__ void apply(long long i, T, T lap, const T*, double* acc) const {
+  __device__ __forceinline__ void apply(long long i, T, T lap, const T*, const Pre& pre, double* acc) const {
     T uu = T(0);
     if (u) {
-      const T ui = (T)u[i];
+      const T ui = (T)pre.u;
       uu = ui * ui;
       acc[0] += (double)ui * (double)ui;
     }
     if (want_r) {
-      const T rh = (T)(4.0 * kPi) * (rho ? (T)rho[i] : uu + (T)b[i]);
+      const T rh = (T)(4.0 * kPi) * (rho ? (T)pre.rho : uu + (T)pre.b);
       const T ri = rh + lap;
       r[i] = ri;
+      if (r32) r32[i] = ff_nearest(ff_of_double((double)ri));
       acc[1] += (double)rh * (double)rh;
       acc[2] += (double)ri * (double)ri;
     }
@@ -1022,6 +1067,9 @@ struct EpiResidual {
 // the variational electrostatic energy of the functional that follows, of
 // (u^2 + b) phi and phi r.  Accuracy: about 2^-48 of the magnitudes of the
 // stencil's terms (the FP64 pass: 2^-53).
+// Bound by the FP32 pipes: 316 operations a node for the stencil at R = 6 and about
+// 80 here.  At 192^3 138 us, 0.49 of the pipes' rate (180 us with a chain per axis,
+// three compensated terms per electrostatic sum and u read when it was used).
 __device__ __forceinline__ float2 ff_prod(float a, float b) {  // a b exactly
   const float p = a * b;
   return make_float2(p, fmaf(a, b, -p));
@@ -1041,17 +1089,19 @@ struct EpiResidualFF {
   int max_it;
   int pc = 0;  // the CG that follows is preconditioned
   float2 fourpi;
+  using Pre = float;  // u, or the explicit density
+  __device__ __forceinline__ Pre prefetch(long long i) const { return rho ? rho[i] : u[i]; }
   __device__ __forceinline__ bool skip() const { return false; }
   __device__ __forceinline__ void load() {}
   __host__ __device__ __forceinline__ const float2* input(int) const { return rho ? nullptr : b2; }
-  __device__ __forceinline__ void apply(long long i, float2 ph, float2 lap_raw, const float2* vin, Acc* acc) const {
+  __device__ __forceinline__ void apply(long long i, float2 ph, float2 lap_raw, const float2* vin, const Pre& pre, Acc* acc) const {
     // the stencil's float-float sum comes unnormalised (lazy chain): renormalise
     const float2 lap = ff_two_sum(lap_raw.x, lap_raw.y);
     float2 rr;
     if (rho) {
-      rr = make_float2(rho[i], 0.0f);
+      rr = make_float2(pre, 0.0f);
     } else {
-      const float ui = u[i];
+      const float ui = pre;
       acc[0].add(ui, ui);
       rr = ff_add(ff_prod(ui, ui), vin[0]);
     }
@@ -1217,6 +1267,16 @@ struct EpiFunctional {
   // MIXED with the float-float residual pass: that pass already summed (u^2 + b) phi
   // and phi r in compensated arithmetic; the functional takes them from here
   const CgScalars* es_sums = nullptr;
+  struct Pre {
+    T s, d, r;
+  };
+  __device__ __forceinline__ Pre prefetch(long long i) const {
+    Pre v;
+    v.s = s_old ? s_old[i] : T(0);
+    v.d = (NIN < 3 && d) ? d[i] : T(0);
+    v.r = rcg ? rcg[i] : T(0);
+    return v;
+  }
   __device__ __forceinline__ bool skip() const { return false; }
   __device__ __forceinline__ void load() {
     const double C = f.h3 * *sum_uu - f.N;
@@ -1231,7 +1291,7 @@ struct EpiFunctional {
     if (j == 1) return ((f.terms & 8) && !es_sums) ? b : nullptr;
     return d;
   }
-  __device__ __forceinline__ void apply(long long i, T uc, T lap, const T* vin, Acc* acc) const {
+  __device__ __forceinline__ void apply(long long i, T uc, T lap, const T* vin, const Pre& pre, Acc* acc) const {
     const T mult = mult_;
     const bool tf = f.terms & 1, vw = f.terms & 2, xc = f.terms & 4, es = f.terms & 8;
     const T ux = fabs(uc);
@@ -1260,7 +1320,7 @@ struct EpiFunctional {
         ph = vin[0];
         const T rho = uc * uc + vin[1];
         acc[3].add(rho, ph);
-        if (rcg) acc[4].add(ph, rcg[i]);
+        if (rcg) acc[4].add(ph, pre.r);
       }
     }
     const T gx = (vw ? lam_ * lap : T(0)) + T(2) * (vk + vxc + ph) * uc + T(2) * mult * uc;
@@ -1283,9 +1343,9 @@ struct EpiFunctional {
       if constexpr (NIN == 3)
         acc[5].add(gx, vin[2]);
       else
-        acc[5].add(gx, d[i]);
+        acc[5].add(gx, pre.d);
     }
-    if (s_old) acc[6].add(gx, s_old[i]);
+    if (s_old) acc[6].add(gx, pre.s);
     acc[7].add_fast(gx, -sx);  // g^2 / diag
     acc[8].add_fast(gx, gx);
     acc[9].add(uc, sx);
@@ -1779,10 +1839,12 @@ struct EpiMgDown {
   using Acc = double;
   T* t;
   const CgScalars* sc;
+  using Pre = NoPre;
+  __device__ __forceinline__ Pre prefetch(long long) const { return {}; }
   __device__ __forceinline__ bool skip() const { return sc->done != 0; }
   __device__ __forceinline__ void load() {}
   __host__ __device__ __forceinline__ const T* input(int) const { return nullptr; }
-  __device__ __forceinline__ void apply(long long i, T, T lap, const T*, Acc*) const { t[i] = lap; }
+  __device__ __forceinline__ void apply(long long i, T, T lap, const T*, const Pre&, Acc*) const { t[i] = lap; }
   __device__ __forceinline__ void operator()(double*) const {}
 };
 // up: z = stencil(y) + s r (r staged with the stencil input); on the finest
@@ -1796,10 +1858,12 @@ struct EpiMgUp {
   T* z;
   T s;
   CgScalars* sc;
+  using Pre = NoPre;
+  __device__ __forceinline__ Pre prefetch(long long) const { return {}; }
   __device__ __forceinline__ bool skip() const { return sc->done != 0; }
   __device__ __forceinline__ void load() {}
   __host__ __device__ __forceinline__ const T* input(int) const { return r; }
-  __device__ __forceinline__ void apply(long long i, T, T lap, const T* vin, Acc* acc) const {
+  __device__ __forceinline__ void apply(long long i, T, T lap, const T* vin, const Pre&, Acc* acc) const {
     const T zi = fma(s, vin[0], lap);
     z[i] = zi;
     if constexpr (DOT) acc[0].add(vin[0], zi);
@@ -2883,6 +2947,24 @@ struct OpLine {
       phi0[i] = phi[i];
     else
       phi[i] = fma(t, phi[i] - phi0[i], phi[i]);
+  }
+  __device__ __forceinline__ void operator()(double*) const {}
+};
+
+// A field's values as float pairs (in place where the pairs' array is the field's own)
+// and, when out32 is given, their FP32 rounding.
+struct OpPairs {
+  static constexpr int K = 0;
+  const double* in;
+  float2* out;
+  float* out32;
+  using Acc = double;
+  __device__ __forceinline__ void load() {}
+  __device__ __forceinline__ bool skip() const { return false; }
+  __device__ __forceinline__ void apply(long long i, double*) const {
+    const float2 p = ff_of_double(in[i]);
+    out[i] = p;
+    if (out32) out32[i] = ff_nearest(p);
   }
   __device__ __forceinline__ void operator()(double*) const {}
 };
