@@ -100,7 +100,7 @@ int mg_prepare(ofdft_ctx* c, const GridDev& g, int R, double h, MgPlan* P) {
     TRY(fd_plan(c, g, R, h, &P->fd));
     if (P->fd.on) {
       TRY(ensure(c, c->v[V_T], fd_scratch(g) * sizeof(T)));
-      return ensure_partials(c, (long long)P->fd.pitch * g.n2 / 32 + 1, 1);
+      return ensure_partials(c, (long long)P->fd.pitch * g.n2 / 16 + 1, 1);
     }
   }
   TRY(ensure(c, c->v[V_T], g.G * sizeof(T)));
@@ -656,7 +656,7 @@ int cg_coop(ofdft_ctx* c, int R, const GridDev& g, const Weights<double>& Wneg, 
 // sets of sampling events and the host reads chunk k's set while chunk k+1 runs.
 template <typename T, typename X = T>
 int cg_iterate(ofdft_ctx* c, int R, const GridDev& g, double h, const Weights<double>& Wneg, X* x, T* r,
-               CgScalars* sc, int max_it, CgScalars* host_sc) {
+               CgScalars* sc, int max_it, CgScalars* host_sc, Behind* behind = nullptr) {
   T* pv = vec<T>(c, V_P0);
   T* qv = vec<T>(c, V_AP);
   const bool per_launch = (c->prof & (1 << OFDFT_K_CG_UPDATE)) != 0;  // per-kernel timing asked for
@@ -681,13 +681,13 @@ int cg_iterate(ofdft_ctx* c, int R, const GridDev& g, double h, const Weights<do
     const int it0 = host_sc->iters;
     TRY((cg_step<T, X>(c, R, g, Wneg, x, r, pv, qv, sc, pb, &mg)));
     if (mg.fd.on) {
-      // one step of the directly inverted operator mostly ends the solve
-      CgScalars first;
-      TRY(sync_scalars(c, sc, sizeof(CgScalars), &first));
-      if (first.done) {
-        if (first.xdefer) TRY(cg_flush<T>(c, g, reinterpret_cast<T*>(x), pv, sc));
-        *host_sc = first;
-        host_sc->xdefer = 0;
+      // one step of the directly inverted operator mostly ends the solve (every
+      // kernel so far did nothing if it had ended before)
+      if (cg_fold<T>(c, g)) TRY(cg_flush<T>(c, g, reinterpret_cast<T*>(x), pv, sc));
+      if (behind) TRY(behind->launch());
+      TRY(sync_behind(c, sc, host_sc, behind));
+      if (host_sc->done) {
+        if (behind) behind->done = true;
         return OFDFT_OK;
       }
     }
@@ -766,7 +766,7 @@ int ensure_cg_vectors(ofdft_ctx* c, long long G, size_t es, bool mixed) {
 // FP64 Poisson solve: r = 4 pi rho + L phi, then CG.  rho = rho_in or u^2 + b.
 // On return r (V_R) holds the final recursive residual; st gets the stats.
 int poisson_fp64(ofdft_ctx* c, int R, const GridDev& g, double h, const double* rho, const double* u,
-                 const double* b, double* phi, double tol, int max_it, ofdft_cg_stats* st) {
+                 const double* b, double* phi, double tol, int max_it, ofdft_cg_stats* st, Behind* behind = nullptr) {
   TRY(ensure_cg_vectors(c, g.G, sizeof(double), false));
   const Weights<double> W = lap_weights(R, h, 1.0), Wneg = lap_weights(R, h, -1.0);
   double* r = vec<double>(c, V_R);
@@ -775,8 +775,12 @@ int poisson_fp64(ofdft_ctx* c, int R, const GridDev& g, double h, const double* 
   TRY(launch_z_r<double>(c, R, g, W, LoadPlain<double>{phi},
                          EpiResidual<double>{rho, u, b, r, c->sc, tol, max_it, 1, mg.ok ? 1 : 0}, OFDFT_K_RESIDUAL));
   CgScalars hs;
-  TRY(sync_scalars(c, c->sc, sizeof(CgScalars), &hs));
-  if (!hs.done) TRY(cg_iterate<double>(c, R, g, h, Wneg, phi, r, c->sc, max_it, &hs));
+  memset(&hs, 0, sizeof(hs));
+  // a directly inverted operator's one step is launched without waiting for the
+  // residual: it does nothing where the residual already meets tol
+  const bool ahead = mg.fd.on && max_it > 0 && c->use_graphs && c->cond_graphs;
+  if (!ahead) TRY(sync_scalars(c, c->sc, sizeof(CgScalars), &hs));
+  if (ahead || !hs.done) TRY(cg_iterate<double>(c, R, g, h, Wneg, phi, r, c->sc, max_it, &hs, ahead ? behind : nullptr));
   if (st) {
     st->iterations = hs.iters;
     st->rel_residual = sqrt(hs.rr / (hs.bb > 0 ? hs.bb : 1.0));
@@ -798,6 +802,7 @@ struct MixedStart {
   const double* line0 = nullptr;  // potential at the line search's origin (t != 0)
   double t = 0.0;
   const float* b32 = nullptr;
+  int chain = 1;                  // direct corrections launched before the first wait
 };
 
 // Mixed Poisson solve (S3 + S10): FP32 corrections of an FP64 potential.  Each round
@@ -823,7 +828,8 @@ struct MixedStart {
 // here after a split.
 int poisson_mixed(ofdft_ctx* c, int R, const GridDev& g, double h, const float* rho32, const float* u,
                   const double* b64, double* phi64, float* phi32, double tol, int max_it, int refine_every,
-                  ofdft_cg_stats* st, int* b2_valid = nullptr, const MixedStart& from = MixedStart{}) {
+                  ofdft_cg_stats* st, int* b2_valid = nullptr, const MixedStart& from = MixedStart{},
+                  Behind* behind = nullptr) {
   TRY(ensure_cg_vectors(c, g.G, sizeof(float), true));
   const Weights<double> W = lap_weights(R, h, 1.0), Wneg = lap_weights(R, h, -1.0);
   double* r64 = vec<double>(c, V_R64);
@@ -880,17 +886,49 @@ int poisson_mixed(ofdft_ctx* c, int R, const GridDev& g, double h, const float* 
     }
     CU(cudaGetLastError());
   }
-  if (!direct) CU(cudaMemsetAsync(e32, 0, g.G * sizeof(float), c->stream));
   const float2 fourpi = ff_of(4.0 * kPi);
-  double rr_old = -1.0;
-  for (int round = 0; round <= max_rounds; ++round) {
-    if (round > 0 && !direct) {
+  // Direct corrections: from.chain of them, each with its residual, are launched
+  // before the first wait (one afterwards), every kernel doing nothing once the solve
+  // is done, and `behind` after them.
+  bool have_r = false;
+  for (double rr_old = -1.0; direct;) {
+    const int k1 = std::max(0, std::min(std::min(have_r ? 1 : from.chain, max_it - total), max_rounds - total));
+    for (int k = have_r ? 1 : 0; k <= k1; ++k) {
+      if (k > 0) TRY(fd_correction(c, g, mg.fd, r32, c->v[V_T].p, phi64, phi2, phi32, c->sc));
+      const EpiResidualFF ep{rho32, rho32 ? nullptr : u, b2, nullptr, r32, c->sc, tol, max_it, 0, fourpi,
+                             k > 0 ? c->sc : nullptr, k};
+      TRY(launch_z_r<float2>(c, R, g, W, LoadPlain<float2>{phi2}, ep, OFDFT_K_RESIDUAL));
+    }
+    if (behind) TRY(behind->launch());
+    TRY(sync_behind(c, c->sc, &hs, behind));
+    total += hs.iters;
+    const double bb = hs.bb > 0 ? hs.bb : 1.0;
+    if (c->trace) fprintf(stderr, "[ofdft] mixed direct corrections %d rel64=%.3e\n", total, sqrt(hs.rr / bb));
+    if (st) {
+      st->iterations = total;
+      st->rel_residual = sqrt(hs.rr / bb);
+    }
+    if (!isfinite(hs.rr)) return fail(c, OFDFT_ENONFINITE, "Poisson residual is not finite");
+    if (behind) behind->done = true;  // (withdrawn where the solve goes on)
+    if (hs.rr <= tol * tol * bb) break;
+    if (total >= max_it || total >= max_rounds) {
+      rc = fail(c, OFDFT_ENOTCONV, "mixed Poisson reached %d FP32 iterations at relative residual %.3e", total,
+                sqrt(hs.rr / bb));
+      break;
+    }
+    if (behind) behind->done = false;
+    if (rr_old >= 0.0 && hs.rr > 0.25 * rr_old) direct = false;  // not halved: go on with CG
+    rr_old = hs.rr;
+    have_r = true;
+  }
+  if (!direct) CU(cudaMemsetAsync(e32, 0, g.G * sizeof(float), c->stream));
+  for (int round = 0; round <= max_rounds && !direct; ++round) {
+    if (round > 0) {
       ProfScope ps_(c, OFDFT_K_VECTOR);
       fold_kernel<<<pb, 256, 0, c->stream>>>(g.G, phi64, e32, phi2);
     }
     if (c->mixed_ff) {
-      const EpiResidualFF ep{rho32, rho32 ? nullptr : u, b2, direct ? nullptr : r2, direct ? r32 : nullptr, c->sc, tol,
-                             max_it, 0, fourpi};
+      const EpiResidualFF ep{rho32, rho32 ? nullptr : u, b2, r2, nullptr, c->sc, tol, max_it, 0, fourpi};
       TRY(launch_z_r<float2>(c, R, g, W, LoadPlain<float2>{phi2}, ep, OFDFT_K_RESIDUAL));
     } else {
       const EpiResidual<double, float, double> ep =
@@ -910,18 +948,6 @@ int poisson_mixed(ofdft_ctx* c, int R, const GridDev& g, double h, const float* 
       rc = fail(c, OFDFT_ENOTCONV, "mixed Poisson reached %d FP32 iterations at relative residual %.3e", total,
                 sqrt(hs.rr / bb));
       break;
-    }
-    if (direct) {
-      if (rr_old >= 0.0 && hs.rr > 0.25 * rr_old) {  // not halved: go on with CG (from a residual in pairs)
-        direct = false;
-        CU(cudaMemsetAsync(e32, 0, g.G * sizeof(float), c->stream));
-        continue;
-      }
-      rr_old = hs.rr;
-      if (c->trace) fprintf(stderr, "[ofdft] mixed round %d rel64=%.3e direct\n", round, sqrt(hs.rr / bb));
-      TRY(fd_correction(c, g, mg.fd, r32, c->v[V_T].p, phi64, phi2, phi32));
-      total += 1;
-      continue;
     }
     const int budget = std::min(refine_every, max_it - total);
     TRY(ensure_partials(c, pb, 1));
@@ -960,10 +986,11 @@ int poisson_mixed(ofdft_ctx* c, int R, const GridDev& g, double h, const float* 
 
 // ------------------------------------------------------ functional (S4) ---
 
+// Launches the functional pass (its sums go to c->scal).
 template <typename T>
-int functional_pass(ofdft_ctx* c, int R, const GridDev& g, double h, const ofdft_params* p, const T* u,
+int functional_launch(ofdft_ctx* c, int R, const GridDev& g, double h, const ofdft_params* p, const T* u,
                     const T* b, const T* phi, const T* rcg, double eta, double mu, double N,
-                    const double* sum_uu_dev, T* G, T* s, const T* d, const T* s_old, EvalOut* out,
+                    const double* sum_uu_dev, T* G, T* s, const T* d, const T* s_old,
                     T* winv = nullptr, const double* phi64 = nullptr, const double* b64 = nullptr,
                     const double* r64 = nullptr, const CgScalars* es_sums = nullptr) {
   const Weights<double> W = lap_weights(R, h, 1.0);
@@ -1001,7 +1028,6 @@ int functional_pass(ofdft_ctx* c, int R, const GridDev& g, double h, const ofdft
     CU(cudaGetLastError());
     if (!d) CU(cudaMemsetAsync(c->scal + 5, 0, sizeof(double), c->stream));
   }
-  TRY(sync_scalars(c, c->scal, 12 * sizeof(double), out->sums));
   return OFDFT_OK;
 }
 
@@ -1117,15 +1143,26 @@ struct Solver {
                  ofdft_energy* out) {
     ofdft_cg_stats cs{0, 0.0};
     const bool es = p->terms & OFDFT_TERM_ES;
-    const double* sum_uu = &c->sc->sum_uu;
+    const double* sum_uu = es ? &c->sc->sum_uu : c->scal + 16;
+    EvalOut o;
+    T* winv = (p->precond_rank1 && sout) ? vec<T>(c, V_W) : nullptr;
+    // the functional goes to the device behind the Poisson solve (the phi.r energy
+    // term uses that solve's residual, FP64 in MIXED)
+    Behind fun;
+    fun.out = &o;
+    fun.launch = [&]() {
+      return functional_launch<T>(c, R, g, h, p, at, b, phi, (es && !mixed) ? vec<T>(c, V_R) : nullptr, eta, mu, N,
+                                  sum_uu, Gout, sout, dd, s_old, winv, mixed ? phi64 : nullptr, mixed ? b64 : nullptr,
+                                  mixed ? vec<double>(c, V_R64) : nullptr, (mixed && c->mixed_ff) ? c->sc : nullptr);
+    };
     if (es) {
       int rc;
       if (!mixed)
         rc = poisson_fp64(c, R, g, h, nullptr, (const double*)at, (const double*)b, (double*)phi, tol_p, p->max_cg,
-                          &cs);
+                          &cs, &fun);
       else
         rc = poisson_mixed(c, R, g, h, nullptr, (const float*)at, b64, phi64, (float*)phi, tol_p, p->max_cg,
-                           std::max(p->refine_every, 1), &cs, &b2_valid, from);
+                           std::max(p->refine_every, 1), &cs, &b2_valid, from, &fun);
       from = MixedStart{};
       if (rc != OFDFT_OK) return rc;
       stats->stencil_apps += cs.iterations + 1;
@@ -1138,15 +1175,11 @@ struct Solver {
         dot2_kernel<T><<<pb, 256, 0, c->stream>>>(g.G, at, at, nullptr, nullptr, c->scal + 16, red(c));
       }
       CU(cudaGetLastError());
-      sum_uu = c->scal + 16;
     }
-    // the phi.r energy term uses the Poisson solve's residual (FP64 in MIXED)
-    const T* rcg = (es && !mixed) ? vec<T>(c, V_R) : nullptr;
-    EvalOut o;
-    T* winv = (p->precond_rank1 && sout) ? vec<T>(c, V_W) : nullptr;
-    TRY(functional_pass<T>(c, R, g, h, p, at, b, phi, rcg, eta, mu, N, sum_uu, Gout, sout, dd, s_old, &o, winv,
-                           mixed ? phi64 : nullptr, mixed ? b64 : nullptr, mixed ? vec<double>(c, V_R64) : nullptr,
-                           (mixed && c->mixed_ff) ? c->sc : nullptr));
+    if (!fun.done) {
+      TRY(fun.launch());
+      TRY(sync_scalars(c, c->scal, 12 * sizeof(double), o.sums));
+    }
     stats->stencil_apps += 2;
     stats->grad_evals += 1;
     fill_energy(o, h, p, E_self, ezz, eta, mu, out);
@@ -2344,6 +2377,7 @@ int ofdft_poisson(ofdft_ctx* c, const ofdft_grid* g, int fd_order, int prec, con
   MixedStart from;
   from.fp32 = true;
   from.b32 = rho ? nullptr : (const float*)b;
+  from.chain = 2;  // a solve from a caller's guess mostly takes two corrections
   ofdft_params dp;
   ofdft_default_params(&dp);
   const int rc = poisson_mixed(c, fd_order / 2, gd, g->h, (const float*)rho, (const float*)u, vec<double>(c, V_B64),
@@ -2368,56 +2402,59 @@ int ofdft_energy_grad(ofdft_ctx* c, const ofdft_grid* g, const ofdft_params* p, 
   const bool es = p->terms & OFDFT_TERM_ES;
   memset(out, 0, sizeof(*out));
   ofdft_cg_stats cs{0, 0.0};
-  const double* sum_uu = &c->sc->sum_uu;
+  const double* sum_uu = es ? &c->sc->sum_uu : c->scal + 16;
   TRY(ensure_cg_vectors(c, gd.G, mixed ? 4 : 8, mixed));
-  if (es) {
-    if (!mixed) {
-      // residual at the incoming phi (and CG if asked): gives r for the energy and sum u^2
-      const int rc = poisson_fp64(c, R, gd, g->h, nullptr, (const double*)u, (const double*)b, (double*)phi,
-                                  p->tol_poisson, solve_poisson ? p->max_cg : 0, &cs);
-      if (rc != OFDFT_OK && !(rc == OFDFT_ENOTCONV && !solve_poisson)) return rc;
-      c->err.clear();
-    } else {
-      TRY(ensure(c, c->v[V_PHI64], gd.G * sizeof(double)));
-      TRY(ensure(c, c->v[V_B64], gd.G * sizeof(double)));
-      MixedStart from;
-      from.fp32 = true;
-      from.b32 = (const float*)b;
-      int rc = poisson_mixed(c, R, gd, g->h, nullptr, (const float*)u, vec<double>(c, V_B64), vec<double>(c, V_PHI64),
-                             (float*)phi, p->tol_poisson, solve_poisson ? p->max_cg : 0, std::max(p->refine_every, 1),
-                             &cs, nullptr, from);
-      if (rc != OFDFT_OK && !(rc == OFDFT_ENOTCONV && !solve_poisson)) return rc;
-      c->err.clear();
-    }
-  } else {
-    const int pb = pointwise_blocks(c, gd.G);
-    TRY(ensure_partials(c, pb, 2));
-    if (mixed)
-      {
-        ProfScope ps_(c, OFDFT_K_VECTOR);
-        dot2_kernel<float><<<pb, 256, 0, c->stream>>>(gd.G, (const float*)u, (const float*)u, nullptr, nullptr, c->scal + 16, red(c));
-      }
-    else
-      {
-        ProfScope ps_(c, OFDFT_K_VECTOR);
-        dot2_kernel<double><<<pb, 256, 0, c->stream>>>(gd.G, (const double*)u, (const double*)u, nullptr, nullptr, c->scal + 16, red(c));
-      }
-    CU(cudaGetLastError());
-    sum_uu = c->scal + 16;
-  }
   EvalOut o;
   const bool r1 = p->precond_rank1 && s;
   if (r1) TRY(ensure(c, c->v[V_W], gd.G * (mixed ? 4 : 8)));
-  if (!mixed)
-    TRY(functional_pass<double>(c, R, gd, g->h, p, (const double*)u, (const double*)b, (const double*)phi,
-                                es ? vec<double>(c, V_R) : nullptr, eta, mu, N, sum_uu, (double*)grad, (double*)s,
-                                (const double*)d, (const double*)s_old, &o, r1 ? vec<double>(c, V_W) : nullptr));
-  else
-    TRY(functional_pass<float>(c, R, gd, g->h, p, (const float*)u, (const float*)b, (const float*)phi, nullptr, eta,
-                               mu, N, sum_uu, (float*)grad, (float*)s, (const float*)d, (const float*)s_old, &o,
-                               r1 ? vec<float>(c, V_W) : nullptr, es ? vec<double>(c, V_PHI64) : nullptr,
-                               es ? vec<double>(c, V_B64) : nullptr, es ? vec<double>(c, V_R64) : nullptr,
-                               (es && c->mixed_ff) ? c->sc : nullptr));
+  if (es && mixed) {
+    TRY(ensure(c, c->v[V_PHI64], gd.G * sizeof(double)));
+    TRY(ensure(c, c->v[V_B64], gd.G * sizeof(double)));
+  }
+  Behind fun;  // the functional, launched behind the Poisson solve
+  fun.out = &o;
+  fun.launch = [&]() -> int {
+    if (!mixed)
+      return functional_launch<double>(c, R, gd, g->h, p, (const double*)u, (const double*)b, (const double*)phi,
+                                       es ? vec<double>(c, V_R) : nullptr, eta, mu, N, sum_uu, (double*)grad, (double*)s,
+                                       (const double*)d, (const double*)s_old, r1 ? vec<double>(c, V_W) : nullptr);
+    return functional_launch<float>(c, R, gd, g->h, p, (const float*)u, (const float*)b, (const float*)phi, nullptr, eta,
+                                    mu, N, sum_uu, (float*)grad, (float*)s, (const float*)d, (const float*)s_old,
+                                    r1 ? vec<float>(c, V_W) : nullptr, es ? vec<double>(c, V_PHI64) : nullptr,
+                                    es ? vec<double>(c, V_B64) : nullptr, es ? vec<double>(c, V_R64) : nullptr,
+                                    (es && c->mixed_ff) ? c->sc : nullptr);
+  };
+  if (es) {
+    int rc;
+    if (!mixed) {
+      // residual at the incoming phi (and CG if asked): gives r for the energy and sum u^2
+      rc = poisson_fp64(c, R, gd, g->h, nullptr, (const double*)u, (const double*)b, (double*)phi, p->tol_poisson,
+                        solve_poisson ? p->max_cg : 0, &cs, &fun);
+    } else {
+      MixedStart from;
+      from.fp32 = true;
+      from.b32 = (const float*)b;
+      from.chain = 2;
+      rc = poisson_mixed(c, R, gd, g->h, nullptr, (const float*)u, vec<double>(c, V_B64), vec<double>(c, V_PHI64),
+                         (float*)phi, p->tol_poisson, solve_poisson ? p->max_cg : 0, std::max(p->refine_every, 1),
+                         &cs, nullptr, from, &fun);
+    }
+    if (rc != OFDFT_OK && !(rc == OFDFT_ENOTCONV && !solve_poisson)) return rc;
+    c->err.clear();
+  } else {
+    const int pb = pointwise_blocks(c, gd.G);
+    TRY(ensure_partials(c, pb, 2));
+    ProfScope ps_(c, OFDFT_K_VECTOR);
+    if (mixed)
+      dot2_kernel<float><<<pb, 256, 0, c->stream>>>(gd.G, (const float*)u, (const float*)u, nullptr, nullptr, c->scal + 16, red(c));
+    else
+      dot2_kernel<double><<<pb, 256, 0, c->stream>>>(gd.G, (const double*)u, (const double*)u, nullptr, nullptr, c->scal + 16, red(c));
+    CU(cudaGetLastError());
+  }
+  if (!fun.done) {
+    TRY(fun.launch());
+    TRY(sync_scalars(c, c->scal, 12 * sizeof(double), o.sums));
+  }
   fill_energy(o, g->h, p, E_self, 0.0, eta, mu, out);
   if (r1) {
     // the preconditioned residual includes the exact inverse of the rank-one term (4 h^3/mu) u u^T

@@ -75,6 +75,7 @@ struct FdJob {
   const float *mxl, *myl, *mzl;  // ... low parts
   double ih2;       // 1 / h^2
   CgScalars* sc;    // the CG this serves (NULL: none; r.z is then not formed)
+  const CgScalars* gate;  // a correction launched ahead: nothing to do when its solve is done
   RedBuf red;       // z: r.z
   int nblocks;
 };
@@ -207,8 +208,11 @@ __device__ __forceinline__ void fd_contract(FdAcc<FF> (&acc)[4][CT], const FdRin
   auto node = [&](const float* wr, int i) {  // node-major
     float f[CT], fl[CT];
 #pragma unroll
-    for (int c = 0; c < CT; c += CT == 4 ? 4 : 2) {
-      if constexpr (CT == 4) {
+    for (int c = 0; c < CT; c += CT) {
+      if constexpr (CT == 1) {
+        f[0] = sh[i * pitch];
+        if constexpr (FF) fl[0] = sl[i * pitch];
+      } else if constexpr (CT == 4) {
         const float4 v = *reinterpret_cast<const float4*>(sh + i * pitch);
         f[0] = v.x, f[1] = v.y, f[2] = v.z, f[3] = v.w;
         if constexpr (FF) {
@@ -538,9 +542,12 @@ __device__ __forceinline__ void fd_panel(const FdJob& J, long long c0, int bid, 
           *reinterpret_cast<float4*>(d) = f4(hi(a[0], k & 1), hi(a[1], k & 1), hi(a[2], k & 1), hi(a[3], k & 1));
           if constexpr (FF)
             *reinterpret_cast<float4*>(dl) = f4(lo(a[0], k & 1), lo(a[1], k & 1), lo(a[2], k & 1), lo(a[3], k & 1));
-        } else {
+        } else if constexpr (CT == 2) {
           *reinterpret_cast<float2*>(d) = make_float2(hi(a[0], k & 1), hi(a[1], k & 1));
           if constexpr (FF) *reinterpret_cast<float2*>(dl) = make_float2(lo(a[0], k & 1), lo(a[1], k & 1));
+        } else {
+          *d = hi(a[0], k & 1);
+          if constexpr (FF) *dl = lo(a[0], k & 1);
         }
       }
     }
@@ -813,7 +820,7 @@ template <typename T, bool XAX, int MODE, int CT, int TPW>
 __global__ void __maxnreg__(TPW == 1 ? 80 : 128) fd_kernel(const __grid_constant__ FdJob J) {
   pdl_enter();
   extern __shared__ __align__(16) float fd_sm[];
-  if (J.sc && J.sc->done) return;
+  if ((J.sc && J.sc->done) || (J.gate && J.gate->done)) return;
   fd_panel<T, XAX, MODE, CT, TPW>(J, (long long)blockIdx.x * (16 * CT), blockIdx.x, fd_sm);
 }
 
@@ -830,7 +837,7 @@ __global__ void __maxnreg__(TPW == 1 ? 80 : 128)
   extern __shared__ __align__(16) float fd_sm[];
   const FdTile t = tiles[blockIdx.x];
   const FdJob J = jobs[t.job];
-  if (J.sc && J.sc->done) return;
+  if ((J.sc && J.sc->done) || (J.gate && J.gate->done)) return;
   fd_panel<T, XAX, MODE, CT, TPW>(J, (long long)t.panel * (16 * CT), t.panel, fd_sm);
 }
 

@@ -12,6 +12,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <functional>
 #include <string>
 #include <type_traits>
 #include <vector>
@@ -800,25 +801,30 @@ template <typename T, bool XAX, int MODE>
 int fd_pass(ofdft_ctx* c, const FdJob& J) {
   const int tiles = J.ax.pe / kFdTile + J.ax.po / kFdTile;
   const int tpw = tiles > 16 ? 2 : 1, warps = (tiles + tpw - 1) / tpw;
-  // FP32: panels of 64 columns, or of 32 where 64 would leave SMs without a block;
-  // float-float: 32 (its accumulators and its panel take twice the room)
-  const bool wide = sizeof(T) == 4 && J.ncols >= 128LL * c->sms;
-  if constexpr (sizeof(T) == 4) {
-    if (wide)
-      return tpw == 1 ? fd_launch<T, XAX, MODE, 4, 1>(c, J, warps) : fd_launch<T, XAX, MODE, 4, 2>(c, J, warps);
-  }
-  return tpw == 1 ? fd_launch<T, XAX, MODE, 2, 1>(c, J, warps) : fd_launch<T, XAX, MODE, 2, 2>(c, J, warps);
+  // Panel width.  Float-float passes keep an SM's FP32 pipes busy with one block, so
+  // the width (16 or 32 columns) that leaves the busiest SM the least columns is
+  // taken, the wider where within a tenth (us per application, 16 | 32: 48^3 56 | 68,
+  // 80^3 123 | 145, 112^3 309 | 296, 192^3 1790 | 1684).  FP32 passes wait more than
+  // they compute on small grids: 64 columns from 128 an SM on (32 | 64: 80^3 60 | 67,
+  // 112^3 92 | 104, 160^3 212 | 200, 192^3 329 | 307).
+  constexpr int HI = sizeof(T) == 4 ? 4 : 2, LO = HI / 2;
+  auto most = [&](int ct) { return (J.ncols + 16LL * ct * c->sms - 1) / (16LL * ct * c->sms) * ct; };
+  const bool wide = sizeof(T) == 4 ? J.ncols >= 128LL * c->sms : most(HI) * 10 <= most(LO) * 11;
+  if (wide) return tpw == 1 ? fd_launch<T, XAX, MODE, HI, 1>(c, J, warps) : fd_launch<T, XAX, MODE, HI, 2>(c, J, warps);
+  return tpw == 1 ? fd_launch<T, XAX, MODE, LO, 1>(c, J, warps) : fd_launch<T, XAX, MODE, LO, 2>(c, J, warps);
 }
 
 // The five passes: z = M r, or (phi64 given) phi64 += M r with its other forms.
 template <typename T>
 int fd_passes(ofdft_ctx* c, const GridDev& g, const FdPlan& P, const T* r, T* z, void* scratch, CgScalars* sc,
-              double* phi64 = nullptr, float2* phi2 = nullptr, float* phi32 = nullptr) {
+              double* phi64 = nullptr, float2* phi2 = nullptr, float* phi32 = nullptr,
+              const CgScalars* gate = nullptr) {
   auto job = [&](int p) {
     FdJob J = fd_job<T>(g, P, p, r, z, scratch, sc);
     J.phi64 = phi64;
     J.phi2 = phi2;
     J.phi32 = phi32;
+    J.gate = gate;
     if (phi64 && (((uintptr_t)phi64 | (uintptr_t)phi2 | (uintptr_t)phi32) & 15u)) J.vec = 0;
     return J;
   };
@@ -837,10 +843,10 @@ int fd_apply(ofdft_ctx* c, const GridDev& g, const FdPlan& P, const T* r, T* z, 
 }
 
 // One correction of a mixed Poisson solve: phi64 += M r, with its pairs and its FP32
-// rounding, in the last pass.
+// rounding, in the last pass; nothing when gate->done.
 inline int fd_correction(ofdft_ctx* c, const GridDev& g, const FdPlan& P, const float* r, void* scratch,
-                         double* phi64, float2* phi2, float* phi32) {
-  return fd_passes<float>(c, g, P, r, nullptr, scratch, nullptr, phi64, phi2, phi32);
+                         double* phi64, float2* phi2, float* phi32, const CgScalars* gate) {
+  return fd_passes<float>(c, g, P, r, nullptr, scratch, nullptr, phi64, phi2, phi32, gate);
 }
 
 template <typename T, int R, int V, class L, class E>
@@ -992,7 +998,7 @@ int launch_z_r(ofdft_ctx* c, int R, const GridDev& g, const Weights<double>& W, 
 inline int sync_scalars(ofdft_ctx* c, const void* dev, size_t bytes, void* host) {
   // through the context's pinned block: a copy to pageable memory is staged by the
   // driver (5 us more a call)
-  void* to = bytes <= 64 * sizeof(double) ? (void*)c->host_scal : host;
+  void* to = bytes <= 32 * sizeof(double) ? (void*)c->host_scal : host;
   CU(cudaMemcpyAsync(to, dev, bytes, cudaMemcpyDeviceToHost, c->stream));
   CU(cudaStreamSynchronize(c->stream));
   if (to != host) memcpy(host, to, bytes);
@@ -1003,6 +1009,26 @@ inline int sync_scalars(ofdft_ctx* c, const void* dev, size_t bytes, void* host)
 struct EvalOut {
   double sums[12];
 };
+
+// What a Poisson solve launches behind its last expected kernel, before it knows
+// whether it has converged, so that both are waited for together: launch() enqueues
+// it and the `sums` (12 doubles at c->scal) come with the solve's scalars.  done:
+// the solve ended with what launch() saw; otherwise the caller launches again.
+struct Behind {
+  std::function<int()> launch;
+  EvalOut* out = nullptr;
+  bool done = false;
+};
+
+// sync_scalars for the CG scalars and, with b, its sums.
+inline int sync_behind(ofdft_ctx* c, const CgScalars* dev, CgScalars* host, Behind* b) {
+  if (!b) return sync_scalars(c, dev, sizeof(CgScalars), host);
+  double* sums = c->host_scal + 32;
+  CU(cudaMemcpyAsync(sums, c->scal, 12 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+  TRY(sync_scalars(c, dev, sizeof(CgScalars), host));
+  memcpy(b->out->sums, sums, 12 * sizeof(double));
+  return OFDFT_OK;
+}
 
 inline void fill_energy(const EvalOut& o, double h, const ofdft_params* p, double E_self, double ezz, double eta,
                  double mu, ofdft_energy* e) {

@@ -1089,9 +1089,11 @@ struct EpiResidualFF {
   int max_it;
   int pc = 0;  // the CG that follows is preconditioned
   float2 fourpi;
+  const CgScalars* gate = nullptr;  // a round launched ahead: nothing to do when its solve is done
+  int round = 0;                    // corrections before this residual, written as sc->iters
   using Pre = float;  // u, or the explicit density
   __device__ __forceinline__ Pre prefetch(long long i) const { return rho ? rho[i] : u[i]; }
-  __device__ __forceinline__ bool skip() const { return false; }
+  __device__ __forceinline__ bool skip() const { return gate && gate->done; }
   __device__ __forceinline__ void load() {}
   __host__ __device__ __forceinline__ const float2* input(int) const { return rho ? nullptr : b2; }
   __device__ __forceinline__ void apply(long long i, float2 ph, float2 lap_raw, const float2* vin, const Pre& pre, Acc* acc) const {
@@ -1127,7 +1129,7 @@ struct EpiResidualFF {
     sc->es_rho_phi = t[3];
     sc->es_phi_r = t[4];
     sc->tol2 = tol * tol;
-    sc->iters = 0;
+    sc->iters = round;
     sc->max_it = max_it;
     sc->first = 1;
     sc->beta = 0.0;
@@ -1190,12 +1192,44 @@ static __global__ void __launch_bounds__(256) ff_prepare_kernel(long long G, con
 }
 
 // ------------------------------------------------------------- functional ---
+// 1 / d, and z = x^{-1/3} with c2 = x^{2/3}, for the functional.  In FP64 they start
+// from the FP32 functions and take one step that triples the number of correct
+// digits (from e = 1 - d r: r += r (e + e^2); from e = 1 - x z^3, the binomial series
+// of (1 - e)^{-1/3}: z += z (e/3 + 2 e^2/9)): 3 and 6 FP64 operations, within a unit
+// in the last place.  Arguments whose seed FP32 could not hold take CUDA's functions.
+// In FP32, where CUDA's functions cost little and z is slower to come by (132 against
+// 125 us at 192^3), z is not formed.
+__device__ __forceinline__ float func_rcp(float d) { return 1.0f / d; }
+__device__ __forceinline__ double func_rcp(double d) {
+  if (!(d > 1e-30 && d < 1e30)) return 1.0 / d;
+  const double r = double_of_float(__fdividef(1.0f, ff_of_double(d).x));
+  const double e = fma(-d, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+__device__ __forceinline__ void func_roots(float x, float& z, float& c2) {
+  const float c = cbrtf(x);
+  c2 = c * c;
+  z = 0.0f;
+}
+__device__ __forceinline__ void func_roots(double x, double& z, double& c2) {
+  if (x > 1e-30 && x < 1e30) {
+    z = double_of_float(rcbrtf(ff_of_double(x).x));
+    const double e = fma(-x, (z * z) * z, 1.0);
+    z = fma(z, e * fma(e, 2.0 / 9.0, 1.0 / 3.0), z);
+    c2 = x * z;
+  } else {
+    const double c = cbrt(x);
+    c2 = c * c;
+    z = x > 0.0 ? 1.0 / c : 0.0;
+  }
+}
+
 // LDA exchange-correlation of Sec. 2 / Sec. 3 (Ceperley-Alder form), density
-// floor u^2 < 1e-30 -> 0.  c13 = u^(2/3) = rho^(1/3) is passed in (the caller
-// already has cbrt(u) for the Thomas-Fermi term); one reciprocal per branch
-// replaces the divisions.
+// floor u^2 < 1e-30 -> 0.  rho13 = u^{2/3} = rho^{1/3} and (FP64) z = |u|^{-1/3} come from
+// the caller's Thomas-Fermi term; with z the Wigner-Seitz radius
+// r_s = (3/(4 pi))^{1/3} z^2 and its root need neither a quotient nor a square root.
 template <typename T>
-__device__ __forceinline__ void xc_eval(T u, T rho13, T& eps, T& v) {
+__device__ __forceinline__ void xc_eval(T u, T z, T rho13, T& eps, T& v) {
   const T rho = u * u;
   if (!(rho >= (T)1e-30)) {
     eps = T(0);
@@ -1207,11 +1241,13 @@ __device__ __forceinline__ void xc_eval(T u, T rho13, T& eps, T& v) {
   const T c3pi = (T)0.98474502184269641;  // (3/pi)^{1/3}
   const T ex = (T)-0.75 * c3pi * rho13;
   const T vx = -c3pi * rho13;
-  const T rs = (T)0.62035049089940009 / rho13;  // (3/(4 pi))^{1/3} / rho^{1/3}
+  constexpr bool wide = sizeof(T) == 8;
+  const T k1 = (T)0.62035049089940002;  // (3/(4 pi))^{1/3}
+  const T rs = wide ? k1 * (z * z) : k1 / rho13;
   T ec, vc;
   if (rs >= T(1)) {
-    const T srs = sqrt(rs);
-    const T iden = T(1) / (T(1) + b1 * srs + b2 * rs);
+    const T srs = wide ? (T)0.78762331789974325 * z : sqrt(rs);  // (3/(4 pi))^{1/6} z
+    const T iden = func_rcp(T(1) + b1 * srs + b2 * rs);
     ec = g1 * iden;
     vc = (g1 + (T)(7.0 / 6.0) * g1 * b1 * srs + (T)(4.0 / 3.0) * g1 * b2 * rs) * (iden * iden);
   } else {
@@ -1221,10 +1257,6 @@ __device__ __forceinline__ void xc_eval(T u, T rho13, T& eps, T& v) {
   }
   eps = ex + ec;
   v = vx + vc;
-}
-template <typename T>
-__device__ __forceinline__ void xc_eval(T u, T& eps, T& v) {
-  xc_eval<T>(u, cbrt(u * u), eps, v);
 }
 
 struct FuncScalars {
@@ -1296,8 +1328,8 @@ struct EpiFunctional {
     const bool tf = f.terms & 1, vw = f.terms & 2, xc = f.terms & 4, es = f.terms & 8;
     const T ux = fabs(uc);
     T vk = T(0), vxc = T(0), exc = T(0), ph = T(0);
-    const T c = (tf || xc) ? cbrt(ux) : T(0);
-    const T c2 = c * c;  // u^(2/3) = rho^(1/3)
+    T zr = T(0), c2 = T(0);  // |u|^{-1/3} (FP64), u^{2/3} = rho^{1/3}
+    if (tf || xc) func_roots(ux, zr, c2);
     if (tf) {
       const T u43 = c2 * c2;
       vk = vk_ * u43;
@@ -1305,7 +1337,7 @@ struct EpiFunctional {
     }
     if (vw) acc[1].add(uc, lap);
     if (xc) {
-      xc_eval<T>(ux, c2, exc, vxc);
+      xc_eval<T>(ux, zr, c2, exc, vxc);
       acc[2].add(exc, ux * ux);
     }
     if (es) {
@@ -1328,7 +1360,7 @@ struct EpiFunctional {
     T md = kin + T(2) * (vxc + ph + mult);
     md = fmax(md, (T)0.25 * kin);
     md = fmax(md, (T)1e-10);
-    const T inv = T(1) / md;
+    const T inv = func_rcp(md);
     const T sx = -gx * inv;
     const T wv = uc * inv;
     if (G) G[i] = gx;
@@ -2561,11 +2593,10 @@ __global__ void __launch_bounds__(256) lm_precond_kernel(long long G, T* g, T* s
   for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < G; i += (long long)gridDim.x * 256) {
     const T uc = u[i], ux = fabs(uc);
     T vk = T(0), vxc = T(0), exc = T(0);
-    if (tf) {
-      const T c = cbrt(ux);
-      vk = (T)(5.0 / 3.0 * f.CF) * ((c * c) * (c * c));
-    }
-    if (xc) xc_eval<T>(ux, exc, vxc);
+    T zr = T(0), c2 = T(0);
+    if (tf || xc) func_roots(ux, zr, c2);
+    if (tf) vk = (T)(5.0 / 3.0 * f.CF) * (c2 * c2);
+    if (xc) xc_eval<T>(ux, zr, c2, exc, vxc);
     const T ph = es ? phi[i] : T(0);
     const T gi = fma(T(-2) * eta, uc, g[i]);
     const T kin = (vw ? (T)f.kin_vw : T(0)) + (T)(14.0 / 3.0) * vk;

@@ -68,7 +68,8 @@ def test_poisson_returns_the_known_field(ctx, dims, order, dtype):
     st = ctx.poisson(g, order, phi, rho=torch.as_tensor(rho, device=DEV), tol=tol)
     cnt = ctx.counters()
     assert st.rel_residual <= tol
-    assert cnt.kind_launches[F.K_MG] == 5 * st.iterations  # five passes a step or correction
+    n = cnt.kind_launches[F.K_MG]  # five passes a step or correction, some launched ahead
+    assert n % 5 == 0 and 5 * st.iterations <= n <= 5 * (st.iterations + 1)
     assert st.iterations <= 6  # V-cycles: 17 to 35
     w = np.abs(O.lap_weights(order // 2, 1.0))
     lam_max, lam_min = 12.0 * w[1:].sum(), 1.5 * (np.pi / (max(dims) + 1)) ** 2
