@@ -836,6 +836,7 @@ int poisson_mixed(ofdft_ctx* c, int R, const GridDev& g, double h, const float* 
   float* r32 = vec<float>(c, V_R);
   float* e32 = vec<float>(c, V_E32);
   const int pb = pointwise_blocks(c, g.G);
+  const int nb8 = (int)std::min<long long>((g.G + 1023) / 1024, 8LL * c->sms);
   MgPlan mg;
   TRY(mg_prepare<float>(c, g, R, h, &mg));
   int total = 0, rc = OFDFT_OK;
@@ -858,11 +859,17 @@ int poisson_mixed(ofdft_ctx* c, int R, const GridDev& g, double h, const float* 
     const bool split_b = b2 && !(b2_valid && *b2_valid);
     {
       ProfScope ps_(c, OFDFT_K_VECTOR);
-      const int nb = (int)std::min<long long>((g.G + 1023) / 1024, 8LL * c->sms);
-      ff_prepare_kernel<<<nb, 256, 0, c->stream>>>(g.G, from.from64 ? from.from64 : phi64, from.line0, from.t,
-                                                   from.fp32 ? phi32 : nullptr, phi64, phi2,
-                                                   (direct && !from.fp32) ? phi32 : nullptr,
-                                                   split_b ? b2 : nullptr, b64, from.b32);
+      const double* in = from.from64 ? from.from64 : phi64;
+      float* out32 = (direct && !from.fp32) ? phi32 : nullptr;
+      if (!from.fp32 && !split_b && g.G % 2 == 0 && ((uintptr_t)phi32 & 7u) == 0) {
+        const double2* o2 = reinterpret_cast<const double2*>(from.line0);
+        (from.line0 ? ff_prepare2_kernel<true> : ff_prepare2_kernel<false>)<<<nb8, 256, 0, c->stream>>>(
+            g.G / 2, reinterpret_cast<const double2*>(in), o2, from.t, reinterpret_cast<double2*>(phi64),
+            reinterpret_cast<float4*>(phi2), reinterpret_cast<float2*>(out32));
+      } else {
+        ff_prepare_kernel<<<nb8, 256, 0, c->stream>>>(g.G, in, from.line0, from.t, from.fp32 ? phi32 : nullptr, phi64,
+                                                      phi2, out32, split_b ? b2 : nullptr, b64, from.b32);
+      }
     }
     CU(cudaGetLastError());
     if (split_b && b2_valid) *b2_valid = 1;

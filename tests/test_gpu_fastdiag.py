@@ -148,6 +148,23 @@ def test_batched_passes_do_not_depend_on_the_mix(ctx, prec):
     bt.close()
 
 
+@pytest.mark.parametrize("dims", [(45, 35, 37), (44, 36, 38)])
+def test_mixed_ground_state_with_odd_and_even_node_counts(ctx, dims):
+    """The passes that prepare the potential and add a correction take two nodes a
+    lane only where the node count is even: a ground state either way is the V-cycle
+    form's (tolerance as in the batch test above: a tenth of it is E's own error)."""
+    from paper_1405_6456_gb300 import workloads as W
+    c = W.tiny_cluster("dimer", h=0.6, fd_order=8)
+    p = F.default_params(fd_order=8, precision=F.PREC_MIXED, tol_E=1e-7, tol_inner=1e-8)
+    g = F.make_grid(*dims, 0.6, tuple(-0.3 * k for k in dims))
+    E, _, st = ctx.solve(c.R, c.Z, c.h, p, grid=g)
+    cv = _context(OFDFT_FD=0)
+    Ev, _, sv = cv.solve(c.R, c.Z, c.h, p, grid=g)
+    cv.close()
+    assert st.converged and sv.converged
+    assert abs(E - Ev) / c.M <= 1e-7
+
+
 def test_mixed_corrections_hand_over_to_cg_at_the_rounding_floor(ctx):
     """A tolerance below what float-float residuals resolve: the direct corrections
     stop halving the residual, the CG form takes over, and the call ends with
