@@ -1752,12 +1752,12 @@ int launch_force_boxes(ofdft_ctx* c, const GridDev& g, const AtomArgs& A, int a0
 template <typename T, int R>
 int launch_force_ball(ofdft_ctx* c, const GridDev& g, const AtomArgs& A, int a0, int na, int bdim, int box,
                       const int* lo, const Weights<double>& W, const Weights<double>& Wt, const double* bbox,
-                      const T* phi, int exact, double* partial, int nblk) {
+                      const double* vbox, int vdim, const T* phi, int exact, double* partial, int nblk) {
   TRY(atom_smem_attr(c, (const void*)force_ball_kernel<T, R>));
   {
     ProfScope ps_(c, OFDFT_K_ATOMS);
-    force_ball_kernel<T, R><<<dim3(nblk, na), 256, kGtabBytes + 3 * box * sizeof(double), c->stream>>>(g, A, a0, bdim, box, lo, W, Wt, bbox, phi, exact,
-                                                                    partial);
+    force_ball_kernel<T, R><<<dim3(nblk, na), 256, kGtabBytes + 3 * box * sizeof(double), c->stream>>>(
+        g, A, a0, bdim, box, lo, W, Wt, bbox, vbox, vdim, phi, exact, partial);
   }
   CU(cudaGetLastError());
   return OFDFT_OK;
@@ -1805,6 +1805,7 @@ int device_forces(ofdft_ctx* c, const ofdft_grid* gr, int R, const double* R_hos
         lo[3 * a + d] = (int)floor((R_host[3 * (a0 + a) + d] - gr->origin[d]) / h - 0.5) - rb + 1;
     CU(cudaMemcpyAsync(lo_dev, lo.data(), 3 * na * sizeof(int), cudaMemcpyHostToDevice, c->stream));
     if (kept) bbox = vec<double>(c, V_BTAB) + (size_t)a0 * bper;
+    const double* vtab = (!exact && !kept) ? vbox : nullptr;
     if (!exact && !kept) {
       switch (R) {
         case 1: TRY((launch_force_boxes<T, 1>(c, g, A, a0, na, vdim, bdim, lo_dev, W, vbox, bbox))); break;
@@ -1816,12 +1817,12 @@ int device_forces(ofdft_ctx* c, const ofdft_grid* gr, int R, const double* R_hos
       }
     }
     switch (R) {
-      case 1: TRY((launch_force_ball<T, 1>(c, g, A, a0, na, bdim, box, lo_dev, W, Wt, bbox, phi, exact, partial, nblk))); break;
-      case 2: TRY((launch_force_ball<T, 2>(c, g, A, a0, na, bdim, box, lo_dev, W, Wt, bbox, phi, exact, partial, nblk))); break;
-      case 3: TRY((launch_force_ball<T, 3>(c, g, A, a0, na, bdim, box, lo_dev, W, Wt, bbox, phi, exact, partial, nblk))); break;
-      case 4: TRY((launch_force_ball<T, 4>(c, g, A, a0, na, bdim, box, lo_dev, W, Wt, bbox, phi, exact, partial, nblk))); break;
-      case 5: TRY((launch_force_ball<T, 5>(c, g, A, a0, na, bdim, box, lo_dev, W, Wt, bbox, phi, exact, partial, nblk))); break;
-      case 6: TRY((launch_force_ball<T, 6>(c, g, A, a0, na, bdim, box, lo_dev, W, Wt, bbox, phi, exact, partial, nblk))); break;
+      case 1: TRY((launch_force_ball<T, 1>(c, g, A, a0, na, bdim, box, lo_dev, W, Wt, bbox, vtab, vdim, phi, exact, partial, nblk))); break;
+      case 2: TRY((launch_force_ball<T, 2>(c, g, A, a0, na, bdim, box, lo_dev, W, Wt, bbox, vtab, vdim, phi, exact, partial, nblk))); break;
+      case 3: TRY((launch_force_ball<T, 3>(c, g, A, a0, na, bdim, box, lo_dev, W, Wt, bbox, vtab, vdim, phi, exact, partial, nblk))); break;
+      case 4: TRY((launch_force_ball<T, 4>(c, g, A, a0, na, bdim, box, lo_dev, W, Wt, bbox, vtab, vdim, phi, exact, partial, nblk))); break;
+      case 5: TRY((launch_force_ball<T, 5>(c, g, A, a0, na, bdim, box, lo_dev, W, Wt, bbox, vtab, vdim, phi, exact, partial, nblk))); break;
+      case 6: TRY((launch_force_ball<T, 6>(c, g, A, a0, na, bdim, box, lo_dev, W, Wt, bbox, vtab, vdim, phi, exact, partial, nblk))); break;
     }
     {
       ProfScope ps_(c, OFDFT_K_ATOMS);
