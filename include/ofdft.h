@@ -188,7 +188,7 @@ int ofdft_destroy(ofdft_ctx* ctx);
  *   OFDFT_PRECOND_NONE: plain CG (the oracle's iteration, iteration for
  *     iteration up to rounding).
  *   OFDFT_PRECOND_MG (default): z = M r.  On grids whose axes all have 32 to 512
- *     nodes M inverts -L_h itself, up to rounding, by diagonalising the three
+ *     nodes (256 in a batch) M inverts -L_h itself, up to rounding, by diagonalising the three
  *     axes' matrices (one CG step in FP64, one per residual correction in MIXED);
  *     on the others M is one symmetric V(1,1)-cycle of the second-order 7-point
  *     Laplacian (damped Jacobi, full weighting, trilinear

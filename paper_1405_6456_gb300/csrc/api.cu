@@ -814,7 +814,8 @@ struct MixedStart {
 // same): the residual pass writes r in FP32, and the last of the five passes adds z
 // to phi64 and rewrites the pairs and the FP32 field beside it.  No CG vectors, no
 // scalars but the residual pass's own (192^3, 12th order, from zero to 1e-8: 1,775 us
-// with a CG step in each of the two rounds, 1,241 us so).  A round that does not at least halve the
+// with a CG step in each of the two rounds, 1,241 us so; 1,094 us since the residual
+// takes fewer operations and the rounds are launched ahead).  A round that does not at least halve the
 // residual (the rounding floor, or an M that is off) hands over to the CG form.
 //
 // Otherwise r, p, q = A p and the correction e of the round are FP32; the FP64
