@@ -158,7 +158,7 @@ inline bool mg_level_fused(const ofdft_ctx* c, const MgPlan& P, int l) {
 // PCG scalars (beta, rz).  Every kernel returns at once when the solve is done.
 template <typename T>
 int mg_vcycle(ofdft_ctx* c, const MgPlan& P, const T* r, T* z, CgScalars* sc) {
-  if (P.fd.on) return fd_apply<T>(c, mg_gdev(P.d[0]), P.fd, r, z, c->v[V_T].p, sc);
+  if (P.fd.on) return fd_passes<T>(c, mg_gdev(P.d[0]), P.fd, r, z, c->v[V_T].p, sc);
   T* cb = static_cast<T*>(c->mgbuf.p);
   T* t0 = vec<T>(c, V_T);
   auto rl = [&](int l) -> T* { return l == 0 ? const_cast<T*>(r) : cb + P.off[l]; };

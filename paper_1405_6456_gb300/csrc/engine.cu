@@ -134,7 +134,7 @@ struct ofdft_batch {
   double* out = nullptr;      // per slot: 16 doubles
   std::vector<CgScalars> h_sc, h_sc32;
   std::vector<double> h_out;
-  DevArena d_tiles, d_desc, d_segs, d_ops;
+  DevArena d_tiles, d_desc, d_ops;
   std::vector<int> free_index;
   long long rounds = 0;
   // CUDA graphs of the batched CG loop: a device-side WHILE loop over one CG
@@ -1588,7 +1588,7 @@ int ofdft_batch_destroy(ofdft_batch* b) {
   cudaFree(b->sc);
   cudaFree(b->sc32);
   cudaFree(b->out);
-  for (DevArena* a : {&b->d_tiles, &b->d_desc, &b->d_segs, &b->d_ops}) cudaFree(a->p);
+  for (DevArena* a : {&b->d_tiles, &b->d_desc, &b->d_ops}) cudaFree(a->p);
   delete b;
   return OFDFT_OK;
 }

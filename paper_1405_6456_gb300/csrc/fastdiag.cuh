@@ -40,7 +40,7 @@ namespace ofd {
 constexpr int kFdTile = 16;     // outputs per warp tile
 constexpr int kFdMaxN = 512;    // longest axis: 16 warps of two tiles each
 constexpr int kFdMinN = 32;     // shortest axis (see fd_usable)
-constexpr int kFdSmem = 216 * 1024;  // dynamic shared memory limit of its kernels (n = 512, float-float: 212 KB)
+constexpr int kFdSmem = 216 * 1024;  // dynamic shared memory limit of its kernels (n = 512, float-float: 193 KB)
 
 // One axis: matrices [contraction][output], outputs padded with zeros to whole
 // tiles, the even half first (ne rows of pe) and then the odd one (no rows of po).
@@ -80,7 +80,7 @@ struct FdJob {
   int nblocks;
 };
 
-// Sum of K doubles over a block of `nt` threads (a multiple of 32, at most 512).
+// Sum of a double over a block of `nt` threads (a multiple of 32, at most 512).
 __device__ __forceinline__ double fd_block_sum(double v, double* smem, int tid, int nt) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
@@ -327,18 +327,16 @@ __device__ __forceinline__ void fd_get(const float* p, float (&v)[2]) {
 }
 
 // phi64 += z with the potential's other forms (v: phi64's old values).
-template <typename T>
-__device__ __forceinline__ void fd_correct(const FdJob& J, long long i, T z) {
-  const double v = J.phi64[i] + (sizeof(T) == 4 ? double_of_float((float)z) : (double)z);
+__device__ __forceinline__ void fd_correct(const FdJob& J, long long i, float z) {
+  const double v = J.phi64[i] + double_of_float(z);
   const float2 p = ff_of_double(v);
   J.phi64[i] = v;
   if (J.phi2) J.phi2[i] = p;
   J.phi32[i] = ff_nearest(p);
 }
-template <typename T>
-__device__ __forceinline__ void fd_correct2(const FdJob& J, long long i, double2 v, const T (&z)[2]) {
-  v.x += sizeof(T) == 4 ? double_of_float((float)z[0]) : (double)z[0];
-  v.y += sizeof(T) == 4 ? double_of_float((float)z[1]) : (double)z[1];
+__device__ __forceinline__ void fd_correct2(const FdJob& J, long long i, double2 v, const float (&z)[2]) {
+  v.x += double_of_float(z[0]);
+  v.y += double_of_float(z[1]);
   const float2 p = ff_of_double(v.x), q = ff_of_double(v.y);
   *reinterpret_cast<double2*>(J.phi64 + i) = v;
   if (J.phi2) *reinterpret_cast<float4*>(J.phi2 + i) = f4(p.x, p.y, q.x, q.y);
@@ -713,7 +711,7 @@ __device__ __forceinline__ void fd_panel(const FdJob& J, long long c0, int bid, 
           dn[GS - 1 - k] = value(e[k], el[k], -d[k], -dl[k]);
         }
       };
-      if (out) {
+      if (FF || out) {  // (only FP32 passes correct)
         constexpr int GS = 16 / (int)sizeof(T);
         const int gr = ne / GS, items = cols * gr;
 #pragma unroll 2
@@ -725,7 +723,7 @@ __device__ __forceinline__ void fd_panel(const FdJob& J, long long c0, int bid, 
           fd_store16(out + o + x, up);
           fd_store16(out + o + n - GS - x, dn);
         }
-      } else {
+      } else if constexpr (!FF) {
         // the potential's old values of four items in flight together
         const int gr = ne / 2, items = cols * gr;
         for (int q0 = tid; q0 < items; q0 += 4 * nt) {
@@ -767,9 +765,9 @@ __device__ __forceinline__ void fd_panel(const FdJob& J, long long c0, int bid, 
             dl = i < no ? sg * pl[c * P + oo + i] : 0.0f;
           }
           const T v = value(ph[c * P + i], el, d, dl);
-          if (out)
+          if (FF || out)
             out[o + x] = v;
-          else
+          else if constexpr (!FF)
             fd_correct(J, o + x, v);
         }
       }

@@ -389,7 +389,7 @@ ZShape zshape(ofdft_ctx* c, const GridDev& g, int blocks_per_sm = 2, int force_n
     double least = 1e300;
     for (int zc = g.n3; zc >= 1; --zc) {
       const int nz = (g.n3 + zc - 1) / zc;
-            const long long blocks = tiles * nz, wave = (long long)c->sms * per_sm;
+      const long long blocks = tiles * nz, wave = (long long)c->sms * per_sm;
       const long long last = blocks % wave;
       double cost = (double)(blocks / wave) * (1.0 + a * (per_sm - 1));
       if (last) cost += 1.0 + a * (double)((last + c->sms - 1) / c->sms - 1);
@@ -814,7 +814,9 @@ int fd_pass(ofdft_ctx* c, const FdJob& J) {
   return tpw == 1 ? fd_launch<T, XAX, MODE, LO, 1>(c, J, warps) : fd_launch<T, XAX, MODE, LO, 2>(c, J, warps);
 }
 
-// The five passes: z = M r, or (phi64 given) phi64 += M r with its other forms.
+// The five passes: z = M r with r.z and the PCG scalars as the V-cycle's last pass
+// forms them, or (phi64 given) phi64 += M r with its other forms.  scratch:
+// fd_scratch(g) elements of T.
 template <typename T>
 int fd_passes(ofdft_ctx* c, const GridDev& g, const FdPlan& P, const T* r, T* z, void* scratch, CgScalars* sc,
               double* phi64 = nullptr, float2* phi2 = nullptr, float* phi32 = nullptr,
@@ -833,13 +835,6 @@ int fd_passes(ofdft_ctx* c, const GridDev& g, const FdPlan& P, const T* r, T* z,
   TRY((fd_pass<T, false, FD_SOLVE>(c, job(2))));
   TRY((fd_pass<T, false, FD_INV>(c, job(3))));
   return fd_pass<T, true, FD_INV>(c, job(4));
-}
-
-// z = M r by fast diagonalisation, with r.z and the PCG scalars as the V-cycle's
-// last pass forms them.  scratch: fd_scratch(g) elements of T.
-template <typename T>
-int fd_apply(ofdft_ctx* c, const GridDev& g, const FdPlan& P, const T* r, T* z, void* scratch, CgScalars* sc) {
-  return fd_passes<T>(c, g, P, r, z, scratch, sc);
 }
 
 // One correction of a mixed Poisson solve: phi64 += M r, with its pairs and its FP32
