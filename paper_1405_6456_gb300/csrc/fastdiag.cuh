@@ -30,7 +30,10 @@
 //
 // Element types: FP32 fields compute in FP32.  FP64 fields compute in float-float
 // pairs (ff, about 2^-46 relative): 12 packed FP32 operations per multiply-add
-// against the 64 FP32 slots that one FP64 FMA costs on this GPU.
+// against the 64 FP32 slots that one FP64 FMA costs on this GPU.  Pairs have FP32's
+// exponents, so the first pass divides r by 2^k ~ ||r|| (from the CG's r.r) and the
+// last one, and r.z, put 2^k back: integer operations on the exponents, exact, and
+// a source of any size FP64 holds is solved alike.
 #pragma once
 
 #include "kernels.cuh"
@@ -73,7 +76,8 @@ struct FdJob {
   int vec;          // x axis: n1 a multiple of 8 and r, z on 16 bytes: rows move as whole vectors
   const float *mx, *my, *mz;     // eigenvalues of h^2 T by axis
   const float *mxl, *myl, *mzl;  // ... low parts
-  double ih2;       // 1 / h^2
+  float2 h2;        // h^2 = h2 2^eh
+  int eh;           // (0 for FP32 fields)
   CgScalars* sc;    // the CG this serves (NULL: none; r.z is then not formed)
   const CgScalars* gate;  // a correction launched ahead: nothing to do when its solve is done
   RedBuf red;       // z: r.z
@@ -279,6 +283,11 @@ __device__ __forceinline__ void fd_contract(FdAcc<FF> (&acc)[4][CT], const FdRin
     for (int c = 0; c < CT; ++c) acc[q][c].finish();
 }
 
+// k with 2^k <= ||r|| < 2^(k+1) for the residual r the job reads (0: no CG).
+__device__ __forceinline__ int fd_exponent(const CgScalars* sc) {
+  return sc ? ((int)(((unsigned)__double2hiint(sc->rr) >> 20) & 0x7ffu) - 1023) >> 1 : 0;
+}
+
 // Float-float helpers on single values.
 __device__ __forceinline__ float2 fd_ff_add(float2 a, float2 b) {
   const float2 s = ff_two_sum(a.x, b.x);
@@ -370,6 +379,7 @@ __device__ __forceinline__ void fd_panel(const FdJob& J, long long c0, int bid, 
   // ---- the panel into shared memory (forwards: sums and differences) ----
   if constexpr (XAX && MODE == FD_FWD) {
     const T* src = static_cast<const T*>(J.in);
+    const int ke = FF ? fd_exponent(J.sc) : 0;
     if (J.vec) {
       constexpr int GS = 16 / (int)sizeof(T);  // elements of a lane's 16 bytes
       const int gr = ne / GS;                  // groups of a half row
@@ -386,7 +396,7 @@ __device__ __forceinline__ void fd_panel(const FdJob& J, long long c0, int bid, 
 #pragma unroll
         for (int k = 0; k < GS; ++k) {
           if constexpr (FF) {
-            const float2 fa = ff_of_double(a[k]), fb = ff_of_double(b[GS - 1 - k]);
+            const float2 fa = ff_of_double(a[k], ke), fb = ff_of_double(b[GS - 1 - k], ke);
             const float2 sv = fd_ff_add(fa, fb), dv = fd_ff_add(fa, fd_neg(fb));
             s[k] = sv.x, sl[k] = sv.y, d[k] = dv.x, dl[k] = dv.y;
           } else {
@@ -413,7 +423,7 @@ __device__ __forceinline__ void fd_panel(const FdJob& J, long long c0, int bid, 
           if (ok && x < no) b = src[o + n - 1 - x];
           float2 s, d;
           if constexpr (FF) {
-            const float2 fa = ff_of_double(a), fb = ff_of_double(b);
+            const float2 fa = ff_of_double(a, ke), fb = ff_of_double(b, ke);
             s = fd_ff_add(fa, fb);
             d = fd_ff_add(fa, fd_neg(fb));
           } else {
@@ -607,8 +617,7 @@ __device__ __forceinline__ void fd_panel(const FdJob& J, long long c0, int bid, 
     const long long col = c0 + cl;
     const bool ok = col < J.ncols;
     const int kx = ok ? (int)(col % J.pitch) : 0, ky = ok ? (int)(col / J.pitch) : 0;
-    const double hh = 1.0 / J.ih2;
-    const float2 h2 = make_float2((float)hh, (float)(hh - (double)(float)hh));
+    const float2 h2 = J.h2;
     DotAcc<float> dot;
 #pragma unroll
     for (int t = 0; t < TPW; ++t) {
@@ -668,6 +677,7 @@ __device__ __forceinline__ void fd_panel(const FdJob& J, long long c0, int bid, 
         for (int b = tid; b < J.nblocks; b += nt) s += __ldcg(&J.red.partials[b]);
         s = fd_block_sum(s, dsm, tid, nt);
         if (tid == 0) {
+          if constexpr (FF) s = scalbn(s, 2 * fd_exponent(J.sc) + J.eh);
           MgFin{J.sc}(&s);
           *J.red.counter = 0u;
         }
@@ -684,10 +694,11 @@ __device__ __forceinline__ void fd_panel(const FdJob& J, long long c0, int bid, 
   // ---- f_i and f_{n-1-i} from the even and odd parts ----
   if constexpr (XAX) {
     T* out = static_cast<T*>(J.out);
+    const int kz = FF ? fd_exponent(J.sc) + J.eh : 0;
     auto value = [&](float e, float el, float d, float dl) -> T {
       if constexpr (FF) {
         const float2 v = fd_ff_add(make_float2(e, el), make_float2(d, dl));
-        return (double)v.x + (double)v.y;
+        return double_of_float(v.x, kz) + double_of_float(v.y, kz);
       } else {
         return e + d;
       }

@@ -431,7 +431,7 @@ struct FdPlan {
   FdAxis ax[3];                       // x, y, z
   const float *mu[3], *mul[3];        // eigenvalues of h^2 T, high and low parts
   int pitch = 0;                      // floats of a scratch row
-  double ih2 = 0.0;
+  double h2 = 0.0;                    // h^2
 };
 
 // Multigrid preconditioner of the Poisson CG (S3): the levels of a grid (kernels
@@ -748,7 +748,7 @@ inline int fd_plan(ofdft_ctx* c, const GridDev& g, int R, double h, FdPlan* P) {
     P->mul[d] = d == 0 ? t->mxl : t->mul;
   }
   P->pitch = fd_pitch(g.n1);
-  P->ih2 = 1.0 / (h * h);
+  P->h2 = h * h;
   P->on = true;
   return OFDFT_OK;
 }
@@ -770,7 +770,8 @@ FdJob fd_job(const GridDev& g, const FdPlan& P, int p, const T* r, T* z, void* s
   J.cs = (long long)P.pitch * g.n2;
   J.mx = P.mu[0], J.my = P.mu[1], J.mz = P.mu[2];
   J.mxl = P.mul[0], J.myl = P.mul[1], J.mzl = P.mul[2];
-  J.ih2 = P.ih2;
+  const double h2 = sizeof(T) == 8 ? frexp(P.h2, &J.eh) : P.h2;
+  J.h2 = make_float2((float)h2, (float)(h2 - (double)(float)h2));
   J.vec = g.n1 % 8 == 0 && (((uintptr_t)r | (uintptr_t)z) & 15u) == 0;
   J.sc = sc;
   return J;

@@ -99,6 +99,26 @@ __device__ __forceinline__ double double_of_float(float f) {
   if (e - 1u < 254u) return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
   return (double)f;
 }
+// The same of v 2^-k (|k| <= 512), and of f 2^k (|k| <= 2000), exactly: the exponents
+// move in the integer operations.
+__device__ __forceinline__ float2 ff_of_double(double v, int k) {
+  const unsigned h = (unsigned)__double2hiint(v), l = (unsigned)__double2loint(v);
+  const unsigned e = ((h >> 20) & 0x7ffu) - (unsigned)k;
+  if (e - 953u < 197u) {
+    const unsigned sign = h & 0x80000000u;
+    const float hi = __uint_as_float(((e - 896u) << 23) | ((h & 0xfffffu) << 3) | (l >> 29) | sign);
+    const float sc = __uint_as_float(((e - 948u) << 23) | sign);
+    return make_float2(hi, (float)(l & 0x1fffffffu) * sc);
+  }
+  return ff_of_double(v * __hiloint2double((1023 - k) << 20, 0));
+}
+__device__ __forceinline__ double double_of_float(float f, int k) {
+  const unsigned b = __float_as_uint(f), e = (b >> 23) & 0xffu, d = e + 896u + (unsigned)k;
+  if (e - 1u < 254u && d - 1u < 2046u)
+    return __hiloint2double((int)((b & 0x80000000u) | (d << 20) | ((b & 0x7fffffu) >> 3)), (int)(b << 29));
+  const int k1 = max(min(k, 1000), -1000);  // zeros, and what one of the formats holds with fewer bits
+  return (double)f * __hiloint2double((1023 + k1) << 20, 0) * __hiloint2double((1023 + k - k1) << 20, 0);
+}
 // The float nearest a pair's value.
 __device__ __forceinline__ float ff_nearest(float2 a) { return a.x + a.y; }
 

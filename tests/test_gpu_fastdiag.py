@@ -185,3 +185,21 @@ def test_mixed_corrections_hand_over_to_cg_at_the_rounding_floor(ctx):
     cv.close()
     # both at their floors: equal to FP32 rounding (2^-24 each, doubled)
     assert np.linalg.norm(sols[0] - sols[1]) <= 2.0**-22 * np.linalg.norm(sols[1])
+
+
+@pytest.mark.parametrize("ke,kh", [(-300, 0), (-80, 0), (80, 0), (300, 0), (0, -100), (0, 100), (-200, 60)])
+def test_fp64_solves_do_not_depend_on_scale(ctx, ke, kh):
+    """Sources and spacings scaled by powers of two far outside FP32's range: every
+    operation of the solve scales exactly, so potential and steps are the unscaled
+    ones bit for bit (phi ~ rho h^2)."""
+    dims, order = (36, 40, 33), 12
+    rho = np.random.default_rng(6).standard_normal(dims[::-1])
+
+    def solve(ke, kh):
+        g = F.make_grid(*dims, float(np.ldexp(0.6, kh)))
+        phi = torch.zeros(g.shape, dtype=torch.float64, device=DEV)
+        st = ctx.poisson(g, order, phi, rho=torch.as_tensor(np.ldexp(rho, ke), device=DEV), tol=1e-10, max_it=50)
+        return np.ldexp(phi.cpu().numpy(), -ke - 2 * kh), st.iterations
+
+    (p0, it0), (p1, it1) = solve(0, 0), solve(ke, kh)
+    assert it0 == it1 and np.array_equal(p0, p1)
