@@ -1767,6 +1767,10 @@ int launch_force_ball(ofdft_ctx* c, const GridDev& g, const AtomArgs& A, int a0,
 template <typename T>
 int device_forces(ofdft_ctx* c, const ofdft_grid* gr, int R, const double* R_host, const double* Z_host, int M,
                   double sigma, double rc, int variant, const T* phi, double* F) {
+  if (!(rc > 0.0)) {  // balls without nodes
+    std::fill(F, F + 3 * (size_t)M, 0.0);
+    return OFDFT_OK;
+  }
   AtomArgs A;
   TRY(upload_atoms(c, R_host, Z_host, M, &A, gr, sigma, rc));
   const GridDev g = gdev(gr);

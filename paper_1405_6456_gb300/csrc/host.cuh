@@ -1084,8 +1084,9 @@ inline const std::vector<double>& gtab_host() {
   return tab;
 }
 // The smallest d2 whose rounded square root is not below rc: r < rc is d2 < rc2
-// exactly, without a square root per node.
+// exactly, without a square root per node.  No distance is below an rc <= 0.
 inline double sq_threshold(double rc) {
+  if (!(rc > 0.0)) return 0.0;
   double x = rc * rc;
   while (sqrt(x) >= rc) x = nextafter(x, 0.0);
   while (sqrt(x) < rc) x = nextafter(x, INFINITY);

@@ -3089,10 +3089,12 @@ __device__ __forceinline__ void gtab_load(double* sm, const double* __restrict__
        i += blockDim.x * blockDim.y * blockDim.z)
     sm[i] = tab[i];
 }
-// V at squared distance d2; is2 = 1/sigma^2, zs = -Z/sigma
-__device__ __forceinline__ double gtab_v(const double* tab, double d2, double is2, double zs, double sigma) {
+// V at squared distance d2; is2 = 1/sigma^2, zs = -Z/sigma; zr / r is V far away
+// (-Z, by sigma's sign), and everywhere for sigma = 0, a point charge
+__device__ __forceinline__ double gtab_far(double Z, double sigma) { return sigma < 0.0 ? Z : -Z; }
+__device__ __forceinline__ double gtab_v(const double* tab, double d2, double is2, double zs, double zr) {
   const double u = fma(d2, is2, 1.0);
-  if (!(u < 512.0)) return zs * sigma / sqrt(d2);
+  if (!(u < 512.0)) return zr / sqrt(d2);
   const int hi = __double2hiint(u);
   const int k = (hi >> 14) - (0x3ff00000 >> 14);
   const double t = u - __hiloint2double((hi & ~0x3fff) | 0x2000, 0);
@@ -3320,7 +3322,7 @@ static __global__ void __launch_bounds__(256) force_vbox_kernel(AtomArgs A, int 
   gtab_load(atom_sm, A.gtab);
   box_squares(q, vdim, bl, Rj, A.h, og);
   __syncthreads();
-  const double is2 = 1.0 / (A.sigma * A.sigma), zs = -A.Z[J] / A.sigma;
+  const double is2 = 1.0 / (A.sigma * A.sigma), zs = -A.Z[J] / A.sigma, zr = gtab_far(A.Z[J], A.sigma);
   double* out = vbox + (size_t)a * per;
   auto ijk = [&](unsigned e, int& i, int& j, int& k) {
     const unsigned jk = e / (unsigned)vdim;
@@ -3340,7 +3342,7 @@ static __global__ void __launch_bounds__(256) force_vbox_kernel(AtomArgs A, int 
                  int i, j, k;
                  ijk(e, i, j, k);
                  const double d2 = __dadd_rn(__dadd_rn(q[i], q[vdim + j]), q[2 * vdim + k]);
-                 out[e] = gtab_v(atom_sm, d2, is2, zs, A.sigma);
+                 out[e] = gtab_v(atom_sm, d2, is2, zs, zr);
                });
 }
 
@@ -3505,7 +3507,7 @@ __global__ void __launch_bounds__(256) force_ball_kernel(GridDev g, AtomArgs A, 
   gtab_load(atom_sm, A.gtab);
   box_squares(qd, box, lo + 3 * a, Rj, A.h, og);
   __syncthreads();
-  const double is2 = 1.0 / (A.sigma * A.sigma), zs = -A.Z[J] / A.sigma;
+  const double is2 = 1.0 / (A.sigma * A.sigma), zs = -A.Z[J] / A.sigma, zr = gtab_far(A.Z[J], A.sigma);
   double acc[3] = {0.0, 0.0, 0.0};
   auto ijk = [&](unsigned t, int& i, int& j, int& k) {
     const unsigned jk = t / (unsigned)box;
@@ -3529,7 +3531,7 @@ __global__ void __launch_bounds__(256) force_ball_kernel(GridDev g, AtomArgs A, 
     // atoms at h = 0.45 in 2,000 us, 2,081 us with V_J formed again), else evaluated
     const long long vd = vdim;
     const double vj = vbox ? vbox[((a * vd + k + 2 * R) * vd + j + 2 * R) * vd + i + 2 * R]
-                           : gtab_v(atom_sm, d2, is2, zs, A.sigma);
+                           : gtab_v(atom_sm, d2, is2, zs, zr);
     const double pv = (double)phi[lin(g, gi, gj, gk)] - vj;
     double gx = 0.0, gy = 0.0, gz = 0.0;
     if (!exact) {

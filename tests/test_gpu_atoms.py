@@ -66,3 +66,24 @@ def test_initial_guess_matches_oracle(ctx, gs, cut, dims, h):
     u_ref = O.initial_guess(og, R, Z, gs, cut)
     # three exponentials multiplied against one of the sum: a few units of 2^-53
     assert np.abs(u.cpu().numpy() - u_ref).max() <= 1e-14 * np.abs(u_ref).max()
+
+
+@pytest.mark.parametrize("variant", [F.FORCE_PAPER, F.FORCE_EXACT])
+def test_forces_of_balls_without_nodes_are_zero(ctx, variant):
+    g, _, R, Z = _case((26, 21, 33), 0.6, 12)
+    phi = torch.ones(g.shape, dtype=torch.float64, device=DEV)
+    for rc in (0.0, -0.3, -1.0, -50.0):
+        assert not ctx.forces(g, 12, R, Z, phi, rc=rc, variant=variant).any()
+
+
+def test_forces_of_point_charges_and_negative_widths(ctx):
+    """ofdft_forces takes any width: sigma = 0 is V = -Z/r (as any width far below the
+    nearest node's distance), and erf is odd, so -sigma is the charge -Z."""
+    dims, h = (26, 21, 33), 0.6
+    g, og, R, Z = _case(dims, h, 12)
+    R, Z = R[:2] + 0.07, Z[:2]
+    phi = 0.01 * np.random.default_rng(3).standard_normal(g.shape)
+    for sigma, ref in ((0.0, dict(sigma=1e-3)), (-0.25, dict(sigma=0.25))):
+        Fd = ctx.forces(g, 12, R, Z, torch.as_tensor(phi, device=DEV), sigma=sigma, rc=5.0)
+        Fo = O.forces(og, 6, R, -Z if sigma < 0 else Z, phi, rc=5.0, **ref)
+        np.testing.assert_allclose(Fd, Fo, rtol=1e-10, atol=1e-11 * np.abs(Fo).max())
