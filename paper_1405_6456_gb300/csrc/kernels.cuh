@@ -3190,7 +3190,7 @@ __device__ __forceinline__ int tile_atoms(const AtomArgs& A, int a0, double cx, 
     const float dx = fmaxf(fabsf((float)(A.R[3 * a] - cx)) - hf, 0.0f);
     const float dy = fmaxf(fabsf((float)(A.R[3 * a + 1] - cy)) - hf, 0.0f);
     const float dz = fmaxf(fabsf((float)(A.R[3 * a + 2] - cz)) - hf, 0.0f);
-    hit = dx * dx + dy * dy + dz * dz < screen_r2(reach);
+    hit = dx * dx + dy * dy + dz * dz <= screen_r2(reach);  // (both may overflow: the node's test decides)
   }
   const unsigned m = __ballot_sync(0xffffffffu, hit);
   if (lane == 0) warp_cnt[warp] = __popc(m);

@@ -87,3 +87,28 @@ def test_forces_of_point_charges_and_negative_widths(ctx):
         Fd = ctx.forces(g, 12, R, Z, torch.as_tensor(phi, device=DEV), sigma=sigma, rc=5.0)
         Fo = O.forces(og, 6, R, -Z if sigma < 0 else Z, phi, rc=5.0, **ref)
         np.testing.assert_allclose(Fd, Fo, rtol=1e-10, atol=1e-11 * np.abs(Fo).max())
+
+
+@pytest.mark.parametrize("k", [-60, 66])
+def test_atom_kernels_do_not_depend_on_the_unit_of_length(ctx, k):
+    """Lengths scaled by a power of two whose squares FP32 cannot hold: the FP32 screens
+    only ever keep more, and the FP64 values scale exactly (b ~ 1/length^3, its self
+    energy ~ 1/length; the forces' sums, in another order, to rounding)."""
+    dims, h = (26, 21, 33), 0.6
+    phi = np.random.default_rng(3).standard_normal(dims[::-1])
+
+    def run(s):
+        g, _, R, Z = _case(dims, h, 12)
+        g = F.make_grid(*dims, h * s, tuple(x * s for x in g.origin))
+        b = torch.empty(g.shape, dtype=torch.float64, device=DEV)
+        es = ctx.pseudocharge(g, 12, R * s, Z, b, sigma=s, rc=7.0 * s)
+        Fd = ctx.forces(g, 12, R * s, Z, torch.as_tensor(phi / s, device=DEV), sigma=s, rc=7.0 * s)
+        u = torch.empty(g.shape, dtype=torch.float64, device=DEV)
+        ctx.initial_guess(g, R * s, Z, u, guess_sigma=2.0 * s, guess_cut=8.0 * s)
+        return b.cpu().numpy() * s**3, es * s, Fd * s**2, u.cpu().numpy() * s**1.5
+
+    (b0, e0, f0, u0), (b1, e1, f1, u1) = run(1.0), run(2.0**k)
+    assert np.array_equal(b0, b1) and e0 == pytest.approx(e1, rel=1e-14)
+    np.testing.assert_allclose(f1, f0, rtol=1e-12, atol=1e-13 * np.abs(f0).max())
+    # the guess's norm is a power, rounded apart at either scale: a few units of 2^-53
+    np.testing.assert_allclose(u1, u0, rtol=1e-14, atol=0.0)
