@@ -1157,7 +1157,9 @@ struct EpiResidualFF {
     sc->err = 0;
     sc->pc = pc;
     const double thr = tol * tol * (t[1] > 0.0 ? t[1] : 1.0);
-    sc->done = (t[2] <= thr || max_it <= 0) ? 1 : 0;
+    // (a residual that is not finite ends the solve here, so that corrections launched
+    // ahead leave the potential alone)
+    sc->done = (t[2] <= thr || max_it <= 0 || !isfinite(t[2])) ? 1 : 0;
   }
 };
 

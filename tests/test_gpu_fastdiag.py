@@ -203,3 +203,17 @@ def test_fp64_solves_do_not_depend_on_scale(ctx, ke, kh):
 
     (p0, it0), (p1, it1) = solve(0, 0), solve(ke, kh)
     assert it0 == it1 and np.array_equal(p0, p1)
+
+
+@pytest.mark.parametrize("bad", [float("nan"), float("inf"), 1e30])
+def test_mixed_solves_of_sources_that_are_not_finite_leave_the_potential(ctx, bad):
+    """The corrections are launched before the host has seen the residual: a source
+    that is not finite, or whose norm FP32 sums cannot hold, ends the call with
+    OFDFT_ENONFINITE and the caller's potential as it was."""
+    g = F.make_grid(36, 34, 33, 0.5)
+    rho = torch.ones(g.shape, dtype=torch.float32, device=DEV)
+    rho[3, 4, 5] = bad
+    phi = torch.full(g.shape, 0.25, dtype=torch.float32, device=DEV)
+    with pytest.raises(F.OfdftError, match="ENONFINITE"):
+        ctx.poisson(g, 12, phi, rho=rho, tol=1e-8)
+    assert bool((phi == 0.25).all())
