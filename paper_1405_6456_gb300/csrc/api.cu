@@ -684,12 +684,10 @@ int cg_iterate(ofdft_ctx* c, int R, const GridDev& g, double h, const Weights<do
       // one step of the directly inverted operator mostly ends the solve (every
       // kernel so far did nothing if it had ended before)
       if (cg_fold<T>(c, g)) TRY(cg_flush<T>(c, g, reinterpret_cast<T*>(x), pv, sc));
-      if (behind) TRY(behind->launch());
+      if (behind) TRY(behind->launch(sc));
       TRY(sync_behind(c, sc, host_sc, behind));
-      if (host_sc->done) {
-        if (behind) behind->done = true;
-        return OFDFT_OK;
-      }
+      if (behind) behind->ended(*host_sc);
+      if (host_sc->done) return OFDFT_OK;
     }
     cudaGraphExec_t wexec = nullptr;
     TRY((cg_while_graph<T, X>(c, R, g, h, Wneg, x, r, pv, qv, sc, pb, &wexec, &mg)));
@@ -907,8 +905,9 @@ int poisson_mixed(ofdft_ctx* c, int R, const GridDev& g, double h, const float* 
                              k > 0 ? c->sc : nullptr, k};
       TRY(launch_z_r<float2>(c, R, g, W, LoadPlain<float2>{phi2}, ep, OFDFT_K_RESIDUAL));
     }
-    if (behind) TRY(behind->launch());
+    if (behind) TRY(behind->launch(c->sc));
     TRY(sync_behind(c, c->sc, &hs, behind));
+    if (behind) behind->ended(hs);
     total += hs.iters;
     const double bb = hs.bb > 0 ? hs.bb : 1.0;
     if (c->trace) fprintf(stderr, "[ofdft] mixed direct corrections %d rel64=%.3e\n", total, sqrt(hs.rr / bb));
@@ -917,14 +916,12 @@ int poisson_mixed(ofdft_ctx* c, int R, const GridDev& g, double h, const float* 
       st->rel_residual = sqrt(hs.rr / bb);
     }
     if (!isfinite(hs.rr)) return fail(c, OFDFT_ENONFINITE, "Poisson residual is not finite");
-    if (behind) behind->done = true;  // (withdrawn where the solve goes on)
     if (hs.rr <= tol * tol * bb) break;
     if (total >= max_it || total >= max_rounds) {
       rc = fail(c, OFDFT_ENOTCONV, "mixed Poisson reached %d FP32 iterations at relative residual %.3e", total,
                 sqrt(hs.rr / bb));
       break;
     }
-    if (behind) behind->done = false;
     if (rr_old >= 0.0 && hs.rr > 0.25 * rr_old) direct = false;  // not halved: go on with CG
     rr_old = hs.rr;
     have_r = true;
@@ -1000,7 +997,8 @@ int functional_launch(ofdft_ctx* c, int R, const GridDev& g, double h, const ofd
                     const T* b, const T* phi, const T* rcg, double eta, double mu, double N,
                     const double* sum_uu_dev, T* G, T* s, const T* d, const T* s_old,
                     T* winv = nullptr, const double* phi64 = nullptr, const double* b64 = nullptr,
-                    const double* r64 = nullptr, const CgScalars* es_sums = nullptr) {
+                    const double* r64 = nullptr, const CgScalars* es_sums = nullptr,
+                    const CgScalars* gate = nullptr, bool gate_any = false) {
   const Weights<double> W = lap_weights(R, h, 1.0);
   FuncScalars f;
   f.h3 = h * h * h;
@@ -1017,6 +1015,8 @@ int functional_launch(ofdft_ctx* c, int R, const GridDev& g, double h, const ofd
   const bool split_dots = c->func_split_dots && G && (d || s_old);
   EpiFunctional<T> ep{es ? phi : nullptr, b, es ? rcg : nullptr, split_dots ? nullptr : d,
                       split_dots ? nullptr : s_old, G, s, winv, sum_uu_dev, f, c->scal};
+  ep.gate = gate;
+  ep.gate_any = gate_any;
   if (es && es_sums) {
     ep.es_sums = es_sums;
   } else if (es && phi64) {
@@ -1158,10 +1158,11 @@ struct Solver {
     // term uses that solve's residual, FP64 in MIXED)
     Behind fun;
     fun.out = &o;
-    fun.launch = [&]() {
+    fun.launch = [&](const CgScalars* gate) {
       return functional_launch<T>(c, R, g, h, p, at, b, phi, (es && !mixed) ? vec<T>(c, V_R) : nullptr, eta, mu, N,
                                   sum_uu, Gout, sout, dd, s_old, winv, mixed ? phi64 : nullptr, mixed ? b64 : nullptr,
-                                  mixed ? vec<double>(c, V_R64) : nullptr, (mixed && c->mixed_ff) ? c->sc : nullptr);
+                                  mixed ? vec<double>(c, V_R64) : nullptr, (mixed && c->mixed_ff) ? c->sc : nullptr,
+                                  gate);
     };
     if (es) {
       int rc;
@@ -1185,7 +1186,7 @@ struct Solver {
       CU(cudaGetLastError());
     }
     if (!fun.done) {
-      TRY(fun.launch());
+      TRY(fun.launch(nullptr));
       TRY(sync_scalars(c, c->scal, 12 * sizeof(double), o.sums));
     }
     stats->stencil_apps += 2;
@@ -2426,16 +2427,18 @@ int ofdft_energy_grad(ofdft_ctx* c, const ofdft_grid* g, const ofdft_params* p, 
   }
   Behind fun;  // the functional, launched behind the Poisson solve
   fun.out = &o;
-  fun.launch = [&]() -> int {
+  fun.anyway = !solve_poisson;
+  fun.launch = [&](const CgScalars* gate) -> int {
     if (!mixed)
       return functional_launch<double>(c, R, gd, g->h, p, (const double*)u, (const double*)b, (const double*)phi,
                                        es ? vec<double>(c, V_R) : nullptr, eta, mu, N, sum_uu, (double*)grad, (double*)s,
-                                       (const double*)d, (const double*)s_old, r1 ? vec<double>(c, V_W) : nullptr);
+                                       (const double*)d, (const double*)s_old, r1 ? vec<double>(c, V_W) : nullptr,
+                                       nullptr, nullptr, nullptr, nullptr, gate, fun.anyway);
     return functional_launch<float>(c, R, gd, g->h, p, (const float*)u, (const float*)b, (const float*)phi, nullptr, eta,
                                     mu, N, sum_uu, (float*)grad, (float*)s, (const float*)d, (const float*)s_old,
                                     r1 ? vec<float>(c, V_W) : nullptr, es ? vec<double>(c, V_PHI64) : nullptr,
                                     es ? vec<double>(c, V_B64) : nullptr, es ? vec<double>(c, V_R64) : nullptr,
-                                    (es && c->mixed_ff) ? c->sc : nullptr);
+                                    (es && c->mixed_ff) ? c->sc : nullptr, gate, fun.anyway);
   };
   if (es) {
     int rc;
@@ -2465,7 +2468,7 @@ int ofdft_energy_grad(ofdft_ctx* c, const ofdft_grid* g, const ofdft_params* p, 
     CU(cudaGetLastError());
   }
   if (!fun.done) {
-    TRY(fun.launch());
+    TRY(fun.launch(nullptr));
     TRY(sync_scalars(c, c->scal, 12 * sizeof(double), o.sums));
   }
   fill_energy(o, g->h, p, E_self, 0.0, eta, mu, out);

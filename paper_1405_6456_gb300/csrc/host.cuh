@@ -1007,13 +1007,19 @@ struct EvalOut {
 };
 
 // What a Poisson solve launches behind its last expected kernel, before it knows
-// whether it has converged, so that both are waited for together: launch() enqueues
-// it and the `sums` (12 doubles at c->scal) come with the solve's scalars.  done:
-// the solve ended with what launch() saw; otherwise the caller launches again.
+// whether it has converged, so that both are waited for together: launch(gate)
+// enqueues it and the `sums` (12 doubles at c->scal) come with the solve's scalars.
+// It writes nothing where the solve has not converged by then (`anyway`, for calls
+// that take the potential as it is: where the residual is not finite).  done: it
+// ran; otherwise the caller launches it again (launch(NULL)) or reports the error.
 struct Behind {
-  std::function<int()> launch;
+  std::function<int(const CgScalars* gate)> launch;
   EvalOut* out = nullptr;
+  bool anyway = false;
   bool done = false;
+  void ended(const CgScalars& s) {  // the scalars that the device's test saw
+    done = anyway ? std::isfinite(s.rr) : s.rr <= s.tol2 * (s.bb > 0.0 ? s.bb : 1.0);
+  }
 };
 
 // sync_scalars for the CG scalars and, with b, its sums.

@@ -217,3 +217,39 @@ def test_mixed_solves_of_sources_that_are_not_finite_leave_the_potential(ctx, ba
     with pytest.raises(F.OfdftError, match="ENONFINITE"):
         ctx.poisson(g, 12, phi, rho=rho, tol=1e-8)
     assert bool((phi == 0.25).all())
+
+
+@pytest.mark.parametrize("prec", [F.PREC_FP64, F.PREC_MIXED])
+def test_evaluations_whose_poisson_solve_fails_write_no_gradient(ctx, prec):
+    """The functional is launched behind the Poisson solve, before the host knows how it
+    ended: where it fails (not converged, or not finite) grad and s stay as they were; and
+    an evaluation at the potential as it is (solve_poisson=False) needs no convergence."""
+    from paper_1405_6456_gb300 import workloads as W
+    c = W.tiny_cluster("dimer", h=0.6, fd_order=8)
+    dtype = torch.float64 if prec == F.PREC_FP64 else torch.float32
+    g = F.make_grid(44, 36, 38, 0.6, (-13.2, -10.8, -11.4))
+    b, u = (torch.empty(g.shape, dtype=dtype, device=DEV) for _ in range(2))
+    Es = ctx.pseudocharge(g, 8, c.R, c.Z, b)
+    ctx.initial_guess(g, c.R, c.Z, u)
+    bad = u.clone()
+    bad[5, 6, 7] = float("nan")
+
+    def evaluate(uu, err=None, **kw):
+        grad, s = torch.full_like(u, 7.0), torch.full_like(u, 7.0)
+        solve = kw.pop("solve_poisson", True)
+        p = F.default_params(fd_order=8, precision=prec, precond_rank1=0, **kw)
+        args = (g, p, uu, b, torch.zeros_like(u), Es, 0.0, float("inf"), c.N, solve)
+        if err is None:
+            return ctx.energy_grad(*args, grad=grad, s=s), grad, s
+        with pytest.raises(F.OfdftError, match=err):
+            ctx.energy_grad(*args, grad=grad, s=s)
+        assert bool((grad == 7.0).all()) and bool((s == 7.0).all())
+
+    evaluate(u, "ENOTCONV", tol_poisson=1e-25, max_cg=1)
+    evaluate(bad, "ENONFINITE", tol_poisson=1e-8)
+    evaluate(bad, "ENONFINITE", tol_poisson=1e-8, solve_poisson=False)
+    e, grad, s = evaluate(u, tol_poisson=1e-8, solve_poisson=False)
+    # at phi = 0 the electrostatic term is absent from the gradient (and without a
+    # penalty it does not depend on sum u^2, which other passes sum in other orders)
+    e0, grad0, s0 = evaluate(u, terms=F.TERM_TF | F.TERM_VW | F.TERM_XC)
+    assert e.poisson.rel_residual > 0.5 and torch.equal(grad, grad0) and torch.equal(s, s0)
