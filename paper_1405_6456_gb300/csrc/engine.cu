@@ -912,6 +912,15 @@ struct Engine {
     return OFDFT_OK;
   }
 
+  // A solve whose tolerance lies below what the float-float residual resolves (about
+  // 1e-13) goes on with the FP64 one: its pseudocharge in FP64 again, r64 the residual's.
+  int leave_pairs(Slot<T>* S) {
+    double es = 0.0;
+    S->ff = false;
+    return device_pseudocharge<double>(c, &S->grid, S->Rr, S->R.data(), S->Z.data(), S->M, S->p.sigma, S->p.rc, S->b64,
+                                       &es);
+  }
+
   // Batched Poisson solves at each slot's evaluation point.
   int poisson(const std::vector<Slot<T>*>& ev) {
     if (ev.empty()) return OFDFT_OK;
@@ -982,8 +991,12 @@ struct Engine {
         S->pstats.rel_residual = sqrt(h.rr / bb);
         if (h.rr <= S->ev_tol * S->ev_tol * bb || S->ptotal >= S->p.max_cg || !isfinite(h.rr)) continue;
         const bool stalled = S->direct && S->rr_old >= 0.0 && h.rr > 0.25 * S->rr_old;
-        if (stalled && S->ff) continue;  // the rounding floor of the residual itself
         next.push_back(S);
+        if (stalled && S->ff) {  // the float-float residual's rounding floor: its FP64 form from here on
+          TRY(leave_pairs(S));
+          S->rr_old = -1.0;
+          continue;
+        }
         if (stalled) {  // not halved: go on with CG
           S->direct = S->fresh32 = false;
           CU(cudaMemsetAsync(S->e32, 0, S->g.G * sizeof(float), c->stream));

@@ -136,3 +136,25 @@ def test_serving_loop_results_match_solo_and_report_latency(ctx):
         assert r.latency_s > 0 and r.finish_s >= r.admit_s >= r.arrival_s - 1e-9
     s = rep.summary()
     assert s["latency_p99_s"] >= s["latency_p50_s"] > 0
+
+
+def test_batch_mixed_poisson_reaches_tolerances_below_the_float_float_floor(ctx):
+    """A Poisson tolerance that the float-float residual cannot resolve: the solve goes
+    on with the FP64 residual and reaches it, alone and beside a solve that keeps the
+    pairs, with the same result bit for bit."""
+    c = W.tiny_cluster("dimer", h=0.6, fd_order=8)
+    dims = (44, 36, 38)
+    g = F.make_grid(*dims, 0.6, tuple(-0.3 * k for k in dims))
+    ps = [F.default_params(fd_order=8, precision=F.PREC_MIXED, tol_E=1e-7, tol_inner=1e-8, tol_poisson=t,
+                           poisson_adapt=0.0) for t in (1e-14, 1e-8)]
+    out = []
+    for mix in ((0,), (0, 1)):
+        bt = F.Batch(ctx, F.PREC_MIXED, 4 * GB)
+        ids = [bt.submit(c.R, c.Z, c.h, ps[k], grid=g) for k in mix]
+        bt.run()
+        out.append([bt.poll(rid) for rid in ids])
+        bt.close()
+    for res in out:
+        for (E, Fv, st), p in zip(res, ps):
+            assert st.converged and 0.0 < st.parts.poisson.rel_residual <= p.tol_poisson
+    assert out[0][0][0] == out[1][0][0] and np.array_equal(out[0][0][1], out[1][0][1])
