@@ -78,19 +78,21 @@ __device__ __forceinline__ float2 ff_mul_lazy(float2 w, float2 a) {
 
 // A double as a float pair, and a float as a double, on the integer and FP32 pipes:
 // conversions between the two widths issue at the FP64 rate here (1/64 of FP32),
-// and the passes over the FP64 potential did little else.  ff_of_double truncates
-// hi to the double's leading 24 bits and keeps the next 24 of the other 29 in lo
-// (an error below 2^-47 of v); values outside +-[2^-70, 2^127), zero among them,
-// take the plain conversions.
-__device__ __forceinline__ float2 ff_of_double(double v) {
+// and the passes over the FP64 potential did little else.  ff_of_double(v, k) is the
+// pair of v 2^-k (|k| <= 512): hi the nearest float, lo the nearest float of the
+// rest, an error below 2^-48 of v (hi truncated, which saves two operations, doubles
+// it).  Values outside +-[2^-70, 2^127), zero among them, take the plain conversions.
+__device__ __forceinline__ float2 ff_of_double(double v, int k = 0) {
   const unsigned h = (unsigned)__double2hiint(v), l = (unsigned)__double2loint(v);
-  const unsigned e = (h >> 20) & 0x7ffu;
-  if (e - 953u < 197u) {  // 2^-70 <= |v| < 2^127
-    const unsigned sign = h & 0x80000000u;
-    const float hi = __uint_as_float((((h << 3) | (l >> 29)) ^ 0x40000000u) & 0x7fffffffu | sign);
+  const unsigned e = ((h >> 20) & 0x7ffu) - (unsigned)k;
+  if (e - 953u < 197u) {  // 2^-70 <= |v| 2^-k < 2^127
+    const unsigned sign = h & 0x80000000u, r = l + 0x10000000u;  // half a unit of hi; the carry may move the exponent
+    const unsigned m = ((h + (r < l ? 1u : 0u)) << 3 | (r >> 29)) - ((896u + (unsigned)k) << 23);
+    const float hi = __uint_as_float((m & 0x7fffffffu) | sign);
     const float sc = __uint_as_float(((e - 948u) << 23) | sign);  // +-2^(e - 1075): the unit of l
-    return make_float2(hi, (float)(l & 0x1fffffffu) * sc);
+    return make_float2(hi, (float)((int)(l << 3) >> 3) * sc);     // l's 29 bits below hi, as a signed remainder
   }
+  if (k != 0) v *= __hiloint2double((1023 - k) << 20, 0);
   const float hi = (float)v;
   return make_float2(hi, isfinite(hi) ? (float)(v - (double)hi) : 0.0f);
 }
@@ -99,19 +101,7 @@ __device__ __forceinline__ double double_of_float(float f) {
   if (e - 1u < 254u) return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
   return (double)f;
 }
-// The same of v 2^-k (|k| <= 512), and of f 2^k (|k| <= 2000), exactly: the exponents
-// move in the integer operations.
-__device__ __forceinline__ float2 ff_of_double(double v, int k) {
-  const unsigned h = (unsigned)__double2hiint(v), l = (unsigned)__double2loint(v);
-  const unsigned e = ((h >> 20) & 0x7ffu) - (unsigned)k;
-  if (e - 953u < 197u) {
-    const unsigned sign = h & 0x80000000u;
-    const float hi = __uint_as_float(((e - 896u) << 23) | ((h & 0xfffffu) << 3) | (l >> 29) | sign);
-    const float sc = __uint_as_float(((e - 948u) << 23) | sign);
-    return make_float2(hi, (float)(l & 0x1fffffffu) * sc);
-  }
-  return ff_of_double(v * __hiloint2double((1023 - k) << 20, 0));
-}
+// f 2^k (|k| <= 2000), the exponent moved in the integer operations
 __device__ __forceinline__ double double_of_float(float f, int k) {
   const unsigned b = __float_as_uint(f), e = (b >> 23) & 0xffu, d = e + 896u + (unsigned)k;
   if (e - 1u < 254u && d - 1u < 2046u)
