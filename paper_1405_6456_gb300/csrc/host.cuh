@@ -12,8 +12,11 @@
 #include <string.h>
 
 #include <algorithm>
+#include <atomic>
 #include <functional>
+#include <new>
 #include <string>
+#include <thread>
 #include <type_traits>
 #include <vector>
 
@@ -618,6 +621,154 @@ inline bool sym_eigen(int m, std::vector<double>& a, std::vector<double>& d, std
   return true;
 }
 
+// fn(0) .. fn(n - 1) on up to eight threads; what threads cannot be had for runs here.
+template <class Fn>
+void host_parallel(int n, Fn fn) {
+  std::atomic<int> next{0};
+  auto work = [&]() {
+    for (int i = next.fetch_add(1); i < n; i = next.fetch_add(1)) fn(i);
+  };
+  std::vector<std::thread> ts;
+  try {
+    const int nt = std::min(n, (int)std::min(8u, std::thread::hardware_concurrency())) - 1;
+    ts.reserve(std::max(nt, 0));
+    for (int k = 0; k < nt; ++k) ts.emplace_back(work);
+  } catch (...) {
+  }
+  work();
+  for (std::thread& t : ts) t.join();
+}
+
+// The same for a matrix of half-bandwidth b, whose lower band a[j (b + 2) + i - j]
+// holds (i - j <= b; the last place is for the bulge): plane rotations reduce the band
+// to a tridiagonal matrix (Schwarz 1968), and the same iteration diagonalises that.
+// The rotations are only recorded, as runs on consecutive rows; rotate() then applies
+// them to the identity, eight columns at a time in cache and on several threads, which
+// is most of the work: 6 m operations for each of about 1.4 m^2 rotations.  512 nodes
+// in 5 ms where sym_eigen takes 29, 400 in 2.7 against 13.5 (Grace, 8 threads).
+struct BandEigen {
+  struct Run {
+    int row, n;
+    size_t at;
+  };
+  int m = 0;
+  std::vector<double> a, d;
+  std::vector<Run> runs;
+  std::vector<double> cs, sn;
+  bool ok = false;
+
+  void turn(int row, double c, double s, bool joins) {
+    if (!joins || runs.empty()) runs.push_back(Run{row, 0, cs.size()});
+    ++runs.back().n;
+    cs.push_back(c);
+    sn.push_back(s);
+  }
+
+  void tridiagonal(int b) {
+    const int w = b + 2;
+    auto L = [&](int i, int j) -> double& { return a[(size_t)j * w + (i - j)]; };
+    for (int k = 0; k + 2 < m; ++k)
+      for (int p = std::min(b, m - 1 - k); p >= 2; --p)
+        for (int col = k, i = k + p - 1; i + 1 < m; col = i, i += b) {  // rows i, i + 1 clear (i + 1, col)
+          const double x = L(i, col), y = L(i + 1, col);
+          if (y == 0.0) break;
+          const double r = sqrt(x * x + y * y), c = x / r, s = y / r;
+          L(i, col) = r;
+          L(i + 1, col) = 0.0;
+          for (int j = col + 1; j < i; ++j) {
+            const double u = L(i, j), v = L(i + 1, j);
+            L(i, j) = c * u + s * v;
+            L(i + 1, j) = c * v - s * u;
+          }
+          const double p0 = L(i, i), q = L(i + 1, i), p1 = L(i + 1, i + 1);
+          L(i, i) = c * c * p0 + 2.0 * c * s * q + s * s * p1;
+          L(i + 1, i + 1) = s * s * p0 - 2.0 * c * s * q + c * c * p1;
+          L(i + 1, i) = (c * c - s * s) * q + c * s * (p1 - p0);
+          for (int j = i + 2; j <= std::min(m - 1, i + 1 + b); ++j) {
+            const double u = j - i <= b ? L(j, i) : 0.0, v = L(j, i + 1);
+            L(j, i) = c * u + s * v;  // (j = i + 1 + b: the bulge, cleared next)
+            L(j, i + 1) = c * v - s * u;
+          }
+          turn(i, c, s, false);
+        }
+  }
+
+  // a as above; false when an eigenvalue does not settle
+  bool solve(int m_, int b, std::vector<double>& band) {
+    m = m_;
+    a.swap(band);
+    tridiagonal(b);
+    d.assign(m, 0.0);
+    std::vector<double> e(m, 0.0);
+    for (int i = 0; i < m; ++i) {
+      d[i] = a[(size_t)i * (b + 2)];
+      if (i + 1 < m) e[i] = a[(size_t)i * (b + 2) + 1];
+    }
+    int hi = m - 1, its = 0;
+    while (hi > 0) {
+      for (int k = 0; k < hi; ++k)
+        if (fabs(e[k]) <= 1.2e-16 * (fabs(d[k]) + fabs(d[k + 1]))) e[k] = 0.0;
+      if (e[hi - 1] == 0.0) {
+        --hi;
+        its = 0;
+        continue;
+      }
+      if (++its > 80) return false;
+      int lo = hi - 1;
+      while (lo > 0 && e[lo - 1] != 0.0) --lo;
+      const double g = 0.5 * (d[hi - 1] - d[hi]), q = e[hi - 1];
+      const double den = g + (g >= 0.0 ? 1.0 : -1.0) * hypot(g, q);
+      const double mu = d[hi] - q * q / den;
+      double x = d[lo] - mu, z = e[lo];
+      for (int k = lo; k < hi; ++k) {  // chase the bulge with plane rotations
+        const double r = sqrt(x * x + z * z);
+        const double c = r > 0.0 ? x / r : 1.0, s = r > 0.0 ? z / r : 0.0;
+        if (k > lo) e[k - 1] = r;
+        const double dk = d[k], dn = d[k + 1], ek = e[k];
+        d[k] = c * c * dk + 2.0 * c * s * ek + s * s * dn;
+        d[k + 1] = s * s * dk - 2.0 * c * s * ek + c * c * dn;
+        e[k] = (c * c - s * s) * ek + c * s * (dn - dk);
+        if (k + 1 < hi) {
+          x = e[k];
+          z = s * e[k + 1];
+          e[k + 1] *= c;
+        }
+        turn(k, c, s, k > lo);
+      }
+    }
+    return true;
+  }
+
+  // Columns [8 q, 8 q + 8) of v, whose row k becomes the eigenvector of d[k]; buf: 8 m doubles.
+  void rotate(int q, double* buf, double* v) const {
+    constexpr int W = 8;
+    for (int i = 0; i < m * W; ++i) buf[i] = 0.0;
+    for (int l = 0; l < W && q * W + l < m; ++l) buf[(size_t)(q * W + l) * W + l] = 1.0;
+    for (const Run& run : runs) {
+      double* p = buf + (size_t)run.row * W;
+      double cur[W];
+      for (int l = 0; l < W; ++l) cur[l] = p[l];
+      for (int t = 0; t < run.n; ++t, p += W) {
+        const double c = cs[run.at + t], s = sn[run.at + t];
+        for (int l = 0; l < W; ++l) {
+          const double nx = p[W + l];
+          p[l] = c * cur[l] + s * nx;
+          cur[l] = c * nx - s * cur[l];
+        }
+      }
+      for (int l = 0; l < W; ++l) p[l] = cur[l];
+    }
+    for (int i = 0; i < m; ++i)
+      for (int l = 0; l < W && q * W + l < m; ++l) v[(size_t)i * m + q * W + l] = buf[(size_t)i * W + l];
+  }
+};
+
+// Axes up to this long take the dense eigenproblem: 0.6 ms at 128 nodes, 1.7 at 192,
+// 3.8 at 256 in a context's first solve on such an axis.  Beyond, the banded one: with
+// the dense one first solves on long thin grids took longer than they had with V-cycles
+// (512 x 48 x 48 MIXED 31 ms against 7.0; 6.1 to 7.0 so).
+constexpr int kFdDense = 256;
+
 // The axis table of n nodes at stencil radius R, in host memory: `mat` holds
 // forwards high, low, backwards high, low (each the even half's ne x pe and the
 // odd half's no x po elements), `mu` the n eigenvalues at spacing 1 (even modes
@@ -636,26 +787,56 @@ inline bool fd_axis_host(int n, int R, FdAxis* ax, std::vector<float>* mat, std:
   const Weights<double> W = lap_weights(R, 1.0, -1.0);
   auto t = [&](int q) { return q == 0 ? W.c / 3.0 : q <= R ? W.w[q] : 0.0; };
   const double r2 = sqrt(0.5);
+  // element (i, j) of a half's matrix
+  auto element = [&](int odd, int i, int j) {
+    const int m = odd ? ax->no : ax->ne;
+    const bool mid = !odd && (n & 1);
+    const double x = t(abs(i - j)), y = t(n - 1 - i - j);
+    const int mids = (mid && i == m - 1) + (mid && j == m - 1);
+    if (mids == 1) return 2.0 * r2 * x;  // sqrt 2 t(|i - m|): both mirror images couple to the middle
+    return mids ? x : x + (odd ? -y : y);
+  };
+  std::vector<double> d[2], v[2];
+  if (n <= kFdDense) {
+    for (int odd = 0; odd < 2; ++odd) {
+      const int m = odd ? ax->no : ax->ne;
+      std::vector<double> a((size_t)m * m);
+      for (int i = 0; i < m; ++i)
+        for (int j = 0; j < m; ++j) a[(size_t)i * m + j] = element(odd, i, j);
+      if (!sym_eigen(m, a, d[odd], v[odd])) return false;
+    }
+  } else {
+    BandEigen eig[2];
+    std::vector<double> buf[2];
+    host_parallel(2, [&](int odd) {
+      const int m = odd ? ax->no : ax->ne, w = R + 2;
+      try {
+        std::vector<double> a((size_t)m * w, 0.0);
+        for (int j = 0; j < m; ++j)
+          for (int i = j; i < std::min(m, j + R + 1); ++i) a[(size_t)j * w + (i - j)] = element(odd, i, j);
+        v[odd].resize((size_t)m * m);
+        buf[odd].resize((size_t)(m + 7) / 8 * 8 * m);
+        eig[odd].ok = eig[odd].solve(m, R, a);
+      } catch (const std::bad_alloc&) {
+        eig[odd].ok = false;
+      }
+    });
+    if (!eig[0].ok || !eig[1].ok) return false;
+    const int q0 = (ax->ne + 7) / 8, q1 = (ax->no + 7) / 8;
+    host_parallel(q0 + q1, [&](int q) {
+      const int odd = q >= q0, k = odd ? q - q0 : q;
+      eig[odd].rotate(k, buf[odd].data() + (size_t)k * 8 * eig[odd].m, v[odd].data());
+    });
+    d[0].swap(eig[0].d);
+    d[1].swap(eig[1].d);
+  }
   for (int odd = 0; odd < 2; ++odd) {
     const int m = odd ? ax->no : ax->ne, wp = odd ? ax->po : ax->pe;
     const bool mid = !odd && (n & 1);
-    std::vector<double> a((size_t)m * m), d, v;
-    for (int i = 0; i < m; ++i)
-      for (int j = 0; j < m; ++j) {
-        double x = t(abs(i - j));
-        const double y = t(n - 1 - i - j);
-        const int mids = (mid && i == m - 1) + (mid && j == m - 1);
-        if (mids == 0)
-          x += odd ? -y : y;
-        else if (mids == 1)
-          x = 2.0 * r2 * x;  // sqrt 2 t(|i - m|): both mirror images couple to the middle
-        a[(size_t)i * m + j] = x;
-      }
-    if (!sym_eigen(m, a, d, v)) return false;
-    for (int k = 0; k < m; ++k) (*mu)[(odd ? ax->ne : 0) + k] = d[k];
+    for (int k = 0; k < m; ++k) (*mu)[(odd ? ax->ne : 0) + k] = d[odd][k];
     for (int k = 0; k < m; ++k)
       for (int i = 0; i < m; ++i) {
-        const double x = v[(size_t)k * m + i] * ((mid && i == m - 1) ? 1.0 : r2);
+        const double x = v[odd][(size_t)k * m + i] * ((mid && i == m - 1) ? 1.0 : r2);
         const float h = (float)x, l = (float)(x - (double)h);
         const size_t f = (odd ? se : 0) + (size_t)i * wp + k, b = (odd ? se : 0) + (size_t)k * wp + i;
         (*mat)[f] = h;
