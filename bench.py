@@ -94,7 +94,8 @@ def load_peaks():
 
 def src_hash():
     h = hashlib.sha256()
-    for rel in ("paper_1405_6456_gb300/csrc/kernels.cuh", "paper_1405_6456_gb300/csrc/common.cuh"):
+    for rel in ("kernels.cuh", "common.cuh", "fastdiag.cuh", "host.cuh"):
+        rel = os.path.join("paper_1405_6456_gb300", "csrc", rel)
         with open(os.path.join(ROOT, rel), "rb") as f:
             h.update(f.read())
     return h.hexdigest()[:16]
@@ -309,12 +310,14 @@ def _traffic(key):
     return None
 
 
-def roofline_entries(cnt, sampled, G, n, prec_name, es, fold, residuals):
+def roofline_entries(cnt, sampled, G, n, prec_name, es, fold, residuals, evaluations):
     """Rooflines of the hot kernels from CUDA-event durations of a profiled
     ground state: one entry per kernel with its algorithmic bytes (or flops) per
     launch over its mean launch duration, and its total time.  `residuals`: the
     residual passes that had work to do (mixed rounds are launched ahead, and those
-    behind a solve that is done return at once: their time counts, they do not)."""
+    behind a solve that is done return at once: their time counts, they do not);
+    `evaluations`: the functional passes that had (one launched behind a solve that
+    has not converged returns at once too)."""
     from paper_1405_6456_gb300 import ofdft as F
     peak_hbm, which = load_peaks()
     out = []
@@ -375,16 +378,17 @@ def roofline_entries(cnt, sampled, G, n, prec_name, es, fold, residuals):
     # fused functional + gradient pass (every launch timed)
     k = F.K_FUNCTIONAL
     if sampled.timed_launches[k] > 0:
-        avg = sampled.timed_ms[k] / sampled.timed_launches[k] / 1e3
+        ran = min(int(sampled.timed_launches[k]), evaluations)
+        avg = sampled.timed_ms[k] / ran / 1e3
         algo = G * 5 * es  # read u (stencil), phi, b, d; write G
         ach = algo / avg / 1e9
         out.append({"kernel": "zstream_kernel<%s,%d,LoadPlain,EpiFunctional> (fused TF + vW + XC + electrostatic "
                               "energy, gradient, preconditioner, 11 sums)" % ("float" if es == 4 else "double", n),
                     "bound": "hbm", "achieved": ach, "peak": peak_hbm, "unit": "GB/s", "frac": ach / peak_hbm,
-                    "peak_source": which, "launches_timed": int(sampled.timed_launches[k]), "avg_us": avg * 1e6,
-                    "total_ms": sampled.timed_ms[k], "algorithmic_bytes_per_launch": algo,
+                    "peak_source": which, "launches_timed": int(sampled.timed_launches[k]), "launches_with_work": ran,
+                    "avg_us": avg * 1e6, "total_ms": sampled.timed_ms[k], "algorithmic_bytes_per_launch": algo,
                     "traffic": _traffic(f"functional_{prec_name}"),
-                    "timing": "CUDA events around every functional launch"})
+                    "timing": "CUDA events around every functional launch, over the launches that had work to do"})
     return out
 
 
@@ -524,7 +528,8 @@ def run_gpu(args):
         ctx.profile(False)
         fold = 5 * G * es > 96 * (1 << 20)
         residuals = args.profile_steps * (st.grad_evals + st.cg_iters)
-        ents = roofline_entries(sampled, sampled, G, c.fd_order // 2, args.precision, es, fold, residuals)
+        evaluations = args.profile_steps * (st.grad_evals + st.energy_evals)
+        ents = roofline_entries(sampled, sampled, G, c.fd_order // 2, args.precision, es, fold, residuals, evaluations)
         ents.sort(key=lambda e: -e["total_ms"])
         if ents:
             out["roofline"] = ents[0]

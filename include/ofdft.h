@@ -189,10 +189,10 @@ int ofdft_destroy(ofdft_ctx* ctx);
  *     iteration up to rounding).
  *   OFDFT_PRECOND_MG (default): z = M r.  On grids whose axes all have 32 to 512
  *     nodes (256 in a batch) M inverts -L_h itself, up to rounding, by diagonalising the three
- *     axes' matrices (one CG step in FP64, one per residual correction in MIXED);
- *     (a context's first solve on an axis length and order computes that matrix's
+ *     axes' matrices (one CG step in FP64, one per residual correction in MIXED;
+ *     a context's first solve on an axis length and order computes that matrix's
  *     eigenvectors on the host, 0.1 ms at 64 nodes, 1.7 at 192, 3.8 at 256, 5 at 512,
- *     and keeps them, 8 n^2 to 9 n^2 bytes, until ofdft_destroy)
+ *     and keeps them, about 8 n^2 bytes, until ofdft_destroy);
  *     on the others M is one symmetric V(1,1)-cycle of the second-order 7-point
  *     Laplacian (damped Jacobi, full weighting, trilinear
  *     prolongation, coarse node I on fine node 2I+1, zero Dirichlet values);
@@ -261,7 +261,8 @@ int ofdft_poisson(ofdft_ctx* ctx, const ofdft_grid* g, int fd_order, int prec, c
  * diag + (4h^3/mu) u u^T applied to -G); optional device inputs d and s_old
  * give out->gd = h^3 G.d and out->gs_old = h^3 G.s_old.  mu = +inf drops the
  * penalty term.  u, b, phi, grad, s, d, s_old: device arrays of the `prec` type
- * (p->precision).  Synchronises; results in *out. */
+ * (p->precision).  When the Poisson solve fails (OFDFT_ENOTCONV, OFDFT_ENONFINITE)
+ * grad and s are left as they were.  Synchronises; results in *out. */
 int ofdft_energy_grad(ofdft_ctx* ctx, const ofdft_grid* g, const ofdft_params* p, const void* u,
                       const void* b, void* phi, double E_self, double eta, double mu, double N,
                       int solve_poisson, void* grad, void* s, const void* d, const void* s_old,

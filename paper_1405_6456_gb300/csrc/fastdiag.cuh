@@ -25,8 +25,9 @@
 // take 48 + 39 + 81 + 40 + 44 = 252 us (40% of the pipes' rate; a V-cycle takes
 // 158 us but 16 to 30 times as many of them are needed).  The same passes with the
 // matrix rows read through L1 took 475 us (42% of them missed); with the x panels
-// transposed on the way in 300 us.  At 128^3 in float-float: 74 + 66 + 137 + 65 +
-// 70 us, 58% of the rate of its 12 operations.
+// transposed on the way in 300 us.  The last pass of a correction takes 95 us instead
+// of 44 (303 us the five).  At 128^3 in float-float: 63 + 62 + 128 + 62 + 67 us, 59% of
+// the rate of its 12 operations.
 //
 // Element types: FP32 fields compute in FP32.  FP64 fields compute in float-float
 // pairs (ff, about 2^-46 relative): 12 packed FP32 operations per multiply-add

@@ -383,10 +383,10 @@ ZShape zshape(ofdft_ctx* c, const GridDev& g, int blocks_per_sm = 2, int force_n
     // slow each other down to 1 + a (k - 1) of that: FP64 passes share a pipe that
     // one block fills (a = 0.95, c0 = 0.7), FP32 and float-float ones mostly wait
     // (a = 0.45, c0 = 2.3).  Fitted to sweeps of 1 to 64 chunks on 48^3 to 192^3;
-    // the chosen split is within 4% of the best measured one, where the former rule
-    // (one wave, chunks of at least 2 R planes) lost 10 to 75% below 160^3
-    // (functional, us: FP64 48^3 245 -> 61, 80^3 283 -> 173; FP32 64^3 68 -> 33,
-    // 128^3 92 -> 71) and nothing above.
+    // the chosen split is within 4% of the best measured one; one wave in chunks of at
+    // least 2 R planes is 10 to 75% slower below 160^3 (functional, us, that | this:
+    // FP64 48^3 245 | 61, 80^3 283 | 173; FP32 64^3 68 | 33, 128^3 92 | 71) and the same
+    // above.
     const double a = sizeof(T) == 8 && std::is_same<T, double>::value ? 0.95 : 0.45;
     const double c0 = std::is_same<T, double>::value ? 0.7 : 2.3;
     double least = 1e300;
@@ -896,17 +896,18 @@ inline int fd_table(ofdft_ctx* c, int n, int R, const FdTable** out) {
 
 // Whether a grid takes the fast diagonalisation: every axis of kFdMinN to
 // kFdMaxN nodes.  Measured against the V-cycle on whole Poisson solves of a random
-// density, order 12 (us; FP64 to 1e-10, MIXED to 1e-8; V-cycle -> here):
-//   32^3       FP64   2,626 ->    242    MIXED   1,402 ->    398
-//   64^3              4,713 ->    257            2,105 ->    411
-//   512x48^2         12,602 ->    947            4,200 ->    671
-//   160^3            30,551 ->  1,786            7,787 ->  1,949
-//   512^2x64        143,156 -> 10,329           26,231 ->  8,768
-//   400^3           482,773 -> 91,501          103,551 -> 43,391
+// density, order 12 (us; FP64 to 1e-10, MIXED to 1e-8; V-cycle | here):
+//   32^3       FP64   2,444 |    115    MIXED   1,248 |    148
+//   64^3              4,167 |    178            1,782 |    180
+//   512x48^2         11,911 |    636            3,793 |    411
+//   160^3            28,141 |  1,787            5,053 |    680
+//   512^2x64        128,135 | 10,388           18,334 |  3,337
+//   400^3           424,080 | 48,156           59,099 | 13,738
 // and to 1e-4 (the loosest a solve asks for) 3 to 9 times faster, so nothing
 // inside the limits goes to the V-cycle.  The upper limit is what one block's
-// panel holds; the work grows with n1 + n2 + n3 per node.  Below kFdMinN the
-// V-cycle keeps the iteration counts that callers who cap them see (a cap of a
+// panel holds; the work grows with n1 + n2 + n3 per node.  The lower one is not where
+// the V-cycle becomes faster (30^3 takes it 1,900 us in FP64 and 1,040 in MIXED): below
+// it the V-cycle keeps the iteration counts that callers who cap them see (a cap of a
 // few steps ends a 24^3 solve with OFDFT_ENOTCONV).
 inline bool fd_usable(const ofdft_ctx* c, const GridDev& g, int nmax = kFdMaxN) {
   const int lo = std::min(g.n1, std::min(g.n2, g.n3)), hi = std::max(g.n1, std::max(g.n2, g.n3));
@@ -988,7 +989,7 @@ int fd_pass(ofdft_ctx* c, const FdJob& J) {
   // taken, the wider where within a tenth (us per application, 16 | 32: 48^3 56 | 68,
   // 80^3 123 | 145, 112^3 309 | 296, 192^3 1790 | 1684).  FP32 passes wait more than
   // they compute on small grids: 64 columns from 128 an SM on (32 | 64: 80^3 60 | 67,
-  // 112^3 92 | 104, 160^3 212 | 200, 192^3 329 | 307).
+  // 112^3 92 | 104, 160^3 212 | 200, 192^3 329 | 307, with the correction in the last pass).
   constexpr int HI = sizeof(T) == 4 ? 4 : 2, LO = HI / 2;
   auto most = [&](int ct) { return (J.ncols + 16LL * ct * c->sms - 1) / (16LL * ct * c->sms) * ct; };
   const bool wide = sizeof(T) == 4 ? J.ncols >= 128LL * c->sms : most(HI) * 10 <= most(LO) * 11;

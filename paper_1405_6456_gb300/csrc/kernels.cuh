@@ -1089,9 +1089,12 @@ struct EpiResidual {
 // the variational electrostatic energy of the functional that follows, of
 // (u^2 + b) phi and phi r.  Accuracy: about 2^-48 of the magnitudes of the
 // stencil's terms (the FP64 pass: 2^-53).
-// Bound by the FP32 pipes: 316 operations a node for the stencil at R = 6 and about
-// 80 here.  At 192^3 138 us, 0.49 of the pipes' rate (180 us with a chain per axis,
-// three compensated terms per electrostatic sum and u read when it was used).
+// Bound by instruction issue (81% of the active cycles): 316 operations a node for
+// the stencil at R = 6 and 91 here.  At 192^3 137 us, 0.52 of the FP32 pipes' rate
+// (180 us with a chain per axis, three compensated terms per electrostatic sum and u
+// read when it is used).  The electrostatic sums' low terms as plain FMAs leave their
+// error where three compensated terms have it (rms over 16 to 1024 terms, of sum
+// |terms|: 6.4e-15 to 3.3e-13 either way).
 __device__ __forceinline__ float2 ff_prod(float a, float b) {  // a b exactly
   const float p = a * b;
   return make_float2(p, fmaf(a, b, -p));
@@ -1169,9 +1172,8 @@ struct EpiResidualFF {
 // in64, extrapolated along a line search by t (in64 - in0) when in0 is given, or
 // from the FP32 field in32), the pairs phi2 the residual pass reads, and the FP32
 // field out32 (when given).  b2: the pseudocharge as pairs, from b64 or b32 (when
-// given).  One pass where there were a copy, an extrapolation, a split and, at the
-// end of the solve, a conversion (together 53 us at 128^3); bound by HBM (28 to 36
-// bytes a node).
+// given).  Bound by HBM (28 to 36 bytes a node); as passes of their own a copy, an
+// extrapolation, a split and a conversion take 53 us at 128^3.
 static __global__ void __launch_bounds__(256) ff_prepare_kernel(long long G, const double* in64, const double* in0,
                                                                 double t, const float* in32, double* phi64,
                                                                 float2* phi2, float* out32, float2* b2,
@@ -1252,8 +1254,11 @@ __global__ void __launch_bounds__(256) ff_prepare2_kernel(long long n, const dou
 // 1 / d, and z = x^{-1/3} with c2 = x^{2/3}, for the functional.  In FP64 they start
 // from the FP32 functions and take one step that triples the number of correct
 // digits (from e = 1 - d r: r += r (e + e^2); from e = 1 - x z^3, the binomial series
-// of (1 - e)^{-1/3}: z += z (e/3 + 2 e^2/9)): 3 and 6 FP64 operations, within a unit
-// in the last place.  Arguments whose seed FP32 could not hold take CUDA's functions.
+// of (1 - e)^{-1/3}: z += z (e/3 + 2 e^2/9)): 3 and 6 FP64 operations.  The gradient's
+// terms come out nearer their values than with CUDA's cube root and quotients (units of
+// 2^-53, rms over |u| from 1e-3 to 10 against 64-bit mantissas: Thomas-Fermi 1.44 | 2.02,
+// exchange-correlation 0.89 | 1.12; from 1e-40 to 1e40 1.61 | 2.03 and 1.01 | 1.17).
+// Arguments whose seed FP32 could not hold take CUDA's functions.
 // In FP32, where CUDA's functions cost little and z is slower to come by (132 against
 // 125 us at 192^3), z is not formed.
 __device__ __forceinline__ float func_rcp(float d) { return 1.0f / d; }
@@ -2551,9 +2556,9 @@ __global__ void __launch_bounds__(256) axpy_abs_kernel(long long G, T* out, cons
 // The Polak-Ribiere direction of the NLCG with everything that belongs to it in one
 // pass: s -= gamma w (the rank-one correction of the evaluation's preconditioned
 // residual; gamma == 0: none), d = s + beta d (d = s when beta == 0), and
-// out[0] = G.d, out[1] = d.d for the line search.  Three passes before, and the
-// correction was applied to trial points whose residual nobody used (48 us an
-// iteration at 128^3 in FP32); bound by HBM.
+// out[0] = G.d, out[1] = d.d for the line search.  Bound by HBM; the correction waits
+// for the point that is kept (trial points' residuals are not used).  As three passes,
+// with the correction at every trial point, 48 us an iteration more at 128^3 in FP32.
 template <typename T>
 __global__ void __launch_bounds__(256) nlcg_direction_kernel(long long G, T* __restrict__ d, T* __restrict__ s,
                                                              const T* __restrict__ w, const T* __restrict__ gr,
